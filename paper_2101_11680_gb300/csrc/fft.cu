@@ -603,13 +603,14 @@ __global__ void __launch_bounds__(ROW_WARPS * 32) k_rows_inv(const __grid_consta
 // place (tensor map `map`).  The m and u1 values of a lane are loaded before
 // its tile is waited for; the next job's tile is requested once the copy out
 // of its buffer has read it.
-template <int P, bool RESID>
+// WIDE: more than P / 2 scan columns (a circular scan fills the grid).
+template <int P, bool RESID, bool WIDE>
 __global__ void __launch_bounds__(ROW_WARPS * 32, P >= 512 ? 2 : 3)
     k_rows_admm_t(const __grid_constant__ CUtensorMap map, int nplanes, int n, const float* __restrict__ m,
                   float* __restrict__ u1, float scale, float inv_s, float rho, const float2* __restrict__ tw,
                   int* __restrict__ flag, long long max_polls) {
   constexpr int R = P / 32;
-  constexpr int RN = R / 2 > 0 ? R / 2 : 1;  // registers that can hold scan columns (n <= P / 2)
+  constexpr int RN = WIDE || R < 2 ? R : R / 2;  // registers that can hold scan columns
   extern __shared__ float4 row_smem4[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const RowSmem S = row_carve<P>(row_smem4, warp);
@@ -991,9 +992,10 @@ ctof_status fft_rows_admm_t(const ctof_kernel_s* k, float2* inter, const float* 
   const size_t sm = row_smem_bytes(k->p);
   const float scale = 1.0f / ((float)k->p * (float)k->p);
   CTOF_P_SWITCH(k->p, {
-    CTOF_CUDA_TRY(allow_smem(k_rows_admm_t<P_, false>, sm));
-    k_rows_admm_t<P_, false><<<row_grid(k->n, k->nt), ROW_WARPS * 32, sm, st>>>(
-        map, k->nt, k->n, m, u1, scale, inv_scale, rho, k->d_tw, k->d_flags, k->max_polls);
+    auto kern = k->n > P_ / 2 ? k_rows_admm_t<P_, false, true> : k_rows_admm_t<P_, false, false>;
+    CTOF_CUDA_TRY(allow_smem(kern, sm));
+    kern<<<row_grid(k->n, k->nt), ROW_WARPS * 32, sm, st>>>(map, k->nt, k->n, m, u1, scale, inv_scale, rho, k->d_tw,
+                                                            k->d_flags, k->max_polls);
   });
   CTOF_CUDA_TRY(cudaGetLastError());
   return CTOF_OK;
@@ -1005,9 +1007,10 @@ ctof_status fft_rows_resid_t(const ctof_kernel_s* k, float2* inter, const float*
   const size_t sm = row_smem_bytes(k->p);
   const float scale = 1.0f / ((float)k->p * (float)k->p);
   CTOF_P_SWITCH(k->p, {
-    CTOF_CUDA_TRY(allow_smem(k_rows_admm_t<P_, true>, sm));
-    k_rows_admm_t<P_, true><<<row_grid(k->n, k->nt), ROW_WARPS * 32, sm, st>>>(
-        map, k->nt, k->n, m, nullptr, scale, 0.f, 0.f, k->d_tw, k->d_flags, k->max_polls);
+    auto kern = k->n > P_ / 2 ? k_rows_admm_t<P_, true, true> : k_rows_admm_t<P_, true, false>;
+    CTOF_CUDA_TRY(allow_smem(kern, sm));
+    kern<<<row_grid(k->n, k->nt), ROW_WARPS * 32, sm, st>>>(map, k->nt, k->n, m, nullptr, scale, 0.f, 0.f, k->d_tw,
+                                                            k->d_flags, k->max_polls);
   });
   CTOF_CUDA_TRY(cudaGetLastError());
   return CTOF_OK;
