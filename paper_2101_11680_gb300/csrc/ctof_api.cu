@@ -129,6 +129,29 @@ ctof_status adjoint_impl(ctof_kernel_s* k, const float* m, float* vol, cudaStrea
   return fft_inverse_planes(k, k->d_spec_z, k->ldz, k->nz, k->n, k->n, k->d_inter_z, vol, k->n, st);
 }
 
+// Measurement m [nt][n][n] (device memory) into `out` as the planes that
+// operator o works on: Q^T m for a time-compressed one, a copy otherwise.
+ctof_status stage_measurement(const ctof_kernel_s* o, const float* m, float* out, cudaStream_t st) {
+  if (o->tz_nt) return time_compress(o, 1, m, out, st);
+  CTOF_CUDA_TRY(cudaMemcpyAsync(out, m, (size_t)o->nt * o->n * o->n * sizeof(float), cudaMemcpyDeviceToDevice, st));
+  return CTOF_OK;
+}
+
+// The operator that a solver runs on.
+ctof_kernel_s* solver_ops(ctof_kernel_s* k, const ctof_solver_params* prm) {
+  return prm->solver == CTOF_SOLVER_TIKHONOV ? ctof_ops_once(k) : ctof_ops(k);
+}
+
+// m = A mu in all nt bins, with `mux` y = S A mu (S acts on all bins alike, so
+// before the expansion).
+ctof_status forward_bins(ctof_kernel_s* k, const float* mu, float* m, bool mux, cudaStream_t st) {
+  ctof_kernel_s* o = ctof_ops_once(k);
+  float* planes = o->tz_nt ? o->d_u1 : m;
+  CTOF_TRY(forward_impl(o, mu, planes, st));
+  if (mux) CTOF_TRY(block_hadamard(planes, o->nt, o->n, st));
+  return o->tz_nt ? time_expand(o, planes, m, st) : CTOF_OK;
+}
+
 // ADMM set-up on the staged measurement d_mstage: the TV weight and the state reset.
 ctof_status admm_setup(ctof_kernel_s* k, const ctof_solver_params* prm, cudaStream_t st) {
   const int nt = k->nt, nz = k->nz, n = k->n, P = k->p;
@@ -518,7 +541,9 @@ ctof_status batch_graph_run(int count, const ctof_kernel* ks, const float* const
       g_side_events.push_back(e);
     }
     // problems whose x-update runs in the one persistent queue launch per iteration
-    CTOF_TRY(admm_queue_build(count, const_cast<ctof_kernel_s* const*>(ks), &g_batch.queue));
+    std::vector<ctof_kernel_s*> os(count);  // the operators ADMM runs on
+    for (int i = 0; i < count; ++i) os[i] = ctof_ops(ks[i]);
+    CTOF_TRY(admm_queue_build(count, os.data(), &g_batch.queue));
     std::vector<char> queued(count, 0);
     for (int i : g_batch.queue.members) queued[i] = 1;
     cudaStream_t cap = nullptr;
@@ -557,11 +582,9 @@ ctof_status batch_graph_run(int count, const ctof_kernel* ks, const float* const
     }
     fork();
     for (int i = 0; i < count && s == CTOF_OK; ++i) {
-      ctof_kernel_s* k = ks[i];
       cudaStream_t side = g_side_streams[stream_of[i]];
-      const size_t mb = (size_t)k->nt * k->n * k->n * sizeof(float);
-      if (cudaMemcpyAsync(k->d_mstage, d_m[i], mb, cudaMemcpyDeviceToDevice, side) != cudaSuccess) s = CTOF_ECUDA;
-      if (s == CTOF_OK) s = admm_setup(k, prm, side);
+      s = stage_measurement(os[i], d_m[i], os[i]->d_mstage, side);
+      if (s == CTOF_OK) s = admm_setup(os[i], prm, side);
     }
     join();
     // iterations in lockstep: the problems with their own x-update run it and their
@@ -573,8 +596,8 @@ ctof_status batch_graph_run(int count, const ctof_kernel* ks, const float* const
       for (int i = 0; i < count && s == CTOF_OK; ++i) {
         if (queued[i]) continue;
         cudaStream_t side = g_side_streams[stream_of[i]];
-        s = admm_contract(ks[i], side);
-        if (s == CTOF_OK) s = admm_side(ks[i], prm, it, side, nullptr);
+        s = admm_contract(os[i], side);
+        if (s == CTOF_OK) s = admm_side(os[i], prm, it, side, nullptr);
       }
       if (s == CTOF_OK) s = admm_queue_launch(g_batch.queue, cap);
       if (s == CTOF_OK && cudaEventRecord(ev_q, cap) != cudaSuccess) s = CTOF_ECUDA;
@@ -582,7 +605,7 @@ ctof_status batch_graph_run(int count, const ctof_kernel* ks, const float* const
         if (!queued[i]) continue;
         cudaStream_t side = g_side_streams[stream_of[i]];
         if (cudaStreamWaitEvent(side, ev_q, 0) != cudaSuccess) s = CTOF_ECUDA;
-        if (s == CTOF_OK) s = admm_side(ks[i], prm, it, side, nullptr);
+        if (s == CTOF_OK) s = admm_side(os[i], prm, it, side, nullptr);
       }
       join();
     }
@@ -654,18 +677,44 @@ void ctof_kernel_destroy(ctof_kernel k) {
   if (!k) return;
   DeviceGuard guard(k->device);
   batch_graph_forget(k);
-  if (k->graph) cudaGraphExecDestroy(k->graph);
-  destroy_events(k);
-  if (k->d_bt_cinv) cudaFree(k->d_bt_cinv);
-  if (k->d_batch) cudaFree(k->d_batch);
-  for (int i = 0; i < 2; ++i)
-    if (k->d_tik_hinv[i]) cudaFree(k->d_tik_hinv[i]);
+  for (ctof_kernel_s* o : {k->tz, k}) {  // what either operator made on first use
+    if (!o) continue;
+    if (o->graph) cudaGraphExecDestroy(o->graph);
+    destroy_events(o);
+    if (o->d_bt_cinv) cudaFree(o->d_bt_cinv);
+    if (o->d_batch) cudaFree(o->d_batch);
+    for (int i = 0; i < 2; ++i)
+      if (o->d_tik_hinv[i]) cudaFree(o->d_tik_hinv[i]);
+  }
+  time_basis_free(k);
+  if (k->d_admm) cudaFree(k->d_admm);
   if (k->d_w) cudaFree(k->d_w);
   if (k->d_base) cudaFree(k->d_base);
   delete k;
 }
 
 namespace {
+
+// The x-update's copies of the tables, for the operator that ADMM runs on.
+ctof_status admm_copies(ctof_kernel_s* k, cudaStream_t st) {
+  if (!k->tz) {
+    const size_t wa = contract_admm_pipe_floats(k->nt, k->nz, 0), ha = contract_admm_pipe_floats(k->nt, k->nz, 1);
+    if (wa) {
+      const size_t wb = ((size_t)k->nclass * wa * sizeof(float) + 255) & ~(size_t)255;
+      k->admm_bytes = wb + (size_t)k->nclass * ha * sizeof(float);
+      if (cudaMalloc(&k->d_admm, k->admm_bytes) != cudaSuccess) {
+        cudaGetLastError();
+        k->d_admm = nullptr;
+        return CTOF_ENOMEM;
+      }
+      k->d_what_admm = static_cast<float*>(k->d_admm);
+      k->d_hinv_admm = reinterpret_cast<float*>(static_cast<char*>(k->d_admm) + wb);
+    }
+  }
+  CTOF_TRY(contract_admm_prepare(ctof_ops(k), st));
+  CTOF_CUDA_TRY(cudaStreamSynchronize(st));
+  return CTOF_OK;
+}
 
 ctof_status build_any(const ctof_optics* optics, const ctof_emission* emission, const ctof_voxel_average* average,
                       const ctof_grid* grid, int flags, void* stream, ctof_kernel* out) {
@@ -728,9 +777,6 @@ ctof_status build_any(const ctof_optics* optics, const ctof_emission* emission, 
   const size_t o_what = cv.take<float>((size_t)k->nclass * nt * k->z4);
   const size_t o_gram = cv.take<double>((size_t)k->nclass * nz * nz);
   const size_t o_hinv = cv.take<float>((size_t)k->nclass * nz * k->z4);
-  const size_t wa_per = contract_admm_pipe_floats(nt, nz, 0), ha_per = contract_admm_pipe_floats(nt, nz, 1);
-  const size_t o_wa = wa_per ? cv.take<float>((size_t)k->nclass * wa_per) : 0;
-  const size_t o_ha = wa_per ? cv.take<float>((size_t)k->nclass * ha_per) : 0;
   const size_t o_tw = cv.take<float2>(fft_twiddle_count(P));
   const size_t o_st = cv.take<float2>((size_t)k->nf * k->ldt);
   const size_t o_st2 = cv.take<float2>((size_t)k->nf * k->ldt);
@@ -760,8 +806,6 @@ ctof_status build_any(const ctof_optics* optics, const ctof_emission* emission, 
   k->d_what = reinterpret_cast<float*>(b + o_what);
   k->d_gram = reinterpret_cast<double*>(b + o_gram);
   k->d_hinv = reinterpret_cast<float*>(b + o_hinv);
-  k->d_what_admm = wa_per ? reinterpret_cast<float*>(b + o_wa) : nullptr;
-  k->d_hinv_admm = wa_per ? reinterpret_cast<float*>(b + o_ha) : nullptr;
   k->d_tw = reinterpret_cast<float2*>(b + o_tw);
   k->d_spec_t = reinterpret_cast<float2*>(b + o_st);
   k->d_spec_t2 = reinterpret_cast<float2*>(b + o_st2);
@@ -805,6 +849,7 @@ ctof_status build_any(const ctof_optics* optics, const ctof_emission* emission, 
       break;
     }
     s = build_kernel_tables(k, st);
+    if (s == CTOF_OK) s = admm_copies(k, st);
   } while (0);
   if (s != CTOF_OK) {
     cudaStreamSynchronize(st);
@@ -846,10 +891,13 @@ ctof_status ctof_kernel_get_info(ctof_kernel k, ctof_kernel_info* info) {
   info->nz = k->nz;
   info->scale = k->scale;
   info->gram_max_diag = k->gram_max;
-  info->admm_stages = k->d_what_admm ? contract_admm_pipe_stages(k->nt, k->nz) : 0;
+  const ctof_kernel_s* o = ctof_ops(k);
+  info->admm_stages = o->d_what_admm ? contract_admm_pipe_stages(o->nt, o->nz) : 0;
   const size_t tik_bytes = (size_t)k->nclass * k->nz * k->z4 * sizeof(float);
-  info->device_bytes = k->bytes + (k->d_w ? (size_t)k->nt * k->nz * k->q * k->q * sizeof(double) : 0) +
+  info->device_bytes = k->bytes + k->admm_bytes + (k->tz ? k->tz->tz_bytes : 0) +
+                       (k->d_w ? (size_t)k->nt * k->nz * k->q * k->q * sizeof(double) : 0) +
                        ((k->d_tik_hinv[0] ? 1 : 0) + (k->d_tik_hinv[1] ? 1 : 0)) * tik_bytes;
+  if (k->tz) info->device_bytes += ((o->d_tik_hinv[0] ? 1 : 0) + (o->d_tik_hinv[1] ? 1 : 0)) * tik_bytes;
   return CTOF_OK;
 }
 
@@ -880,14 +928,18 @@ ctof_status ctof_forward(ctof_kernel k, const float* d_mu, float* d_m, void* str
   if (!k || !d_mu || !d_m) return CTOF_EINVAL;
   DeviceGuard g(k->device);
   if (!g.ok) return CTOF_ECUDA;
-  return forward_impl(k, d_mu, d_m, static_cast<cudaStream_t>(stream));
+  return forward_bins(k, d_mu, d_m, false, static_cast<cudaStream_t>(stream));
 }
 
 ctof_status ctof_adjoint(ctof_kernel k, const float* d_m, float* d_vol, void* stream) {
   if (!k || !d_m || !d_vol) return CTOF_EINVAL;
   DeviceGuard g(k->device);
   if (!g.ok) return CTOF_ECUDA;
-  return adjoint_impl(k, d_m, d_vol, static_cast<cudaStream_t>(stream));
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  ctof_kernel_s* o = ctof_ops_once(k);
+  if (!o->tz_nt) return adjoint_impl(k, d_m, d_vol, st);
+  CTOF_TRY(time_compress(o, 1, d_m, o->d_u1, st));
+  return adjoint_impl(o, o->d_u1, d_vol, st);
 }
 
 ctof_status ctof_contract_forward_batch(ctof_kernel k, int nvol, const float* d_in, float* d_out, void* stream) {
@@ -911,9 +963,7 @@ ctof_status ctof_forward_multiplexed(ctof_kernel k, const float* d_mu, float* d_
   if (k->n % 8 != 0) return CTOF_EUNSUPPORTED;
   DeviceGuard g(k->device);
   if (!g.ok) return CTOF_ECUDA;
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
-  CTOF_TRY(forward_impl(k, d_mu, d_y, st));
-  return block_hadamard(d_y, k->nt, k->n, st);
+  return forward_bins(k, d_mu, d_y, true, static_cast<cudaStream_t>(stream));
 }
 
 ctof_status ctof_adjoint_multiplexed(ctof_kernel k, const float* d_y, float* d_vol, void* stream) {
@@ -922,10 +972,10 @@ ctof_status ctof_adjoint_multiplexed(ctof_kernel k, const float* d_y, float* d_v
   DeviceGuard g(k->device);
   if (!g.ok) return CTOF_ECUDA;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const size_t meas = (size_t)k->nt * k->n * k->n;
-  CTOF_CUDA_TRY(cudaMemcpyAsync(k->d_u1, d_y, meas * sizeof(float), cudaMemcpyDeviceToDevice, st));
-  CTOF_TRY(block_hadamard(k->d_u1, k->nt, k->n, st));
-  return adjoint_impl(k, k->d_u1, d_vol, st);
+  ctof_kernel_s* o = ctof_ops_once(k);
+  CTOF_TRY(stage_measurement(o, d_y, o->d_u1, st));
+  CTOF_TRY(block_hadamard(o->d_u1, o->nt, o->n, st));
+  return adjoint_impl(o, o->d_u1, d_vol, st);
 }
 
 ctof_status ctof_reconstruct(ctof_kernel k, const float* d_m, const ctof_solver_params* params, float* d_mu,
@@ -935,11 +985,11 @@ ctof_status ctof_reconstruct(ctof_kernel k, const float* d_m, const ctof_solver_
   DeviceGuard g(k->device);
   if (!g.ok) return CTOF_ECUDA;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const size_t mbytes = (size_t)k->nt * k->n * k->n * sizeof(float);
   const size_t vbytes = (size_t)k->nz * k->n * k->n * sizeof(float);
   double lambda = 0.0;
-  CTOF_CUDA_TRY(cudaMemcpyAsync(k->d_mstage, d_m, mbytes, cudaMemcpyDeviceToDevice, st));
-  CTOF_TRY(solve_staged(k, params, &lambda, st));
+  ctof_kernel_s* o = solver_ops(k, params);
+  CTOF_TRY(stage_measurement(o, d_m, o->d_mstage, st));
+  CTOF_TRY(solve_staged(o, params, &lambda, st));
   CTOF_CUDA_TRY(cudaMemcpyAsync(d_mu, k->d_vstage, vbytes, cudaMemcpyDeviceToDevice, st));
   if (report) return fill_report(k, params, lambda, report, st);
   return CTOF_OK;
@@ -956,7 +1006,9 @@ ctof_status ctof_reconstruct_host(ctof_kernel k, const float* h_m, const ctof_so
   const size_t vbytes = (size_t)k->nz * k->n * k->n * sizeof(float);
   double lambda = 0.0;
   CTOF_CUDA_TRY(cudaMemcpyAsync(k->d_mstage, h_m, mbytes, cudaMemcpyHostToDevice, st));
-  CTOF_TRY(solve_staged(k, params, &lambda, st));
+  ctof_kernel_s* o = solver_ops(k, params);
+  if (o->tz_nt) CTOF_TRY(time_compress(o, 1, k->d_mstage, o->d_mstage, st));
+  CTOF_TRY(solve_staged(o, params, &lambda, st));
   CTOF_CUDA_TRY(cudaMemcpyAsync(h_mu, k->d_vstage, vbytes, cudaMemcpyDeviceToHost, st));
   if (report) return fill_report(k, params, lambda, report, st);
   return take_device_status(k, st);
@@ -980,18 +1032,22 @@ ctof_status ctof_reconstruct_batch_tikhonov(ctof_kernel k, int batch, const floa
     ctof_solver_params prm{};
     prm.solver = CTOF_SOLVER_TIKHONOV;
     prm.tik_lambda_rel = lambda_rel;
+    ctof_kernel_s* o = ctof_ops_once(k);
     for (int b = 0; b < batch; ++b) {
       double lam = 0.0;
-      CTOF_CUDA_TRY(cudaMemcpyAsync(k->d_mstage, d_m + b * mvol, mvol * sizeof(float), cudaMemcpyDeviceToDevice, st));
-      CTOF_TRY(tikhonov_run(k, &prm, st, &lam));
+      CTOF_TRY(stage_measurement(o, d_m + b * mvol, o->d_mstage, st));
+      CTOF_TRY(tikhonov_run(o, &prm, st, &lam));
       CTOF_CUDA_TRY(cudaMemcpyAsync(d_mu + b * xvol, k->d_vstage, xvol * sizeof(float), cudaMemcpyDeviceToDevice, st));
     }
     return CTOF_OK;
   }
+  const bool tz = k->tz != nullptr;
+  k = ctof_ops(k);
   const int ldm = ctof_round_up(batch * k->nt, 8), ldx = ctof_round_up(batch * k->nz, 8);
   const size_t b_sm = (size_t)k->nf * ldm * sizeof(float2), b_sx = (size_t)k->nf * ldx * sizeof(float2);
   const size_t b_in = (size_t)batch * (k->nt > k->nz ? k->nt : k->nz) * k->n * k->hp * sizeof(float2);
-  const size_t need = ((b_sm + 255) & ~(size_t)255) + ((b_sx + 255) & ~(size_t)255) + b_in;
+  const size_t b_fft = ((b_sm + 255) & ~(size_t)255) + ((b_sx + 255) & ~(size_t)255) + ((b_in + 255) & ~(size_t)255);
+  const size_t need = b_fft + (tz ? (size_t)batch * k->nt * k->n * k->n * sizeof(float) : 0);
   if (need > k->batch_bytes) {
     CTOF_CUDA_TRY(cudaStreamSynchronize(st));
     if (k->d_batch) cudaFree(k->d_batch);
@@ -1008,6 +1064,11 @@ ctof_status ctof_reconstruct_batch_tikhonov(ctof_kernel k, int batch, const floa
   float2* spec_m = reinterpret_cast<float2*>(base);
   float2* spec_x = reinterpret_cast<float2*>(base + ((b_sm + 255) & ~(size_t)255));
   float2* inter = reinterpret_cast<float2*>(base + ((b_sm + 255) & ~(size_t)255) + ((b_sx + 255) & ~(size_t)255));
+  if (tz) {
+    float* planes = reinterpret_cast<float*>(base + b_fft);
+    CTOF_TRY(time_compress(k, batch, d_m, planes, st));
+    d_m = planes;
+  }
   CTOF_TRY(fft_forward_planes(k, d_m, batch * k->nt, k->n, k->n, k->n, inter, spec_m, ldm, st));
   CTOF_TRY(batch_tikhonov_prepare(k, lambda, st));
   CTOF_TRY(batch_tikhonov_contract(k, precision, batch, spec_m, ldm, spec_x, ldx, refine_steps, st));
@@ -1018,12 +1079,14 @@ ctof_status ctof_kernel_autotune(ctof_kernel k, void* stream) {
   if (!k) return CTOF_EINVAL;
   DeviceGuard g(k->device);
   if (!g.ok) return CTOF_ECUDA;
+  k = ctof_ops(k);
   k->tuned = 0;
   return autotune(k, static_cast<cudaStream_t>(stream));
 }
 
 ctof_status ctof_kernel_get_tuning(ctof_kernel k, int* h_pb4) {
   if (!k || !h_pb4) return CTOF_EINVAL;
+  k = ctof_ops(k);
   for (int i = 0; i < 4; ++i) h_pb4[i] = k->tune_pb[i];
   return k->tuned ? CTOF_OK : CTOF_EUNSUPPORTED;
 }
@@ -1041,13 +1104,14 @@ ctof_status ctof_reconstruct_batch(int count, const ctof_kernel* ks, const float
   DeviceGuard g(ks[0]->device);
   if (!g.ok) return CTOF_ECUDA;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  for (int i = 0; i < count; ++i) CTOF_TRY(autotune(ks[i], st));
+  for (int i = 0; i < count; ++i) CTOF_TRY(autotune(ctof_ops(ks[i]), st));
   return batch_graph_run(count, ks, d_m, params, d_mu, st);
 }
 
 ctof_status ctof_set_wait_limit(ctof_kernel k, long long polls) {
   if (!k || polls < 0) return CTOF_EINVAL;
   k->max_polls = polls;
+  if (k->tz) k->tz->max_polls = polls;
   return CTOF_OK;
 }
 
@@ -1060,13 +1124,14 @@ ctof_status ctof_sync_status(ctof_kernel k, void* stream) {
 
 ctof_status ctof_set_timing(ctof_kernel k, int enable) {
   if (!k || (enable != 0 && enable != 1)) return CTOF_EINVAL;
-  k->timing = enable;
+  ctof_ops(k)->timing = enable;
   return CTOF_OK;
 }
 
 ctof_status ctof_get_timing(ctof_kernel k, ctof_timing* out) {
   if (!k || !out) return CTOF_EINVAL;
   memset(out, 0, sizeof(*out));
+  k = ctof_ops(k);
   out->graph_kernel_nodes = k->graph_kernel_nodes;
   if (!k->graph || !k->graph_timing) return CTOF_EUNSUPPORTED;
   DeviceGuard g(k->device);

@@ -46,6 +46,8 @@ struct ctof_kernel_s {
   float* d_what;       // [nclass][nt][z4] (zero padding)
   double* d_gram;      // [nclass][nz][nz]
   float* d_hinv;       // [nclass][nz][z4]  (ADMM normal matrix inverse, normalised units)
+  void* d_admm;        // the two copies below (own allocation; null when `tz` holds them)
+  size_t admm_bytes;
   float* d_what_admm;  // W_hat in the ADMM kernel's block layout [nclass][tm/8][zm/8][64] (or null)
   float* d_hinv_admm;  // H^-1 in the same layout [nclass][zm/8][zm/8][64] (or null)
   float2* d_tw;        // FFT twiddle table (fft_twiddle_table layout)
@@ -101,7 +103,33 @@ struct ctof_kernel_s {
   int tune_pb[4];
   int tuned;
   unsigned long long uid;  // unique per handle (batch graph cache key)
+
+  // Time compression (time_basis.cu): `tz` is this handle's operator on r < nt
+  // planes (V = Q^T W_hat in place of W_hat; null where it does not pay).  It
+  // borrows this handle's buffers and tables and owns the rest (d_tz_base, its
+  // graph, Tikhonov and precision-form tables); the fields below are its own.
+  ctof_kernel_s* tz;
+  void* d_tz_base;
+  size_t tz_bytes;
+  int tz_nt;               // bins of the measurement domain
+  float* d_tz_q;           // [tz_nt][16] rows of the windows' bases
+  int4* d_tz_win;          // windows: bins [x, y), first plane z, planes w
+  int4* d_tz_tiles;        // the windows cut into tiles of up to 32 bins
+  int tz_nwin, tz_ntiles;
 };
+
+// The operator that the iterative solvers and the batched Tikhonov of handle k
+// run on (one projection of the measurement serves the whole solve).
+inline ctof_kernel_s* ctof_ops(ctof_kernel_s* k) { return k->tz ? k->tz : k; }
+inline const ctof_kernel_s* ctof_ops(const ctof_kernel_s* k) { return k->tz ? k->tz : k; }
+
+// The operator that a single application (forward, adjoint, one Tikhonov
+// solve) runs on: the projection is a launch of its own, so the T-side
+// spectrum that it saves has to be large.
+constexpr size_t TZ_ONE_SHOT_BYTES = (size_t)8 << 20;
+inline ctof_kernel_s* ctof_ops_once(ctof_kernel_s* k) {
+  return k->tz && (size_t)k->nf * (k->nt - k->tz->nt) * sizeof(float2) >= TZ_ONE_SHOT_BYTES ? k->tz : k;
+}
 
 // Makes `dev` current for a scope and restores the previous device after it.
 struct DeviceGuard {
@@ -248,6 +276,17 @@ ctof_status build_kernel_tables(ctof_kernel_s* k, cudaStream_t st);
 ctof_status build_tikhonov_factors(ctof_kernel_s* k, int slot, double lambda, cudaStream_t st);
 // (G + lambda I)^-1 for an absolute lambda, made on first use (two cached lambdas).
 ctof_status tikhonov_inverse(ctof_kernel_s* k, double lambda, const float** hinv, cudaStream_t st);
+
+// ---- time_basis.cu ------------------------------------------------------
+// Fit the time basis on W_hat (FP64 [nclass][nt][nz]) and make k->tz where it
+// pays and holds.  Synchronous.
+ctof_status time_basis_build(ctof_kernel_s* k, const double* what64, cudaStream_t st);
+// Frees what k->tz owns from time_basis_build and clears it.
+void time_basis_free(ctof_kernel_s* k);
+// Q^T m for `batch` measurements [nt][n][n] -> [z->nt][n][n] (z = some k->tz).
+ctof_status time_compress(const ctof_kernel_s* z, int batch, const float* m, float* out, cudaStream_t st);
+// Q y: [z->nt][n][n] -> [nt][n][n].
+ctof_status time_expand(const ctof_kernel_s* z, const float* y, float* m, cudaStream_t st);
 
 // ---- admm.cu ------------------------------------------------------------
 ctof_status admm_tv_stencil(const ctof_kernel_s* k, const float* x, const float* u2_old,

@@ -1,0 +1,504 @@
+// Time-compressed operator.  Every lateral operation of the convolutional
+// model (Eq. 11: FFTs, crop, Hadamard multiplexing, the ADMM and FISTA
+// updates of the measurement side) acts on all time bins alike, and only
+// W_hat mixes them.  The diffusion responses are smooth in time, so W_hat's
+// rows span far fewer directions than there are bins: with an orthonormal
+// basis Q [nt][r] of that row space
+//     W_hat(f) = Q V(f),   V(f) = Q^T W_hat(f)   [r][nz],
+// and K^T c = V^T (Q^T c), K x = Q (V x).  The measurement side of every
+// solver then works on Q^T m (r planes in place of nt), and only ctof_forward
+// expands back to nt bins.
+//
+// Q is block-diagonal over windows of consecutive bins (each window ends when
+// its bin number has doubled or the response has fallen by 1000 within it),
+// each with at most 16 columns.  The windows keep the factorisation faithful
+// bin by bin, not only in norm: inside one window the response's dynamic
+// range is small, so FP32 rounding of V and Q stays relative to the bins'
+// own magnitude, and late bins (12 decades below the first) or deep layers
+// lose nothing.  The rank of a window is where the residual, each bin scaled
+// by its DC response and each depth by its share of it, falls below 1e-10:
+// FP32 rounding (6e-8) is three orders above.  Ranks at 0.5 mm / 25 ps: 59 of
+// 256 bins (48 depths), 78 of 512 (64 depths); 39 of 64 at 1 mm / 50 ps.
+// The factorisation is checked on the device over every frequency class and
+// is dropped (the handle then works on the nt bins) if it does not hold.
+#include <cuda_runtime.h>
+#include <math.h>
+#include <string.h>
+
+#include <algorithm>
+#include <new>
+#include <vector>
+
+#include "ctof_internal.h"
+
+namespace {
+
+constexpr int TZ_R = 16;             // columns of one window's basis at most (row pitch of the device table)
+constexpr int TZ_FIRST = 16;         // bins of the first window
+constexpr double TZ_FALL = 1e-3;     // a window ends where the response has fallen by this factor
+constexpr double TZ_EPS = 1e-10;     // scaled residual at which a window's rank is reached
+constexpr double TZ_FLOOR = 1e-6;    // depths below this share of a bin's response are scaled by it instead
+constexpr double TZ_CHECK = 2e-8;    // largest |W_hat - Q V| per bin relative to its DC response
+constexpr int TZ_SAMPLES = 96;       // frequency classes whose rows the basis is fitted on
+constexpr int TZ_TILE = 32;          // bins per tile of the expansion
+
+// out[t][s nz + z] = W_hat of class cls[s]
+__global__ void k_sample_classes(const double* __restrict__ what64, int nt, int nz, const int* __restrict__ cls,
+                                 int ns, double* __restrict__ out) {
+  const long long n = (long long)nt * ns * nz;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    const int t = (int)(i / (ns * nz)), rem = (int)(i - (long long)t * ns * nz);
+    const int s = rem / nz, z = rem - s * nz;
+    out[i] = what64[((size_t)cls[s] * nt + t) * nz + z];
+  }
+}
+
+// One class per block: V = Q^T W_hat (stored FP32 [r][z4], zero padding), and
+// the largest |W_hat - Q V| over the class, each bin relative to dinv[t], as
+// the bits of a non-negative double.
+__global__ void __launch_bounds__(256) k_project(const double* __restrict__ what64, int nt, int nz, int z4,
+                                                 const double* __restrict__ q, const int4* __restrict__ win, int nwin,
+                                                 const double* __restrict__ dinv, int rows, float* __restrict__ v32,
+                                                 unsigned long long* __restrict__ worst) {
+  __shared__ double s_v[TZ_R * 64];
+  const int c = blockIdx.x;
+  const double* w = what64 + (size_t)c * nt * nz;
+  float* out = v32 + (size_t)c * rows * z4;
+  double bad = 0.0;
+  for (int k = 0; k < nwin; ++k) {
+    const int4 g = win[k];  // bins [x, y), first column z, columns w
+    for (int i = threadIdx.x; i < g.w * z4; i += blockDim.x) {
+      const int j = i / z4, z = i - j * z4;
+      double acc = 0.0;
+      if (z < nz) {
+        for (int t = g.x; t < g.y; ++t) acc = fma(q[(size_t)t * TZ_R + j], w[(size_t)t * nz + z], acc);
+        s_v[j * nz + z] = acc;
+      }
+      out[(size_t)(g.z + j) * z4 + z] = (float)acc;
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < (g.y - g.x) * nz; i += blockDim.x) {
+      const int t = g.x + i / nz, z = i - (i / nz) * nz;
+      double acc = w[(size_t)t * nz + z];
+      for (int j = 0; j < g.w; ++j) acc = fma(-q[(size_t)t * TZ_R + j], s_v[j * nz + z], acc);
+      bad = fmax(bad, fabs(acc) * dinv[t]);
+    }
+    __syncthreads();
+  }
+  // padding rows of the table
+  const int used = win[nwin - 1].z + win[nwin - 1].w;
+  for (int i = threadIdx.x; i < (rows - used) * z4; i += blockDim.x) out[(size_t)used * z4 + i] = 0.f;
+  for (int o = 16; o > 0; o >>= 1) bad = fmax(bad, __shfl_xor_sync(0xffffffffu, bad, o));
+  if ((threadIdx.x & 31) == 0 && bad > 0.0) atomicMax(worst, (unsigned long long)__double_as_longlong(bad));
+}
+
+template <int V>
+struct Pix;
+template <>
+struct Pix<1> {
+  using T = float;
+  static __device__ __forceinline__ void get(float (&a)[1], const float* p) { a[0] = *p; }
+  static __device__ __forceinline__ void put(float* p, const float (&a)[1]) { *p = a[0]; }
+};
+template <>
+struct Pix<2> {
+  static __device__ __forceinline__ void get(float (&a)[2], const float* p) {
+    const float2 v = *reinterpret_cast<const float2*>(p);
+    a[0] = v.x;
+    a[1] = v.y;
+  }
+  static __device__ __forceinline__ void put(float* p, const float (&a)[2]) {
+    *reinterpret_cast<float2*>(p) = make_float2(a[0], a[1]);
+  }
+};
+
+// out[b][r0 + j][p] = sum over the window's bins t of Q[t][j] m[b][t][p].
+// Reads m once: the memory system bounds it (16 FMA per 4 bytes).  A block
+// takes 32 V scan points of one window; its eight warps split the window's
+// bins (so that a 100-bin window is 13 independent loads per lane, not a
+// chain of 100) and meet in shared memory in a fixed order.
+template <int V>
+__global__ void __launch_bounds__(256) k_compress(const float* __restrict__ m, int nt, int npix,
+                                                  const float* __restrict__ q, const int4* __restrict__ win, int nwin,
+                                                  int rows, float* __restrict__ out) {
+  __shared__ float s_p[8][TZ_R][32 * V];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int4 g = win[blockIdx.y];
+  const int p0 = blockIdx.x * 32 * V;
+  const int p = p0 + lane * V;
+  const float* src = m + (size_t)blockIdx.z * nt * npix + p;
+  const bool in = p < npix;  // V divides npix
+  float acc[V][TZ_R];
+#pragma unroll
+  for (int u = 0; u < V; ++u)
+#pragma unroll
+    for (int j = 0; j < TZ_R; ++j) acc[u][j] = 0.f;
+  constexpr int U = 8;
+  for (int t0 = g.x + warp; t0 < g.y; t0 += 8 * U) {
+    float v[U][V];
+#pragma unroll
+    for (int i = 0; i < U; ++i) {
+#pragma unroll
+      for (int u = 0; u < V; ++u) v[i][u] = 0.f;
+      if (in && t0 + 8 * i < g.y) Pix<V>::get(v[i], src + (size_t)(t0 + 8 * i) * npix);
+    }
+#pragma unroll
+    for (int i = 0; i < U; ++i) {
+      if (t0 + 8 * i >= g.y) break;
+      const float4* row = reinterpret_cast<const float4*>(q + (size_t)(t0 + 8 * i) * TZ_R);
+#pragma unroll
+      for (int j = 0; j < TZ_R / 4; ++j) {
+        if (4 * j >= g.w) break;
+        const float4 c = __ldg(row + j);
+#pragma unroll
+        for (int u = 0; u < V; ++u) {
+          acc[u][4 * j] = fmaf(c.x, v[i][u], acc[u][4 * j]);
+          acc[u][4 * j + 1] = fmaf(c.y, v[i][u], acc[u][4 * j + 1]);
+          acc[u][4 * j + 2] = fmaf(c.z, v[i][u], acc[u][4 * j + 2]);
+          acc[u][4 * j + 3] = fmaf(c.w, v[i][u], acc[u][4 * j + 3]);
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < TZ_R; ++j)
+#pragma unroll
+    for (int u = 0; u < V; ++u) s_p[warp][j][lane * V + u] = acc[u][j];
+  __syncthreads();
+  float* dst = out + ((size_t)blockIdx.z * rows + g.z) * npix + p0;
+  for (int i = threadIdx.x; i < g.w * 32 * V; i += 256) {
+    const int j = i / (32 * V), x = i - j * 32 * V;
+    if (p0 + x < npix) {
+      float s = 0.f;
+#pragma unroll
+      for (int w = 0; w < 8; ++w) s += s_p[w][j][x];
+      dst[(size_t)j * npix + x] = s;
+    }
+  }
+  // the padding planes behind the last window
+  if (blockIdx.y == nwin - 1) {
+    float* pad = out + ((size_t)blockIdx.z * rows + g.z + g.w) * npix + p0;
+    for (int i = threadIdx.x; i < (rows - g.z - g.w) * 32 * V; i += 256) {
+      const int j = i / (32 * V), x = i - j * 32 * V;
+      if (p0 + x < npix) pad[(size_t)j * npix + x] = 0.f;
+    }
+  }
+}
+
+// m[t][p] = sum_j Q[t][j] y[r0 + j][p] for the bins of one tile (up to 32 bins
+// of one window): the window's planes are held in registers, the bins written
+// as they are formed.  Bound by the writes of m.
+template <int V>
+__global__ void __launch_bounds__(256) k_expand(const float* __restrict__ y, int npix, const float* __restrict__ q,
+                                                const int4* __restrict__ tiles, float* __restrict__ m) {
+  __shared__ float4 s_q[TZ_TILE * TZ_R / 4];
+  const int4 g = tiles[blockIdx.y];  // bins [x, y), first column z, columns w
+  for (int i = threadIdx.x; i < (g.y - g.x) * (TZ_R / 4); i += 256)
+    s_q[i] = reinterpret_cast<const float4*>(q + (size_t)g.x * TZ_R)[i];
+  __syncthreads();
+  const int p = (blockIdx.x * 256 + threadIdx.x) * V;
+  if (p >= npix) return;
+  float v[TZ_R][V];
+#pragma unroll
+  for (int j = 0; j < TZ_R; ++j) {
+#pragma unroll
+    for (int u = 0; u < V; ++u) v[j][u] = 0.f;
+    if (j < g.w) Pix<V>::get(v[j], y + (size_t)(g.z + j) * npix + p);
+  }
+#pragma unroll 4
+  for (int t = 0; t < g.y - g.x; ++t) {
+    float a[V];
+#pragma unroll
+    for (int u = 0; u < V; ++u) a[u] = 0.f;
+#pragma unroll
+    for (int j = 0; j < TZ_R / 4; ++j) {
+      const float4 c = s_q[t * (TZ_R / 4) + j];
+#pragma unroll
+      for (int u = 0; u < V; ++u) {
+        a[u] = fmaf(c.x, v[4 * j][u], a[u]);
+        a[u] = fmaf(c.y, v[4 * j + 1][u], a[u]);
+        a[u] = fmaf(c.z, v[4 * j + 2][u], a[u]);
+        a[u] = fmaf(c.w, v[4 * j + 3][u], a[u]);
+      }
+    }
+    Pix<V>::put(m + (size_t)(g.x + t) * npix + p, a);
+  }
+}
+
+double dot(const double* a, const double* b, size_t n) {
+  double s[4] = {0, 0, 0, 0};
+  size_t i = 0;
+  for (; i + 4 <= n; i += 4)
+    for (int u = 0; u < 4; ++u) s[u] += a[i + u] * b[i + u];
+  for (; i < n; ++i) s[0] += a[i] * b[i];
+  return (s[0] + s[1]) + (s[2] + s[3]);
+}
+
+void axpy(double f, const double* x, double* y, size_t n) {
+  for (size_t i = 0; i < n; ++i) y[i] += f * x[i];
+}
+
+// Basis of the rows [a, b) of w [nt][cols] (column z of sample s at s nz + z):
+// q[t - a][j], j < rank; the rank, or -1 when it is above TZ_R.
+int window_basis(const double* w, int nz, int ns, const double* d, int a, int b, double* q) {
+  const int len = b - a;
+  const size_t cols = (size_t)nz * ns;
+  // scaled rows, columns of no weight dropped
+  std::vector<double> cz(nz, TZ_FLOOR);
+  for (int t = a; t < b; ++t)
+    for (int z = 0; z < nz; ++z) cz[z] = std::max(cz[z], w[t * cols + z] / d[t]);  // sample 0 is DC
+  std::vector<char> keep(cols, 0);
+  for (int t = a; t < b; ++t)
+    for (size_t i = 0; i < cols; ++i)
+      if (fabs(w[t * cols + i]) > 0.1 * TZ_EPS * d[t] * cz[i % nz]) keep[i] = 1;
+  std::vector<size_t> idx;
+  for (size_t i = 0; i < cols; ++i)
+    if (keep[i]) idx.push_back(i);
+  if (idx.empty()) idx.push_back(0);
+  const size_t n = idx.size();
+  std::vector<double> e(len * n), res;
+  for (int t = 0; t < len; ++t)
+    for (size_t i = 0; i < n; ++i) e[t * n + i] = w[(a + t) * cols + idx[i]] / (d[a + t] * cz[idx[i] % nz]);
+  res = e;
+  // rows pivoted by norm, orthonormalised twice, until the residual is below TZ_EPS everywhere
+  std::vector<double> v;
+  int r = 0;
+  for (; r < len; ++r) {
+    double top = 0.0, best = -1.0;
+    int piv = 0;
+    for (int t = 0; t < len; ++t) {
+      const double* x = res.data() + t * n;
+      for (size_t i = 0; i < n; ++i) top = std::max(top, fabs(x[i]));
+      const double nn = dot(x, x, n);
+      if (nn > best) {
+        best = nn;
+        piv = t;
+      }
+    }
+    if (!(top >= TZ_EPS)) break;
+    if (r == TZ_R) return -1;
+    std::vector<double> x(res.begin() + piv * n, res.begin() + (piv + 1) * n);
+    for (int pass = 0; pass < 2; ++pass)
+      for (int j = 0; j < r; ++j) axpy(-dot(x.data(), &v[j * n], n), &v[j * n], x.data(), n);
+    const double nrm = sqrt(dot(x.data(), x.data(), n));
+    if (!(nrm > 0.0)) break;
+    for (double& u : x) u /= nrm;
+    v.insert(v.end(), x.begin(), x.end());
+    for (int t = 0; t < len; ++t) axpy(-dot(&res[t * n], x.data(), n), x.data(), &res[t * n], n);
+  }
+  if (r >= len - 1) {  // nothing to gain: the bins themselves
+    for (int t = 0; t < len; ++t)
+      for (int j = 0; j < len; ++j) q[t * TZ_R + j] = t == j ? 1.0 : 0.0;
+    return len;
+  }
+  // the same space in unscaled bins, orthonormal (the pivot order keeps it graded)
+  std::vector<double> g((size_t)r * len);
+  for (int j = 0; j < r; ++j)
+    for (int t = 0; t < len; ++t) g[j * len + t] = dot(&e[t * n], &v[j * n], n) * d[a + t];
+  for (int j = 0; j < r; ++j) {
+    for (int pass = 0; pass < 3; ++pass) {
+      for (int l = 0; l < j; ++l) axpy(-dot(&g[j * len], &g[l * len], len), &g[l * len], &g[j * len], len);
+      const double nrm = sqrt(dot(&g[j * len], &g[j * len], len));
+      if (!(nrm > 0.0) || !isfinite(nrm)) return -1;
+      for (int t = 0; t < len; ++t) g[j * len + t] /= nrm;
+    }
+    for (int t = 0; t < len; ++t) q[t * TZ_R + j] = g[j * len + t];
+  }
+  return r;
+}
+
+struct Basis {
+  std::vector<double> q;      // [nt][TZ_R]
+  std::vector<int4> win;      // bins [x, y), first column z, columns w
+  std::vector<double> dinv;   // [nt] 1 / DC response of each bin
+  int rank = 0;
+};
+
+bool fit(const std::vector<double>& w, int nt, int nz, int ns, Basis* out) {
+  const size_t cols = (size_t)nz * ns;
+  std::vector<double> d(nt);
+  for (int t = 0; t < nt; ++t) {
+    double mx = 0.0;
+    for (size_t i = 0; i < cols; ++i) {
+      if (!isfinite(w[t * cols + i])) return false;
+      if (i < (size_t)nz) mx = std::max(mx, fabs(w[t * cols + i]));
+    }
+    d[t] = mx > 1e-280 ? mx : 1.0;
+  }
+  std::vector<std::pair<int, int>> todo;
+  for (int a = 0; a < nt;) {
+    int b = std::min(nt, a == 0 ? TZ_FIRST : 2 * a);
+    double mx = d[a];
+    for (int t = a + 1; t < b; ++t) {
+      mx = std::max(mx, d[t]);
+      if (d[t] < TZ_FALL * mx) b = t;
+    }
+    todo.push_back({a, b});
+    a = b;
+  }
+  std::reverse(todo.begin(), todo.end());
+  out->q.assign((size_t)nt * TZ_R, 0.0);
+  out->dinv.resize(nt);
+  for (int t = 0; t < nt; ++t) out->dinv[t] = 1.0 / d[t];
+  while (!todo.empty()) {
+    const auto [a, b] = todo.back();
+    todo.pop_back();
+    const int r = window_basis(w.data(), nz, ns, d.data(), a, b, out->q.data() + (size_t)a * TZ_R);
+    if (r < 0) {
+      if (b - a <= 1) return false;
+      std::fill(out->q.begin() + (size_t)a * TZ_R, out->q.begin() + (size_t)b * TZ_R, 0.0);
+      const int mid = (a + b) / 2;
+      todo.push_back({mid, b});
+      todo.push_back({a, mid});
+      continue;
+    }
+    out->win.push_back(make_int4(a, b, out->rank, r));
+    out->rank += r;
+  }
+  return true;
+}
+
+}  // namespace
+
+// Planes the compressed operator works on for a basis of `rank` columns (a
+// multiple of 16: the plane tiles of the FFT passes and of the tensor-core
+// contractions), or 0 where the nt bins are as cheap: at 48 of 64 planes (config
+// 1) a forward call took 32.8 us against 26.6 on the bins.
+static int compressed_planes(int nt, int rank) {
+  const int rows = ctof_round_up(rank, 16);
+  return 2 * rows <= nt ? rows : 0;
+}
+
+ctof_status time_basis_build(ctof_kernel_s* k, const double* what64, cudaStream_t st) {
+  k->tz = nullptr;
+  const int nt = k->nt, nz = k->nz;
+  if (compressed_planes(nt, TZ_FIRST) == 0) return CTOF_OK;  // too few bins
+  // the classes to fit on: the lowest frequencies (DC first) and an even spread of the rest
+  std::vector<int> cls;
+  for (int i = 0; i < std::min(k->nclass, TZ_SAMPLES / 3); ++i) cls.push_back(i);
+  for (int i = 1; i <= TZ_SAMPLES - TZ_SAMPLES / 3; ++i) {
+    const int c = (int)((long long)(k->nclass - 1) * i / (TZ_SAMPLES - TZ_SAMPLES / 3));
+    if (c > cls.back()) cls.push_back(c);
+  }
+  const int ns = (int)cls.size();
+  std::vector<double> w((size_t)nt * ns * nz);
+  struct Buf {
+    void* p = nullptr;
+    ~Buf() {
+      if (p) cudaFree(p);
+    }
+  } d_cls, d_w, d_q, d_worst;
+  CTOF_CUDA_TRY(cudaMalloc(&d_cls.p, cls.size() * sizeof(int)));
+  CTOF_CUDA_TRY(cudaMalloc(&d_w.p, w.size() * sizeof(double)));
+  CTOF_CUDA_TRY(cudaMemcpyAsync(d_cls.p, cls.data(), cls.size() * sizeof(int), cudaMemcpyHostToDevice, st));
+  k_sample_classes<<<152 * 4, 256, 0, st>>>(what64, nt, nz, static_cast<int*>(d_cls.p), ns,
+                                            static_cast<double*>(d_w.p));
+  CTOF_CUDA_TRY(cudaGetLastError());
+  CTOF_CUDA_TRY(cudaMemcpyAsync(w.data(), d_w.p, w.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
+  CTOF_CUDA_TRY(cudaStreamSynchronize(st));
+  Basis b;
+  if (!fit(w, nt, nz, ns, &b)) return CTOF_OK;
+  const int rows = compressed_planes(nt, b.rank);
+  if (rows == 0) return CTOF_OK;
+  std::vector<int4> tiles;
+  for (const int4& g : b.win)
+    for (int t = g.x; t < g.y; t += TZ_TILE) tiles.push_back(make_int4(t, std::min(g.y, t + TZ_TILE), g.z, g.w));
+  std::vector<float> q32(b.q.size());
+  for (size_t i = 0; i < q32.size(); ++i) q32[i] = (float)b.q[i];
+
+  ctof_kernel_s* z = new (std::nothrow) ctof_kernel_s(*k);
+  if (!z) return CTOF_ENOMEM;
+  z->tz = nullptr;
+  z->nt = rows;
+  z->ldt = rows;
+  auto at = [](size_t& off, size_t bytes) {
+    off = (off + 255) & ~(size_t)255;
+    const size_t o = off;
+    off += bytes;
+    return o;
+  };
+  size_t off = 0;
+  const size_t wa = contract_admm_pipe_floats(rows, nz, 0), ha = contract_admm_pipe_floats(rows, nz, 1);
+  const size_t o_v = at(off, (size_t)k->nclass * rows * k->z4 * sizeof(float));
+  const size_t o_wa = at(off, (size_t)k->nclass * wa * sizeof(float));
+  const size_t o_ha = at(off, (size_t)k->nclass * ha * sizeof(float));
+  const size_t o_q = at(off, q32.size() * sizeof(float));
+  const size_t o_win = at(off, b.win.size() * sizeof(int4));
+  const size_t o_tiles = at(off, tiles.size() * sizeof(int4));
+  const size_t o_m = at(off, (size_t)rows * k->n * k->n * sizeof(float));
+  z->tz_bytes = off;
+  z->d_tz_base = nullptr;
+  if (cudaMalloc(&z->d_tz_base, off) != cudaSuccess) {
+    cudaGetLastError();
+    delete z;
+    return CTOF_ENOMEM;
+  }
+  k->tz = z;  // freed with the handle from here on
+  char* base = static_cast<char*>(z->d_tz_base);
+  z->d_what = reinterpret_cast<float*>(base + o_v);
+  z->d_what_admm = wa ? reinterpret_cast<float*>(base + o_wa) : nullptr;
+  z->d_hinv_admm = wa ? reinterpret_cast<float*>(base + o_ha) : nullptr;
+  z->d_mstage = reinterpret_cast<float*>(base + o_m);
+  z->d_tz_q = reinterpret_cast<float*>(base + o_q);
+  z->d_tz_win = reinterpret_cast<int4*>(base + o_win);
+  z->d_tz_tiles = reinterpret_cast<int4*>(base + o_tiles);
+  z->tz_nwin = (int)b.win.size();
+  z->tz_ntiles = (int)tiles.size();
+  z->tz_nt = nt;
+  const size_t qb = b.q.size() * sizeof(double), db = nt * sizeof(double);
+  CTOF_CUDA_TRY(cudaMalloc(&d_q.p, qb + db));
+  CTOF_CUDA_TRY(cudaMalloc(&d_worst.p, sizeof(unsigned long long)));
+  double* d_dinv = static_cast<double*>(d_q.p) + b.q.size();
+  CTOF_CUDA_TRY(cudaMemcpyAsync(d_q.p, b.q.data(), qb, cudaMemcpyHostToDevice, st));
+  CTOF_CUDA_TRY(cudaMemcpyAsync(d_dinv, b.dinv.data(), db, cudaMemcpyHostToDevice, st));
+  CTOF_CUDA_TRY(cudaMemcpyAsync(z->d_tz_q, q32.data(), q32.size() * sizeof(float), cudaMemcpyHostToDevice, st));
+  CTOF_CUDA_TRY(cudaMemcpyAsync(z->d_tz_win, b.win.data(), b.win.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
+  CTOF_CUDA_TRY(cudaMemcpyAsync(z->d_tz_tiles, tiles.data(), tiles.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
+  CTOF_CUDA_TRY(cudaMemsetAsync(d_worst.p, 0, sizeof(unsigned long long), st));
+  k_project<<<k->nclass, 256, 0, st>>>(what64, nt, nz, k->z4, static_cast<double*>(d_q.p), z->d_tz_win, z->tz_nwin,
+                                       d_dinv, rows, z->d_what, static_cast<unsigned long long*>(d_worst.p));
+  CTOF_CUDA_TRY(cudaGetLastError());
+  unsigned long long bits = 0;
+  CTOF_CUDA_TRY(cudaMemcpyAsync(&bits, d_worst.p, sizeof(bits), cudaMemcpyDeviceToHost, st));
+  CTOF_CUDA_TRY(cudaStreamSynchronize(st));
+  double worst;
+  memcpy(&worst, &bits, sizeof(worst));
+  if (!(worst <= TZ_CHECK)) time_basis_free(k);
+  return CTOF_OK;
+}
+
+void time_basis_free(ctof_kernel_s* k) {
+  ctof_kernel_s* z = k->tz;
+  if (!z) return;
+  cudaFree(z->d_tz_base);
+  delete z;
+  k->tz = nullptr;
+}
+
+ctof_status time_compress(const ctof_kernel_s* z, int batch, const float* m, float* out, cudaStream_t st) {
+  const int npix = z->n * z->n;
+  const bool pair = npix % 2 == 0 && (reinterpret_cast<uintptr_t>(m) & 7) == 0;
+  for (int b0 = 0; b0 < batch; b0 += 65535) {
+    const int nb = std::min(batch - b0, 65535);
+    const float* src = m + (size_t)b0 * z->tz_nt * npix;
+    float* dst = out + (size_t)b0 * z->nt * npix;
+    if (pair)
+      k_compress<2><<<dim3(ctof_div_up(npix, 64), z->tz_nwin, nb), 256, 0, st>>>(src, z->tz_nt, npix, z->d_tz_q,
+                                                                                z->d_tz_win, z->tz_nwin, z->nt, dst);
+    else
+      k_compress<1><<<dim3(ctof_div_up(npix, 32), z->tz_nwin, nb), 256, 0, st>>>(src, z->tz_nt, npix, z->d_tz_q,
+                                                                                z->d_tz_win, z->tz_nwin, z->nt, dst);
+  }
+  CTOF_CUDA_TRY(cudaGetLastError());
+  return CTOF_OK;
+}
+
+ctof_status time_expand(const ctof_kernel_s* z, const float* y, float* m, cudaStream_t st) {
+  const int npix = z->n * z->n;
+  if (npix % 2 == 0 && (reinterpret_cast<uintptr_t>(m) & 7) == 0)
+    k_expand<2><<<dim3(ctof_div_up(npix, 512), z->tz_ntiles), 256, 0, st>>>(y, npix, z->d_tz_q, z->d_tz_tiles, m);
+  else
+    k_expand<1><<<dim3(ctof_div_up(npix, 256), z->tz_ntiles), 256, 0, st>>>(y, npix, z->d_tz_q, z->d_tz_tiles, m);
+  CTOF_CUDA_TRY(cudaGetLastError());
+  return CTOF_OK;
+}
