@@ -955,6 +955,7 @@ ctof_status contract_admm_prepare(ctof_kernel_s* k, cudaStream_t st) {
 
 ctof_status contract_admm(const ctof_kernel_s* k, const float2* c_hat, const float2* s_hat, float2* x_hat,
                           float2* kx_hat, float inv_scale, cudaStream_t st) {
+  if (k->d_what_pitch) return contract_warp_admm(k, c_hat, s_hat, x_hat, kx_hat, inv_scale, st);
   const int stages = k->d_what_admm ? pipe_stages(k->nt, k->nz) : 0;
   if (stages) {
     const PipePlan P = make_pipe_plan(k->nt, k->nz, stages);

@@ -698,20 +698,28 @@ namespace {
 // The x-update's copies of the tables, for the operator that ADMM runs on.
 ctof_status admm_copies(ctof_kernel_s* k, cudaStream_t st) {
   if (!k->tz) {
-    const size_t wa = contract_admm_pipe_floats(k->nt, k->nz, 0), ha = contract_admm_pipe_floats(k->nt, k->nz, 1);
-    if (wa) {
-      const size_t wb = ((size_t)k->nclass * wa * sizeof(float) + 255) & ~(size_t)255;
-      k->admm_bytes = wb + (size_t)k->nclass * ha * sizeof(float);
+    const bool warp = contract_warp_floats(k->nt, k->nz, 0) > 0;
+    Carver cv;
+    const size_t o_wp = cv.take<float>(k->nclass * contract_warp_floats(k->nt, k->nz, 0));
+    const size_t o_w = cv.take<float>(
+        k->nclass * (warp ? contract_warp_floats(k->nt, k->nz, 1) : contract_admm_pipe_floats(k->nt, k->nz, 0)));
+    const size_t o_h = cv.take<float>(
+        k->nclass * (warp ? contract_warp_floats(k->nt, k->nz, 2) : contract_admm_pipe_floats(k->nt, k->nz, 1)));
+    if (cv.off > 0) {
+      k->admm_bytes = cv.off;
       if (cudaMalloc(&k->d_admm, k->admm_bytes) != cudaSuccess) {
         cudaGetLastError();
         k->d_admm = nullptr;
         return CTOF_ENOMEM;
       }
-      k->d_what_admm = static_cast<float*>(k->d_admm);
-      k->d_hinv_admm = reinterpret_cast<float*>(static_cast<char*>(k->d_admm) + wb);
+      char* b = static_cast<char*>(k->d_admm);
+      (warp ? k->d_what_block : k->d_what_admm) = reinterpret_cast<float*>(b + o_w);
+      (warp ? k->d_hinv_block : k->d_hinv_admm) = reinterpret_cast<float*>(b + o_h);
+      if (warp) k->d_what_pitch = reinterpret_cast<float*>(b + o_wp);
     }
   }
   CTOF_TRY(contract_admm_prepare(ctof_ops(k), st));
+  CTOF_TRY(contract_warp_prepare(ctof_ops(k), st));
   CTOF_CUDA_TRY(cudaStreamSynchronize(st));
   return CTOF_OK;
 }
@@ -892,7 +900,9 @@ ctof_status ctof_kernel_get_info(ctof_kernel k, ctof_kernel_info* info) {
   info->scale = k->scale;
   info->gram_max_diag = k->gram_max;
   const ctof_kernel_s* o = ctof_ops(k);
-  info->admm_stages = o->d_what_admm ? contract_admm_pipe_stages(o->nt, o->nz) : 0;
+  info->admm_stages = o->d_what_pitch  ? contract_warp_slots(o->nt, o->nz)
+                      : o->d_what_admm ? contract_admm_pipe_stages(o->nt, o->nz)
+                                       : 0;
   const size_t tik_bytes = (size_t)k->nclass * k->nz * k->z4 * sizeof(float);
   info->device_bytes = k->bytes + k->admm_bytes + (k->tz ? k->tz->tz_bytes : 0) +
                        (k->d_w ? (size_t)k->nt * k->nz * k->q * k->q * sizeof(double) : 0) +

@@ -46,8 +46,11 @@ struct ctof_kernel_s {
   float* d_what;       // [nclass][nt][z4] (zero padding)
   double* d_gram;      // [nclass][nz][nz]
   float* d_hinv;       // [nclass][nz][z4]  (ADMM normal matrix inverse, normalised units)
-  void* d_admm;        // the two copies below (own allocation; null when `tz` holds them)
+  void* d_admm;        // the copies below (own allocation; null when `tz` holds them)
   size_t admm_bytes;
+  float* d_what_pitch; // W_hat rows at the pitch of the one-warp-per-class kernels (or null)
+  float* d_what_block; // with it: W_hat and H^-1 in the 8 x 8 blocks of their x-update
+  float* d_hinv_block;
   float* d_what_admm;  // W_hat in the ADMM kernel's block layout [nclass][tm/8][zm/8][64] (or null)
   float* d_hinv_admm;  // H^-1 in the same layout [nclass][zm/8][zm/8][64] (or null)
   float2* d_tw;        // FFT twiddle table (fft_twiddle_table layout)
@@ -114,7 +117,7 @@ struct ctof_kernel_s {
   int tz_nt;               // bins of the measurement domain
   float* d_tz_q;           // [tz_nt][16] rows of the windows' bases
   int4* d_tz_win;          // windows: bins [x, y), first plane z, planes w
-  int4* d_tz_tiles;        // the windows cut into tiles of up to 32 bins
+  int4* d_tz_tiles;        // the windows cut into tiles of up to 16 bins
   int tz_nwin, tz_ntiles;
 };
 
@@ -264,6 +267,21 @@ struct AdmmQueue {
 ctof_status admm_queue_build(int count, ctof_kernel_s* const* ks, AdmmQueue* out);
 ctof_status admm_queue_launch(const AdmmQueue& q, cudaStream_t st);
 void admm_queue_free(AdmmQueue* q);
+
+// ---- contract_warp.cu -----------------------------------------------------
+// One warp per frequency class, for class blocks of which several fit in
+// shared memory.  Floats per class of their copies (which = 0: pitched W_hat, 1:
+// blocked W_hat, 2: blocked H^-1; 0 floats: they do not apply), the
+// shared-memory slots of the x-update, and the copies' fill.
+size_t contract_warp_floats(int nt, int nz, int which);
+int contract_warp_slots(int nt, int nz);
+ctof_status contract_warp_prepare(const ctof_kernel_s* k, cudaStream_t st);
+ctof_status contract_warp_forward(const ctof_kernel_s* k, const float2* in_z, float2* out_t, cudaStream_t st);
+ctof_status contract_warp_adjoint(const ctof_kernel_s* k, const float2* in_t, float2* out_z, cudaStream_t st);
+ctof_status contract_warp_tikhonov(const ctof_kernel_s* k, const float* hinv, const float2* m_hat, float2* x_hat,
+                                   cudaStream_t st);
+ctof_status contract_warp_admm(const ctof_kernel_s* k, const float2* c_hat, const float2* s_hat, float2* x_hat,
+                               float2* kx_hat, float inv_scale, cudaStream_t st);
 
 // ---- batch_tikhonov.cu ----------------------------------------------------
 size_t batch_tikhonov_smem_bytes(int nt, int nz);

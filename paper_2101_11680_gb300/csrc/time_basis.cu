@@ -418,8 +418,12 @@ ctof_status time_basis_build(ctof_kernel_s* k, const double* what64, cudaStream_
     return o;
   };
   size_t off = 0;
-  const size_t wa = contract_admm_pipe_floats(rows, nz, 0), ha = contract_admm_pipe_floats(rows, nz, 1);
+  const size_t wp = contract_warp_floats(rows, nz, 0);
+  const size_t wa = wp ? 0 : contract_admm_pipe_floats(rows, nz, 0), ha = wp ? 0 : contract_admm_pipe_floats(rows, nz, 1);
   const size_t o_v = at(off, (size_t)k->nclass * rows * k->z4 * sizeof(float));
+  const size_t o_wp = at(off, (size_t)k->nclass * wp * sizeof(float));
+  const size_t o_wb = at(off, (size_t)k->nclass * contract_warp_floats(rows, nz, 1) * sizeof(float));
+  const size_t o_hb = at(off, (size_t)k->nclass * contract_warp_floats(rows, nz, 2) * sizeof(float));
   const size_t o_wa = at(off, (size_t)k->nclass * wa * sizeof(float));
   const size_t o_ha = at(off, (size_t)k->nclass * ha * sizeof(float));
   const size_t o_q = at(off, q32.size() * sizeof(float));
@@ -436,6 +440,9 @@ ctof_status time_basis_build(ctof_kernel_s* k, const double* what64, cudaStream_
   k->tz = z;  // freed with the handle from here on
   char* base = static_cast<char*>(z->d_tz_base);
   z->d_what = reinterpret_cast<float*>(base + o_v);
+  z->d_what_pitch = wp ? reinterpret_cast<float*>(base + o_wp) : nullptr;
+  z->d_what_block = wp ? reinterpret_cast<float*>(base + o_wb) : nullptr;
+  z->d_hinv_block = wp ? reinterpret_cast<float*>(base + o_hb) : nullptr;
   z->d_what_admm = wa ? reinterpret_cast<float*>(base + o_wa) : nullptr;
   z->d_hinv_admm = wa ? reinterpret_cast<float*>(base + o_ha) : nullptr;
   z->d_mstage = reinterpret_cast<float*>(base + o_m);
