@@ -29,6 +29,7 @@
 #include <new>
 #include <vector>
 
+#include "bulk.cuh"
 #include "ctof_internal.h"
 
 namespace {
@@ -40,7 +41,7 @@ constexpr double TZ_EPS = 1e-10;     // scaled residual at which a window's rank
 constexpr double TZ_FLOOR = 1e-6;    // depths below this share of a bin's response are scaled by it instead
 constexpr double TZ_CHECK = 2e-8;    // largest |W_hat - Q V| per bin relative to its DC response
 constexpr int TZ_SAMPLES = 96;       // frequency classes whose rows the basis is fitted on
-constexpr int TZ_TILE = 32;          // bins per tile of the expansion
+constexpr int TZ_TILE = 16;          // bins per tile of the expansion
 
 // out[t][s nz + z] = W_hat of class cls[s]
 __global__ void k_sample_classes(const double* __restrict__ what64, int nt, int nz, const int* __restrict__ cls,
@@ -92,100 +93,192 @@ __global__ void __launch_bounds__(256) k_project(const double* __restrict__ what
   if ((threadIdx.x & 31) == 0 && bad > 0.0) atomicMax(worst, (unsigned long long)__double_as_longlong(bad));
 }
 
-template <int V>
-struct Pix;
-template <>
-struct Pix<1> {
-  using T = float;
-  static __device__ __forceinline__ void get(float (&a)[1], const float* p) { a[0] = *p; }
-  static __device__ __forceinline__ void put(float* p, const float (&a)[1]) { *p = a[0]; }
-};
-template <>
-struct Pix<2> {
-  static __device__ __forceinline__ void get(float (&a)[2], const float* p) {
-    const float2 v = *reinterpret_cast<const float2*>(p);
-    a[0] = v.x;
-    a[1] = v.y;
-  }
-  static __device__ __forceinline__ void put(float* p, const float (&a)[2]) {
-    *reinterpret_cast<float2*>(p) = make_float2(a[0], a[1]);
-  }
-};
-
 // out[b][r0 + j][p] = sum over the window's bins t of Q[t][j] m[b][t][p].
-// Reads m once: the memory system bounds it (16 FMA per 4 bytes).  A block
-// takes 32 V scan points of one window; its eight warps split the window's
-// bins (so that a 100-bin window is 13 independent loads per lane, not a
-// chain of 100) and meet in shared memory in a fixed order.
-template <int V>
+// m is read once; with up to 16 FMA per value the FMA rate comes next to the
+// memory (one volume of 512 bins x 128 x 128: 34 MB, 0.1 GFMA).  Two kernels.
+//
+// k_compress_bulk (scan points in multiples of 4, 16-byte aligned m): a CTA
+// takes 512 / G scan points of one window; the window's rows stream through a
+// four-stage ring of bulk copies (8 G rows and their Q rows per stage, 16 KB),
+// each thread two points, so that the loads in flight do not depend on the
+// registers that the sums need (the register-staged version of this kernel
+// took 288 us for 16 volumes of 512 bins x 128 x 128, 537 MB, against 133 us
+// here).  G = 4 (few CTAs): four groups of threads split each stage's rows and
+// meet in shared memory in a fixed order, which shortens the chain of a
+// 100-bin window from 13 stages to 4.
+//
+// k_compress (anything else): a block takes 32 scan points of one window and
+// its eight warps split the window's bins; their sums meet in shared memory in
+// a fixed order.
+constexpr int CB_PIX = 512, CB_ROWS = 8, CB_STAGES = 4;  // at G = 1
+__host__ __device__ constexpr int cb_stage_bytes(int G) { return CB_ROWS * (CB_PIX + G * TZ_R) * 4; }
+__host__ __device__ constexpr int cb_smem(int G) { return CB_STAGES * (cb_stage_bytes(G) + 8); }
+
+template <int R, int G>
+__device__ __forceinline__ bool compress_window(const float* __restrict__ src, int npix, int pix, int len,
+                                                const float* __restrict__ q, int w, float* __restrict__ dst,
+                                                unsigned char* sm, int* flag, long long max_polls) {
+  constexpr int PIX = CB_PIX / G, ROWS = CB_ROWS * G, SB = cb_stage_bytes(G);
+  uint64_t* bar = reinterpret_cast<uint64_t*>(sm + CB_STAGES * SB);
+  const int nst = (len + ROWS - 1) / ROWS;
+  auto issue = [&](int s) {  // one warp: a row per lane
+    unsigned char* st = sm + (s % CB_STAGES) * SB;
+    const int t0 = s * ROWS, nr = min(ROWS, len - t0), r = threadIdx.x;
+    uint64_t* b = bar + s % CB_STAGES;
+    if (r == 0) {
+      bulk::arrive_expect(b, (unsigned)(nr * (pix + TZ_R) * 4));
+      bulk::g2s(st + ROWS * PIX * 4, q + (size_t)t0 * TZ_R, nr * TZ_R * 4, b);
+    }
+    __syncwarp();
+    if (r < nr) bulk::g2s(st + r * PIX * 4, src + (size_t)(t0 + r) * npix, pix * 4, b);
+  };
+  if (threadIdx.x < 32)
+    for (int s = 0; s < CB_STAGES && s < nst; ++s) issue(s);
+  const int grp = threadIdx.x / (256 / G), pp = threadIdx.x % (256 / G);  // row group, pair of points
+  float2 acc[R];
+#pragma unroll
+  for (int j = 0; j < R; ++j) acc[j] = make_float2(0.f, 0.f);
+  for (int s = 0; s < nst; ++s) {
+    if (!bulk::block_wait(bar + s % CB_STAGES, (uint32_t)(s / CB_STAGES) & 1u, max_polls)) {
+      if (threadIdx.x == 0) {
+        atomicOr(flag, 1);
+        for (int i = s; i < s + CB_STAGES && i < nst; ++i)
+          bulk::wait(bar + i % CB_STAGES, (uint32_t)(i / CB_STAGES) & 1u, bulk::DRAIN_POLLS);
+      }
+      return false;
+    }
+    const unsigned char* st = sm + (s % CB_STAGES) * SB;
+    const float2* row = reinterpret_cast<const float2*>(st) + pp;
+    const float4* qr = reinterpret_cast<const float4*>(st + ROWS * PIX * 4);
+    const int nr = min(ROWS, len - s * ROWS);
+    auto one = [&](int r) {
+      const float2 v = row[r * (PIX / 2)];
+#pragma unroll
+      for (int j = 0; j < R; j += 4) {
+        const float4 c = qr[r * (TZ_R / 4) + j / 4];
+        acc[j] = make_float2(fmaf(c.x, v.x, acc[j].x), fmaf(c.x, v.y, acc[j].y));
+        acc[j + 1] = make_float2(fmaf(c.y, v.x, acc[j + 1].x), fmaf(c.y, v.y, acc[j + 1].y));
+        acc[j + 2] = make_float2(fmaf(c.z, v.x, acc[j + 2].x), fmaf(c.z, v.y, acc[j + 2].y));
+        acc[j + 3] = make_float2(fmaf(c.w, v.x, acc[j + 3].x), fmaf(c.w, v.y, acc[j + 3].y));
+      }
+    };
+    if (nr == ROWS) {
+#pragma unroll
+      for (int r = 0; r < CB_ROWS; ++r) one(G * r + grp);
+    } else {
+      for (int r = grp; r < nr; r += G) one(r);
+    }
+    bulk::fence_smem();  // this stage's reads, before the copies that overwrite it
+    __syncthreads();
+    if (threadIdx.x < 32 && s + CB_STAGES < nst) issue(s + CB_STAGES);
+  }
+  if constexpr (G > 1) {  // the groups' sums, through the (now idle) first stages
+    float2* part = reinterpret_cast<float2*>(sm);
+    if (grp > 0) {
+#pragma unroll
+      for (int j = 0; j < R; ++j) part[((grp - 1) * R + j) * (256 / G) + pp] = acc[j];
+    }
+    __syncthreads();
+    if (grp == 0) {
+#pragma unroll
+      for (int j = 0; j < R; ++j)
+#pragma unroll
+        for (int u = 0; u < G - 1; ++u) {
+          const float2 o = part[(u * R + j) * (256 / G) + pp];
+          acc[j].x += o.x;
+          acc[j].y += o.y;
+        }
+    }
+  }
+  if (grp == 0 && 2 * pp < pix) {
+#pragma unroll
+    for (int j = 0; j < R; ++j)
+      if (j < w) *reinterpret_cast<float2*>(dst + (size_t)j * npix + 2 * pp) = acc[j];
+  }
+  return true;
+}
+
+template <int G>
+__global__ void __launch_bounds__(256, 3) k_compress_bulk(const float* __restrict__ m, int nt, int npix,
+                                                          const float* __restrict__ q, const int4* __restrict__ win,
+                                                          int nwin, int rows, float* __restrict__ out,
+                                                          int* __restrict__ flag, long long max_polls) {
+  extern __shared__ __align__(128) unsigned char csm[];
+  // the longest windows come last: start with them
+  const int k = nwin - 1 - blockIdx.y;
+  const int4 g = win[k];
+  const int p0 = blockIdx.x * (CB_PIX / G), pix = min(CB_PIX / G, npix - p0);
+  if (threadIdx.x == 0)
+    for (int s = 0; s < CB_STAGES; ++s)
+      bulk::bar_init(reinterpret_cast<uint64_t*>(csm + CB_STAGES * cb_stage_bytes(G)) + s, 1);
+  __syncthreads();
+  const float* src = m + ((size_t)blockIdx.z * nt + g.x) * npix + p0;
+  float* dst = out + ((size_t)blockIdx.z * rows + g.z) * npix + p0;
+  const float* qw = q + (size_t)g.x * TZ_R;
+  bool ok;
+  if (g.w <= 4)
+    ok = compress_window<4, G>(src, npix, pix, g.y - g.x, qw, g.w, dst, csm, flag, max_polls);
+  else if (g.w <= 8)
+    ok = compress_window<8, G>(src, npix, pix, g.y - g.x, qw, g.w, dst, csm, flag, max_polls);
+  else if (g.w <= 12)
+    ok = compress_window<12, G>(src, npix, pix, g.y - g.x, qw, g.w, dst, csm, flag, max_polls);
+  else
+    ok = compress_window<16, G>(src, npix, pix, g.y - g.x, qw, g.w, dst, csm, flag, max_polls);
+  if (!ok || k != nwin - 1) return;
+  for (int i = threadIdx.x; i < (rows - g.z - g.w) * (CB_PIX / G); i += 256) {  // the planes behind the last window
+    const int j = i / (CB_PIX / G), x = i % (CB_PIX / G);
+    if (x < pix) dst[(size_t)(g.w + j) * npix + x] = 0.f;
+  }
+}
+
 __global__ void __launch_bounds__(256) k_compress(const float* __restrict__ m, int nt, int npix,
                                                   const float* __restrict__ q, const int4* __restrict__ win, int nwin,
                                                   int rows, float* __restrict__ out) {
-  __shared__ float s_p[8][TZ_R][32 * V];
+  __shared__ float s_p[8][TZ_R][32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int4 g = win[blockIdx.y];
-  const int p0 = blockIdx.x * 32 * V;
-  const int p = p0 + lane * V;
+  const int p = blockIdx.x * 32 + lane;
   const float* src = m + (size_t)blockIdx.z * nt * npix + p;
-  const bool in = p < npix;  // V divides npix
-  float acc[V][TZ_R];
+  const bool in = p < npix;
+  float acc[TZ_R];
 #pragma unroll
-  for (int u = 0; u < V; ++u)
-#pragma unroll
-    for (int j = 0; j < TZ_R; ++j) acc[u][j] = 0.f;
+  for (int j = 0; j < TZ_R; ++j) acc[j] = 0.f;
   constexpr int U = 8;
   for (int t0 = g.x + warp; t0 < g.y; t0 += 8 * U) {
-    float v[U][V];
+    float v[U];
 #pragma unroll
-    for (int i = 0; i < U; ++i) {
-#pragma unroll
-      for (int u = 0; u < V; ++u) v[i][u] = 0.f;
-      if (in && t0 + 8 * i < g.y) Pix<V>::get(v[i], src + (size_t)(t0 + 8 * i) * npix);
-    }
+    for (int i = 0; i < U; ++i) v[i] = in && t0 + 8 * i < g.y ? src[(size_t)(t0 + 8 * i) * npix] : 0.f;
 #pragma unroll
     for (int i = 0; i < U; ++i) {
       if (t0 + 8 * i >= g.y) break;
       const float4* row = reinterpret_cast<const float4*>(q + (size_t)(t0 + 8 * i) * TZ_R);
 #pragma unroll
       for (int j = 0; j < TZ_R / 4; ++j) {
-        if (4 * j >= g.w) break;
         const float4 c = __ldg(row + j);
-#pragma unroll
-        for (int u = 0; u < V; ++u) {
-          acc[u][4 * j] = fmaf(c.x, v[i][u], acc[u][4 * j]);
-          acc[u][4 * j + 1] = fmaf(c.y, v[i][u], acc[u][4 * j + 1]);
-          acc[u][4 * j + 2] = fmaf(c.z, v[i][u], acc[u][4 * j + 2]);
-          acc[u][4 * j + 3] = fmaf(c.w, v[i][u], acc[u][4 * j + 3]);
-        }
+        acc[4 * j] = fmaf(c.x, v[i], acc[4 * j]);
+        acc[4 * j + 1] = fmaf(c.y, v[i], acc[4 * j + 1]);
+        acc[4 * j + 2] = fmaf(c.z, v[i], acc[4 * j + 2]);
+        acc[4 * j + 3] = fmaf(c.w, v[i], acc[4 * j + 3]);
       }
     }
   }
 #pragma unroll
-  for (int j = 0; j < TZ_R; ++j)
-#pragma unroll
-    for (int u = 0; u < V; ++u) s_p[warp][j][lane * V + u] = acc[u][j];
+  for (int j = 0; j < TZ_R; ++j) s_p[warp][j][lane] = acc[j];
   __syncthreads();
-  float* dst = out + ((size_t)blockIdx.z * rows + g.z) * npix + p0;
-  for (int i = threadIdx.x; i < g.w * 32 * V; i += 256) {
-    const int j = i / (32 * V), x = i - j * 32 * V;
-    if (p0 + x < npix) {
-      float s = 0.f;
+  if (!in) return;
+  float* dst = out + ((size_t)blockIdx.z * rows + g.z) * npix + p;
+  const int end = blockIdx.y == nwin - 1 ? rows - g.z : g.w;  // with the padding planes behind the last window
+  for (int j = warp; j < end; j += 8) {
+    float s = 0.f;
+    if (j < g.w) {
 #pragma unroll
-      for (int w = 0; w < 8; ++w) s += s_p[w][j][x];
-      dst[(size_t)j * npix + x] = s;
+      for (int w = 0; w < 8; ++w) s += s_p[w][j][lane];
     }
-  }
-  // the padding planes behind the last window
-  if (blockIdx.y == nwin - 1) {
-    float* pad = out + ((size_t)blockIdx.z * rows + g.z + g.w) * npix + p0;
-    for (int i = threadIdx.x; i < (rows - g.z - g.w) * 32 * V; i += 256) {
-      const int j = i / (32 * V), x = i - j * 32 * V;
-      if (p0 + x < npix) pad[(size_t)j * npix + x] = 0.f;
-    }
+    dst[(size_t)j * npix] = s;
   }
 }
 
-// m[t][p] = sum_j Q[t][j] y[r0 + j][p] for the bins of one tile (up to 32 bins
+// m[t][p] = sum_j Q[t][j] y[r0 + j][p] for the bins of one tile (up to 16 bins
 // of one window): the window's planes are held in registers, the bins written
 // as they are formed.  Bound by the writes of m.
 template <int V>
@@ -193,35 +286,45 @@ __global__ void __launch_bounds__(256) k_expand(const float* __restrict__ y, int
                                                 const int4* __restrict__ tiles, float* __restrict__ m) {
   __shared__ float4 s_q[TZ_TILE * TZ_R / 4];
   const int4 g = tiles[blockIdx.y];  // bins [x, y), first column z, columns w
-  for (int i = threadIdx.x; i < (g.y - g.x) * (TZ_R / 4); i += 256)
-    s_q[i] = reinterpret_cast<const float4*>(q + (size_t)g.x * TZ_R)[i];
-  __syncthreads();
-  const int p = (blockIdx.x * 256 + threadIdx.x) * V;
-  if (p >= npix) return;
+  if ((int)threadIdx.x < (g.y - g.x) * (TZ_R / 4))
+    s_q[threadIdx.x] = reinterpret_cast<const float4*>(q + (size_t)g.x * TZ_R)[threadIdx.x];
+  const int p = (blockIdx.x * 256 + threadIdx.x) * V;  // V divides npix
   float v[TZ_R][V];
 #pragma unroll
   for (int j = 0; j < TZ_R; ++j) {
 #pragma unroll
     for (int u = 0; u < V; ++u) v[j][u] = 0.f;
-    if (j < g.w) Pix<V>::get(v[j], y + (size_t)(g.z + j) * npix + p);
+    if (j < g.w && p < npix) {
+      const float* src = y + (size_t)(g.z + j) * npix + p;
+      if constexpr (V == 2) {
+        const float2 f = *reinterpret_cast<const float2*>(src);
+        v[j][0] = f.x;
+        v[j][V - 1] = f.y;
+      } else {
+        v[j][0] = *src;
+      }
+    }
   }
+  __syncthreads();
+  if (p >= npix) return;
 #pragma unroll 4
   for (int t = 0; t < g.y - g.x; ++t) {
     float a[V];
 #pragma unroll
     for (int u = 0; u < V; ++u) a[u] = 0.f;
 #pragma unroll
-    for (int j = 0; j < TZ_R / 4; ++j) {
-      const float4 c = s_q[t * (TZ_R / 4) + j];
+    for (int j = 0; j < TZ_R; j += 4) {
+      if (j >= g.w) break;
+      const float4 c = s_q[t * (TZ_R / 4) + j / 4];
 #pragma unroll
-      for (int u = 0; u < V; ++u) {
-        a[u] = fmaf(c.x, v[4 * j][u], a[u]);
-        a[u] = fmaf(c.y, v[4 * j + 1][u], a[u]);
-        a[u] = fmaf(c.z, v[4 * j + 2][u], a[u]);
-        a[u] = fmaf(c.w, v[4 * j + 3][u], a[u]);
-      }
+      for (int u = 0; u < V; ++u)
+        a[u] = fmaf(c.w, v[j + 3][u], fmaf(c.z, v[j + 2][u], fmaf(c.y, v[j + 1][u], fmaf(c.x, v[j][u], a[u]))));
     }
-    Pix<V>::put(m + (size_t)(g.x + t) * npix + p, a);
+    float* dst = m + (size_t)(g.x + t) * npix + p;
+    if constexpr (V == 2)
+      *reinterpret_cast<float2*>(dst) = make_float2(a[0], a[V - 1]);
+    else
+      *dst = a[0];
   }
 }
 
@@ -484,17 +587,22 @@ void time_basis_free(ctof_kernel_s* k) {
 
 ctof_status time_compress(const ctof_kernel_s* z, int batch, const float* m, float* out, cudaStream_t st) {
   const int npix = z->n * z->n;
-  const bool pair = npix % 2 == 0 && (reinterpret_cast<uintptr_t>(m) & 7) == 0;
+  const bool bulk = npix % 4 == 0 && (reinterpret_cast<uintptr_t>(m) & 15) == 0;  // (`out` is the library's own)
+  // at G = 1 a CTA takes 512 points of a window: four groups per CTA while those do not fill the chip twice over
+  const bool few = (long long)ctof_div_up(npix, CB_PIX) * z->tz_nwin * batch < 2 * 3 * 152;
+  auto kern = few ? k_compress_bulk<4> : k_compress_bulk<1>;
+  const int smem = few ? cb_smem(4) : cb_smem(1), tile = few ? CB_PIX / 4 : CB_PIX;
+  CTOF_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   for (int b0 = 0; b0 < batch; b0 += 65535) {
     const int nb = std::min(batch - b0, 65535);
     const float* src = m + (size_t)b0 * z->tz_nt * npix;
     float* dst = out + (size_t)b0 * z->nt * npix;
-    if (pair)
-      k_compress<2><<<dim3(ctof_div_up(npix, 64), z->tz_nwin, nb), 256, 0, st>>>(src, z->tz_nt, npix, z->d_tz_q,
-                                                                                z->d_tz_win, z->tz_nwin, z->nt, dst);
+    if (bulk)
+      kern<<<dim3(ctof_div_up(npix, tile), z->tz_nwin, nb), 256, smem, st>>>(
+          src, z->tz_nt, npix, z->d_tz_q, z->d_tz_win, z->tz_nwin, z->nt, dst, z->d_flags, z->max_polls);
     else
-      k_compress<1><<<dim3(ctof_div_up(npix, 32), z->tz_nwin, nb), 256, 0, st>>>(src, z->tz_nt, npix, z->d_tz_q,
-                                                                                z->d_tz_win, z->tz_nwin, z->nt, dst);
+      k_compress<<<dim3(ctof_div_up(npix, 32), z->tz_nwin, nb), 256, 0, st>>>(src, z->tz_nt, npix, z->d_tz_q,
+                                                                             z->d_tz_win, z->tz_nwin, z->nt, dst);
   }
   CTOF_CUDA_TRY(cudaGetLastError());
   return CTOF_OK;
