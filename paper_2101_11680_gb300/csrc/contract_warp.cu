@@ -12,15 +12,15 @@
 // phases.  Launch times with a thread block / a warp per class: forward at
 // 256 x 256 x 32 x 128 (48 planes) 162 / 47 us (42 us of HBM time for what it
 // reads and writes), adjoint at 128 x 128 x 48 x 256 76 / 37 us (20), x-update
-// there 97 / 73 us (37).  Here a CTA (one per SM) holds a ring of shared-memory slots filled by bulk asynchronous
+// there 97 / 66 us (37; 73 us before the depth blocks became a template parameter).  Here a CTA (one per SM) holds a ring of shared-memory slots filled by bulk asynchronous
 // copies, one class per slot, and each of its warps takes every NW-th class
 // through all phases by itself: no block barrier, the warps drift apart and
 // their phases overlap.  The warp that finishes a class refills its slot with
 // the class that follows a ring's length later, so up to NS classes (200 KB)
 // are in flight per SM.
 //
-// Arithmetic is FP32 FMA (fma.rn.f32x2 with the complex pair as the two halves;
-// the x-update: TF32 tensor-core products in three terms, as in contract_admm.cu).  Adjoint passes give a lane one 16-byte chunk of a
+// Arithmetic is FP32 FMA (the x-update: TF32 tensor-core products in three terms,
+// as in contract_admm.cu).  Adjoint passes give a lane one 16-byte chunk of a
 // row and one of 32/q interleaved row sets, for all eight right-hand sides, so
 // each word of the block is read once; the row sets meet in the warp's scratch.
 // Forward passes give a lane whole rows (row pitch 4 (q | 1) words: 16-byte
@@ -134,20 +134,9 @@ struct WarpArgs {
   float inv_s;
 };
 
-__device__ __forceinline__ unsigned long long pack2(float a, float b) {
-  unsigned long long r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ float2 unpack2(unsigned long long v) {
-  float2 r;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-  return r;
-}
-__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
-  unsigned long long d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
+__device__ __forceinline__ void cfma(float2& acc, float w, float x, float y) {
+  acc.x = fmaf(w, x, acc.x);
+  acc.y = fmaf(w, y, acc.y);
 }
 
 // Partials over row set j of sum M[r][z] v[m][r], one lane per (j, chunk);
@@ -156,11 +145,11 @@ __device__ __forceinline__ void adj_pass(const WarpPlan& P, const float* M, int 
                                          int vpitch, float2* part, int lane) {
   const int j = lane / P.q, k = lane - j * P.q;
   if (j < P.J) {
-    unsigned long long acc[4][4];
+    float2 acc[4][4];
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
-      for (int m = 0; m < 4; ++m) acc[a][m] = 0ull;
+      for (int m = 0; m < 4; ++m) acc[a][m] = make_float2(0.f, 0.f);
     const int per = ((rows + P.J - 1) / P.J + 1) & ~1;
     const int r0 = j * per, r1 = min(rows, r0 + per);
     const float* mp = M + 4 * k;
@@ -169,30 +158,40 @@ __device__ __forceinline__ void adj_pass(const WarpPlan& P, const float* M, int 
     for (; r + 2 <= r1; r += 2) {
       const float4 w0 = *reinterpret_cast<const float4*>(mp + r * pitch);
       const float4 w1 = *reinterpret_cast<const float4*>(mp + (r + 1) * pitch);
-      const unsigned long long p0[4] = {pack2(w0.x, w0.x), pack2(w0.y, w0.y), pack2(w0.z, w0.z), pack2(w0.w, w0.w)};
-      const unsigned long long p1[4] = {pack2(w1.x, w1.x), pack2(w1.y, w1.y), pack2(w1.z, w1.z), pack2(w1.w, w1.w)};
+      float4 c[4];
+#pragma unroll
+      for (int m = 0; m < 4; ++m) c[m] = *reinterpret_cast<const float4*>(v + m * vpitch + r);
 #pragma unroll
       for (int m = 0; m < 4; ++m) {
-        const ulonglong2 c = *reinterpret_cast<const ulonglong2*>(v + m * vpitch + r);
+        cfma(acc[0][m], w0.x, c[m].x, c[m].y);
+        cfma(acc[1][m], w0.y, c[m].x, c[m].y);
+        cfma(acc[2][m], w0.z, c[m].x, c[m].y);
+        cfma(acc[3][m], w0.w, c[m].x, c[m].y);
+      }
 #pragma unroll
-        for (int a = 0; a < 4; ++a) acc[a][m] = fma2(p1[a], c.y, fma2(p0[a], c.x, acc[a][m]));
+      for (int m = 0; m < 4; ++m) {
+        cfma(acc[0][m], w1.x, c[m].z, c[m].w);
+        cfma(acc[1][m], w1.y, c[m].z, c[m].w);
+        cfma(acc[2][m], w1.z, c[m].z, c[m].w);
+        cfma(acc[3][m], w1.w, c[m].z, c[m].w);
       }
     }
     if (r < r1) {
       const float4 w0 = *reinterpret_cast<const float4*>(mp + r * pitch);
-      const unsigned long long p0[4] = {pack2(w0.x, w0.x), pack2(w0.y, w0.y), pack2(w0.z, w0.z), pack2(w0.w, w0.w)};
 #pragma unroll
       for (int m = 0; m < 4; ++m) {
-        const unsigned long long c = *reinterpret_cast<const unsigned long long*>(v + m * vpitch + r);
-#pragma unroll
-        for (int a = 0; a < 4; ++a) acc[a][m] = fma2(p0[a], c, acc[a][m]);
+        const float2 c = v[m * vpitch + r];
+        cfma(acc[0][m], w0.x, c.x, c.y);
+        cfma(acc[1][m], w0.y, c.x, c.y);
+        cfma(acc[2][m], w0.z, c.x, c.y);
+        cfma(acc[3][m], w0.w, c.x, c.y);
       }
     }
-    ulonglong2* dst = reinterpret_cast<ulonglong2*>(part) + lane;
+    float4* dst = reinterpret_cast<float4*>(part) + lane;
 #pragma unroll
     for (int a = 0; a < 4; ++a) {
-      dst[(2 * a) * PART_PITCH] = make_ulonglong2(acc[a][0], acc[a][1]);
-      dst[(2 * a + 1) * PART_PITCH] = make_ulonglong2(acc[a][2], acc[a][3]);
+      dst[(2 * a) * PART_PITCH] = make_float4(acc[a][0].x, acc[a][0].y, acc[a][1].x, acc[a][1].y);
+      dst[(2 * a + 1) * PART_PITCH] = make_float4(acc[a][2].x, acc[a][2].y, acc[a][3].x, acc[a][3].y);
     }
   }
   __syncwarp();
@@ -218,28 +217,31 @@ __device__ __forceinline__ void fwd_pass(const WarpPlan& P, const float* W, cons
     const bool two = t0 + 32 < P.nt;
     const float* wa = W + t0 * P.sw;
     const float* wb = two ? wa + 32 * P.sw : wa;
-    unsigned long long a[4], b[4];
+    float2 a[4], b[4];
 #pragma unroll
-    for (int m = 0; m < 4; ++m) a[m] = b[m] = 0ull;
+    for (int m = 0; m < 4; ++m) a[m] = b[m] = make_float2(0.f, 0.f);
 #pragma unroll 2
     for (int k = 0; k < P.q; ++k) {
       const float4 u = *reinterpret_cast<const float4*>(wa + 4 * k);
       const float4 v = *reinterpret_cast<const float4*>(wb + 4 * k);
-      const unsigned long long pu[4] = {pack2(u.x, u.x), pack2(u.y, u.y), pack2(u.z, u.z), pack2(u.w, u.w)};
-      const unsigned long long pv[4] = {pack2(v.x, v.x), pack2(v.y, v.y), pack2(v.z, v.z), pack2(v.w, v.w)};
 #pragma unroll
-      for (int m = 0; m < 4; ++m) {
-        const ulonglong2 c0 = *reinterpret_cast<const ulonglong2*>(x + m * xpitch + 4 * k);
-        const ulonglong2 c1 = *reinterpret_cast<const ulonglong2*>(x + m * xpitch + 4 * k + 2);
-        a[m] = fma2(pu[3], c1.y, fma2(pu[2], c1.x, fma2(pu[1], c0.y, fma2(pu[0], c0.x, a[m]))));
-        b[m] = fma2(pv[3], c1.y, fma2(pv[2], c1.x, fma2(pv[1], c0.y, fma2(pv[0], c0.x, b[m]))));
+      for (int h = 0; h < 2; ++h) {
+        const float u0 = h ? u.z : u.x, u1 = h ? u.w : u.y, v0 = h ? v.z : v.x, v1 = h ? v.w : v.y;
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+          const float4 c = *reinterpret_cast<const float4*>(x + m * xpitch + 4 * k + 2 * h);
+          cfma(a[m], u0, c.x, c.y);
+          cfma(b[m], v0, c.x, c.y);
+          cfma(a[m], u1, c.z, c.w);
+          cfma(b[m], v1, c.z, c.w);
+        }
       }
     }
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
       if (mem[m] < 0) continue;
-      out[(size_t)mem[m] * ld + t0] = unpack2(a[m]);
-      if (two) out[(size_t)mem[m] * ld + t0 + 32] = unpack2(b[m]);
+      out[(size_t)mem[m] * ld + t0] = a[m];
+      if (two) out[(size_t)mem[m] * ld + t0 + 32] = b[m];
     }
   }
 }
@@ -363,7 +365,7 @@ __device__ __forceinline__ bool pair_any(int id, bool v) {
 // two products split their K steps between the warps, which exchange half of
 // the partial sums: warp `half` finishes rows 8 half + g of every 16-row tile;
 // the third splits the t tiles.
-template <int MZ>
+template <int ZB>
 __device__ __forceinline__ void do_admm(const WarpArgs& A, const unsigned char* st, float* vec, int half, int bar,
                                         int lane) {
   const WarpPlan& P = A.P;
@@ -371,7 +373,8 @@ __device__ __forceinline__ void do_admm(const WarpArgs& A, const unsigned char* 
   const int offF0 = 4 * g + tg, offF2 = 32 + 4 * ((g + 4) & 7) + tg;  // (row g, columns tg, tg + 4)
   const int offA0 = 32 * hg + 4 * ((tg + 4 * hg) & 7) + (g & 3);      // (row tg, column g)
   const int offA2 = 32 * hg + 4 * ((tg + 4 + 4 * hg) & 7) + (g & 3);  // (row tg + 4, column g)
-  const int TB = P.tb, ZB = P.zb, nt = P.nt, nz = P.nz;
+  constexpr int MZ = (ZB + 1) / 2;  // 16-row z tiles
+  const int TB = P.tb, nt = P.nt, nz = P.nz;
   const float* W = reinterpret_cast<const float*>(st);
   const float* H = reinterpret_cast<const float*>(st + P.o_h);
   const float* C = reinterpret_cast<const float*>(st + P.o_c) + (g >> 1) * 2 * P.cs + (g & 1);
@@ -452,7 +455,7 @@ __device__ __forceinline__ void do_admm(const WarpArgs& A, const unsigned char* 
 #pragma unroll
   for (int kk = 0; kk < MZ; ++kk) {
     const int ks = 2 * kk + half;
-    if (ks >= ZB) break;
+    if (ks >= ZB) break;  // (odd ZB: the second warp has one step less)
     unsigned b[4];
     split_fast(vec[(8 * ks + tg) * 8 + g], b[0], b[2]);
     split_fast(vec[(8 * ks + tg + 4) * 8 + g], b[1], b[3]);
@@ -480,10 +483,9 @@ __device__ __forceinline__ void do_admm(const WarpArgs& A, const unsigned char* 
   }
   pair_sync(bar);
   // ---- Kx = W x / s, two 16-row tiles at a time ----
-  unsigned xb[2 * MZ][4];
+  unsigned xb[ZB][4];
 #pragma unroll
-  for (int ks = 0; ks < 2 * MZ; ++ks) {
-    if (ks >= ZB) break;
+  for (int ks = 0; ks < ZB; ++ks) {
     split_fast(vec[(8 * ks + tg) * 8 + g], xb[ks][0], xb[ks][2]);
     split_fast(vec[(8 * ks + tg + 4) * 8 + g], xb[ks][1], xb[ks][3]);
   }
@@ -497,8 +499,7 @@ __device__ __forceinline__ void do_admm(const WarpArgs& A, const unsigned char* 
     const float* w = W + (size_t)r0 * ZB * 64;
     const bool b1 = r0 + 1 < TB, b2 = r0 + 2 < TB, b3 = r0 + 3 < TB;
 #pragma unroll
-    for (int ks = 0; ks < 2 * MZ; ++ks) {
-      if (ks >= ZB) break;
+    for (int ks = 0; ks < ZB; ++ks) {
       const float* q = w + ks * 64;
       const float a0[4] = {q[offF0], b1 ? q[ZB * 64 + offF0] : 0.f, q[offF2], b1 ? q[ZB * 64 + offF2] : 0.f};
       mma_3x(eh[0], el[0], a0, xb[ks]);
@@ -541,8 +542,8 @@ __device__ __forceinline__ bool wait_fill(uint64_t* full, const int* issued, int
   return bulk::wait(full, (uint32_t)(n - 1) & 1u, max_polls);
 }
 
-// MZ: 16-row z tiles of the ADMM products (ceil(nz / 16)).
-template <int MODE, int MZ>
+// ZB: 8-row z blocks of the ADMM products (ceil(nz / 8)).
+template <int MODE, int ZB>
 __global__ void __launch_bounds__(MODE == WM_ADMM ? MAX_PAIRS * 64 : MAX_WARPS * 32, 1) k_contract_warp(const __grid_constant__ WarpArgs A,
                                                                      int* __restrict__ flag, long long max_polls) {
   extern __shared__ __align__(128) unsigned char wsm[];
@@ -589,7 +590,7 @@ __global__ void __launch_bounds__(MODE == WM_ADMM ? MAX_PAIRS * 64 : MAX_WARPS *
     }
     unsigned char* scr = wsm + P.o_scr + worker * P.scratch;
     if constexpr (MODE == WM_ADMM)
-      do_admm<MZ>(A, wsm + s * P.slot, reinterpret_cast<float*>(scr), (threadIdx.x >> 5) & 1, 1 + worker, lane);
+      do_admm<ZB>(A, wsm + s * P.slot, reinterpret_cast<float*>(scr), (threadIdx.x >> 5) & 1, 1 + worker, lane);
     else
       do_class<MODE>(A, wsm + s * P.slot, scr, lane);
     bulk::fence_smem();  // the worker's accesses of the slot, before the copies into it
@@ -631,7 +632,7 @@ __global__ void k_block_rows(const float* __restrict__ src, int rows, int cols, 
   }
 }
 
-template <int MODE, int MZ>
+template <int MODE, int ZB>
 ctof_status launch(const ctof_kernel_s* k, const WarpPlan& P, WarpArgs& A, cudaStream_t st) {
   A.P = P;
   A.w = MODE == WM_ADMM ? k->d_what_block : k->d_what_pitch;
@@ -640,7 +641,7 @@ ctof_status launch(const ctof_kernel_s* k, const WarpPlan& P, WarpArgs& A, cudaS
   A.nclass = k->nclass;
   A.ldt = k->ldt;
   A.ldz = k->ldz;
-  auto kern = k_contract_warp<MODE, MZ>;
+  auto kern = k_contract_warp<MODE, ZB>;
   CTOF_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, P.total));
   int nsm = 152;
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, k->device);
@@ -714,10 +715,14 @@ ctof_status contract_warp_admm(const ctof_kernel_s* k, const float2* c_hat, cons
   A.x_hat = x_hat;
   A.out_t = kx_hat;
   A.inv_s = inv_scale;
-  switch ((k->nz + 15) / 16) {
+  switch ((k->nz + 7) / 8) {
     case 1: return launch<WM_ADMM, 1>(k, P, A, st);
     case 2: return launch<WM_ADMM, 2>(k, P, A, st);
     case 3: return launch<WM_ADMM, 3>(k, P, A, st);
-    default: return launch<WM_ADMM, 4>(k, P, A, st);
+    case 4: return launch<WM_ADMM, 4>(k, P, A, st);
+    case 5: return launch<WM_ADMM, 5>(k, P, A, st);
+    case 6: return launch<WM_ADMM, 6>(k, P, A, st);
+    case 7: return launch<WM_ADMM, 7>(k, P, A, st);
+    default: return launch<WM_ADMM, 8>(k, P, A, st);
   }
 }
