@@ -176,21 +176,19 @@ ctof_status admm_contract(ctof_kernel_s* k, cudaStream_t st) {
   return contract_admm(k, k->d_spec_t2, k->d_spec_z, k->d_spec_z2, k->d_spec_t, (float)(1.0 / k->scale), st);
 }
 
-// The rest of iteration `it`: T side (K x -> v1/u1 -> c_hat; not after the
-// last iteration) and Z side (x -> TV / nonnegativity prox -> s_hat; the last
-// iteration writes the crop of v3 to d_vstage).  `ev_mid` (optional) is
-// recorded between the two.
-ctof_status admm_side(ctof_kernel_s* k, const ctof_solver_params* prm, int it, cudaStream_t st, cudaEvent_t ev_mid) {
-  const int nt = k->nt, nz = k->nz, n = k->n, P = k->p;
-  const float inv_s = (float)(1.0 / k->scale);
+// T side of an iteration (not after the last): K x -> v1/u1 -> c_hat.
+ctof_status admm_t_side(ctof_kernel_s* k, const ctof_solver_params* prm, cudaStream_t st) {
+  CTOF_TRY(fft_cols_inverse(k, k->d_spec_t, k->ldt, k->nt, k->n, k->d_inter_t, st));
+  CTOF_TRY(fft_rows_admm_t(k, k->d_inter_t, k->d_mstage, k->d_u1, (float)(1.0 / k->scale), (float)prm->rho, st));
+  return fft_cols_forward(k, k->d_inter_t, k->nt, k->n, k->d_spec_t2, k->ldt, st);
+}
+
+// Z side of iteration `it`: x -> TV / nonnegativity prox -> s_hat (the last
+// iteration writes the crop of v3 to d_vstage instead).
+ctof_status admm_z_side(ctof_kernel_s* k, const ctof_solver_params* prm, int it, cudaStream_t st) {
+  const int nz = k->nz, P = k->p;
   const float rho = (float)prm->rho;
   const bool last = it == prm->iters - 1;
-  if (!last) {
-    CTOF_TRY(fft_cols_inverse(k, k->d_spec_t, k->ldt, nt, n, k->d_inter_t, st));
-    CTOF_TRY(fft_rows_admm_t(k, k->d_inter_t, k->d_mstage, k->d_u1, inv_s, rho, st));
-    CTOF_TRY(fft_cols_forward(k, k->d_inter_t, nt, n, k->d_spec_t2, k->ldt, st));
-  }
-  if (ev_mid) CTOF_CUDA_TRY(cudaEventRecordWithFlags(ev_mid, st, cudaEventRecordExternal));
   float* u2[2] = {k->d_u2a, k->d_u2b};
   CTOF_TRY(fft_cols_inverse(k, k->d_spec_z2, k->ldz, nz, P, k->d_inter_z, st));
   CTOF_TRY(fft_rows_inverse(k, k->d_inter_z, nz, P, P, k->d_xs, P, st));
@@ -203,9 +201,53 @@ ctof_status admm_side(ctof_kernel_s* k, const ctof_solver_params* prm, int it, c
   return CTOF_OK;
 }
 
+// The rest of iteration `it` after the x-update, one side after the other;
+// `ev_mid` (optional) is recorded between the two.
+ctof_status admm_side(ctof_kernel_s* k, const ctof_solver_params* prm, int it, cudaStream_t st, cudaEvent_t ev_mid) {
+  if (it != prm->iters - 1) CTOF_TRY(admm_t_side(k, prm, st));
+  if (ev_mid) CTOF_CUDA_TRY(cudaEventRecordWithFlags(ev_mid, st, cudaEventRecordExternal));
+  return admm_z_side(k, prm, it, st);
+}
+
+// A branch of a captured graph: `side` runs from where `st` is at fork() until join().
+struct GraphBranch {
+  cudaStream_t side = nullptr;
+  cudaEvent_t ev = nullptr;
+  ~GraphBranch() {
+    if (ev) cudaEventDestroy(ev);
+    if (side) cudaStreamDestroy(side);
+  }
+  ctof_status make() {
+    CTOF_CUDA_TRY(cudaStreamCreateWithFlags(&side, cudaStreamNonBlocking));
+    CTOF_CUDA_TRY(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+    return CTOF_OK;
+  }
+  ctof_status order(cudaStream_t first, cudaStream_t then) {
+    CTOF_CUDA_TRY(cudaEventRecord(ev, first));
+    CTOF_CUDA_TRY(cudaStreamWaitEvent(then, ev, 0));
+    return CTOF_OK;
+  }
+};
+
 // ADMM on the staged measurement d_mstage; result (crop of v3) in d_vstage.
+// The two sides of an iteration touch different state and neither fills the
+// chip alone (short chains of latency-bound passes), so they run as two
+// branches of the graph (one after the other when the stages are timed).
 ctof_status admm_enqueue(ctof_kernel_s* k, const ctof_solver_params* prm, cudaStream_t st, bool timed) {
   CTOF_TRY(admm_setup(k, prm, st));
+  if (!(timed && k->timing)) {
+    GraphBranch br;
+    CTOF_TRY(br.make());
+    for (int it = 0; it < prm->iters; ++it) {
+      CTOF_TRY(admm_contract(k, st));
+      if (it == prm->iters - 1) return admm_z_side(k, prm, it, st);
+      CTOF_TRY(br.order(st, br.side));
+      CTOF_TRY(admm_t_side(k, prm, br.side));
+      CTOF_TRY(admm_z_side(k, prm, it, st));
+      CTOF_TRY(br.order(br.side, st));
+    }
+    return CTOF_OK;
+  }
   cudaEvent_t* ev = (timed && k->timing) ? k->events : nullptr;
   for (int it = 0; it < prm->iters; ++it) {
     if (ev) CTOF_CUDA_TRY(cudaEventRecordWithFlags(ev[4 * it + 0], st, cudaEventRecordExternal));
