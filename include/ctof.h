@@ -321,22 +321,17 @@ ctof_status ctof_learned_reconstruct_checked(ctof_learned net, ctof_kernel k, in
 
 /* Batching form: ADMM reconstructions of `count` independent problems of
  * uneven sizes and optics (one handle each, distinct handles), d_m[i] ->
- * d_mu[i] with the layouts of ctof_reconstruct, all with `params`.  The batch
- * is one captured CUDA graph: per iteration, the x-update of every problem
- * whose class blocks fit the shared stages of the largest of them runs as one
- * persistent launch whose thread blocks take (problem, frequency class) items
- * from a device work queue; the other problems' x-updates and every problem's
- * FFT / TV stages run on forked streams.  The graph is kept and replayed
- * while the same handles, buffers and parameters come back (one cached batch
- * graph per process); results are bit-identical to reconstructing each
- * problem alone.  Handles not yet tuned are autotuned first (see
- * ctof_kernel_autotune), so the first call synchronises and must not be made
- * inside a stream capture.  The batch must not overlap other calls on its
- * handles.  Asynchronous after the first call; a bounded wait that runs out
- * in the queued launch is reported on the first queued handle (the wait limit
- * in force when the graph was made applies).  Errors: EINVAL (bad or
- * repeated handle, null buffer, handles on different devices), ENOMEM,
- * ECUDA. */
+ * d_mu[i] with the layouts of ctof_reconstruct, all with `params`.  Every
+ * problem runs its handle's captured ADMM graph (the one ctof_reconstruct uses,
+ * kept while the parameters come back, whatever the buffers) on a stream of its
+ * own that starts where `stream` is; `stream` goes on when all are done.
+ * Results are bit-identical to reconstructing each problem alone.  Handles not
+ * yet tuned are autotuned first (see ctof_kernel_autotune), so the first call
+ * synchronises and must not be made inside a stream capture.  The batch must
+ * not overlap other calls on its handles.  Asynchronous after the first call;
+ * a bounded wait that runs out is reported on the handle of its problem.
+ * Errors: EINVAL (bad or repeated handle, null buffer, handles on different
+ * devices), ENOMEM, ECUDA. */
 ctof_status ctof_reconstruct_batch(int count, const ctof_kernel* ks, const float* const* d_m,
                                    const ctof_solver_params* params, float* const* d_mu, void* stream);
 

@@ -51,9 +51,6 @@
 //   forward part: one warp per 16-row tile of t.
 #include <cuda_runtime.h>
 
-#include <algorithm>
-#include <vector>
-
 #include "ctof_internal.h"
 
 namespace {
@@ -526,7 +523,6 @@ struct PipeProb {
   float2* kx_hat;        // [nf][ldt] out
   int ldt, ldz;
   float inv_s;
-  int item0;             // first work-queue item of this problem
 };
 
 // Producer: class c of problem q into stage `st` (header, then the bulk copies
@@ -541,10 +537,7 @@ __device__ __forceinline__ void produce_item(const PipeProb& q, int c, unsigned 
     if (f[m] >= 0) bytes += P.c_bytes + 2 * P.v_bytes;
   }
   // the class header (members + 1, diagonal of L) for the consumers; the
-  // arrive below releases these stores to them.  Header words stay small
-  // non-negative integers or finite floats: in the many-problem kernel one
-  // problem's header may sit inside another's operand padding, which is then
-  // multiplied by zero.
+  // arrive below releases these stores to them
   int* hdr = reinterpret_cast<int*>(st + P.o_hdr);
 #pragma unroll
   for (int m = 0; m < 4; ++m) hdr[m] = f[m] + 1;
@@ -570,15 +563,12 @@ struct PipeScratch {
   unsigned* xl;
 };
 
-// Consumers (8 warps): the x-update of the class in stage `st`.  KZC > 0 fixes
-// the forward K steps at compile time; KZC = 0 takes them from the problem
-// (at most 8), with the same operations in the same order.  `gave_up` is this
-// thread's full-barrier timeout; returns true when the CTA must stop.
-template <int KZC>
+// Consumers (8 warps): the x-update of the class in stage `st`; KZ = forward K
+// steps = ceil(nz / 8).  `gave_up` is this thread's full-barrier timeout;
+// returns true when the CTA must stop.
+template <int KZ>
 __device__ __forceinline__ bool consume_item(const PipeProb& q, const unsigned char* st, const PipeScratch& scr,
                                              int gave_up) {
-  constexpr int KZM = KZC > 0 ? KZC : 8;
-  constexpr int MZM = (KZM + 1) / 2;
   const PipePlan& P = q.P;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int g = lane >> 2, tg = lane & 3;
@@ -589,8 +579,7 @@ __device__ __forceinline__ bool consume_item(const PipeProb& q, const unsigned c
   const int offA0 = 32 * hg + 4 * ((tg + 4 * hg) & 7) + (g & 3);      // (row tg, column g)
   const int offA2 = 32 * hg + 4 * ((tg + 4 + 4 * hg) & 7) + (g & 3);  // (row tg + 4, column g)
   const int nt = P.nt, nz = P.nz;
-  const int KZ = KZC > 0 ? KZC : (nz + 7) >> 3;
-  const int MZ = (KZ + 1) >> 1, ZB = 2 * MZ, ZM = 16 * MZ;
+  constexpr int MZ = (KZ + 1) / 2, ZB = 2 * MZ, ZM = 16 * MZ;
   const int kt = (nt + 7) >> 3, mtt = P.tm >> 4;
   const float inv_s = q.inv_s;
   const float* W = reinterpret_cast<const float*>(st + P.o_w);
@@ -602,9 +591,9 @@ __device__ __forceinline__ bool consume_item(const PipeProb& q, const unsigned c
 
   // ---- A: adjoint partial sums y_w[z][r] = sum over this warp's t of W[t][z] c[t][r] ----
   {
-    float acc[MZM][4];
+    float acc[MZ][4];
 #pragma unroll
-    for (int mt = 0; mt < MZM; ++mt)
+    for (int mt = 0; mt < MZ; ++mt)
 #pragma unroll
       for (int i = 0; i < 4; ++i) acc[mt][i] = 0.f;
     const float* cr = C + (g >> 1) * P.cs + 2 * tg + (g & 1) + 16 * warp;  // t = 8 ks + tg
@@ -616,23 +605,19 @@ __device__ __forceinline__ bool consume_item(const PipeProb& q, const unsigned c
       split_fast(cr[0], bh0, bl0);
       split_fast(cr[8], bh1, bl1);
 #pragma unroll
-      for (int mt = 0; mt < MZM; ++mt) {
-        if (mt < MZ) {
-          const float a[4] = {wa0[128 * mt], wa0[128 * mt + 64], wa2[128 * mt], wa2[128 * mt + 64]};
-          mma_split_a(acc[mt], a, bh0, bh1, bl0, bl1);
-        }
+      for (int mt = 0; mt < MZ; ++mt) {
+        const float a[4] = {wa0[128 * mt], wa0[128 * mt + 64], wa2[128 * mt], wa2[128 * mt + 64]};
+        mma_split_a(acc[mt], a, bh0, bh1, bl0, bl1);
       }
       cr += 16 * PIPE_CONS_WARPS;
       wa0 += PIPE_CONS_WARPS * ZB * 64;
       wa2 += PIPE_CONS_WARPS * ZB * 64;
     }
 #pragma unroll
-    for (int mt = 0; mt < MZM; ++mt) {
-      if (mt < MZ) {
-        float* p = scr.part + (warp * ZM + 16 * mt + g) * 8 + 2 * tg;
-        *reinterpret_cast<float2*>(p) = make_float2(acc[mt][0], acc[mt][1]);
-        *reinterpret_cast<float2*>(p + 64) = make_float2(acc[mt][2], acc[mt][3]);
-      }
+    for (int mt = 0; mt < MZ; ++mt) {
+      float* p = scr.part + (warp * ZM + 16 * mt + g) * 8 + 2 * tg;
+      *reinterpret_cast<float2*>(p) = make_float2(acc[mt][0], acc[mt][1]);
+      *reinterpret_cast<float2*>(p + 64) = make_float2(acc[mt][2], acc[mt][3]);
     }
   }
   if (cons_sync_or(gave_up)) return true;
@@ -667,13 +652,11 @@ __device__ __forceinline__ bool consume_item(const PipeProb& q, const unsigned c
     float ah[4] = {0.f, 0.f, 0.f, 0.f}, al[4] = {0.f, 0.f, 0.f, 0.f};
     const float* h0 = H + 2 * warp * ZB * 64;  // block (z / 8 = 2 warp, w / 8 = 0)
 #pragma unroll
-    for (int ks = 0; ks < 2 * MZM; ++ks) {
-      if (ks < ZB) {
-        const float* hb = h0 + ks * 64;
-        const float a[4] = {hb[offF0], hb[ZB * 64 + offF0], hb[offF2], hb[ZB * 64 + offF2]};
-        const int b0 = (8 * ks + tg) * 8 + g, b1 = b0 + 32;
-        mma_split_a_2acc(ah, al, a, scr.bh[b0], scr.bh[b1], scr.bl[b0], scr.bl[b1]);
-      }
+    for (int ks = 0; ks < 2 * MZ; ++ks) {
+      const float* hb = h0 + ks * 64;
+      const float a[4] = {hb[offF0], hb[ZB * 64 + offF0], hb[offF2], hb[ZB * 64 + offF2]};
+      const int b0 = (8 * ks + tg) * 8 + g, b1 = b0 + 32;
+      mma_split_a_2acc(ah, al, a, scr.bh[b0], scr.bh[b1], scr.bl[b0], scr.bl[b1]);
     }
 #pragma unroll
     for (int hf = 0; hf < 2; ++hf) {
@@ -691,16 +674,14 @@ __device__ __forceinline__ bool consume_item(const PipeProb& q, const unsigned c
   cons_sync();
   // ---- D: Kx[t][r] = sum_z W[t][z] x_new[z][r] / s; each warp two 16-row t tiles at a time ----
   {
-    unsigned xb[KZM][4];  // B fragments (hi0, hi1, lo0, lo1) of every K step, shared by the tiles
+    unsigned xb[KZ][4];  // B fragments (hi0, hi1, lo0, lo1) of every K step, shared by the tiles
 #pragma unroll
-    for (int ks = 0; ks < KZM; ++ks) {
-      if (ks < KZ) {
-        const int b0 = (8 * ks + tg) * 8 + g;
-        xb[ks][0] = scr.xh[b0];
-        xb[ks][1] = scr.xh[b0 + 32];
-        xb[ks][2] = scr.xl[b0];
-        xb[ks][3] = scr.xl[b0 + 32];
-      }
+    for (int ks = 0; ks < KZ; ++ks) {
+      const int b0 = (8 * ks + tg) * 8 + g;
+      xb[ks][0] = scr.xh[b0];
+      xb[ks][1] = scr.xh[b0 + 32];
+      xb[ks][2] = scr.xl[b0];
+      xb[ks][3] = scr.xl[b0 + 32];
     }
     float2* dst = mem_tg >= 0 ? q.kx_hat + (size_t)mem_tg * q.ldt : nullptr;
     for (int mt = warp; mt < mtt; mt += 2 * PIPE_CONS_WARPS) {
@@ -710,16 +691,14 @@ __device__ __forceinline__ bool consume_item(const PipeProb& q, const unsigned c
       const float* w0 = W + 2 * mt * ZB * 64;  // block (t / 8 = 2 mt, z / 8 = 0)
       const float* w1 = W + 2 * mt2 * ZB * 64;
 #pragma unroll
-      for (int ks = 0; ks < KZM; ++ks) {
-        if (ks < KZ) {
-          const float a0[4] = {w0[ks * 64 + offF0], w0[(ZB + ks) * 64 + offF0], w0[ks * 64 + offF2],
-                               w0[(ZB + ks) * 64 + offF2]};
-          mma_split_a_2acc(dh[0], dlo[0], a0, xb[ks][0], xb[ks][1], xb[ks][2], xb[ks][3]);
-          if (two) {
-            const float a1[4] = {w1[ks * 64 + offF0], w1[(ZB + ks) * 64 + offF0], w1[ks * 64 + offF2],
-                                 w1[(ZB + ks) * 64 + offF2]};
-            mma_split_a_2acc(dh[1], dlo[1], a1, xb[ks][0], xb[ks][1], xb[ks][2], xb[ks][3]);
-          }
+      for (int ks = 0; ks < KZ; ++ks) {
+        const float a0[4] = {w0[ks * 64 + offF0], w0[(ZB + ks) * 64 + offF0], w0[ks * 64 + offF2],
+                             w0[(ZB + ks) * 64 + offF2]};
+        mma_split_a_2acc(dh[0], dlo[0], a0, xb[ks][0], xb[ks][1], xb[ks][2], xb[ks][3]);
+        if (two) {
+          const float a1[4] = {w1[ks * 64 + offF0], w1[(ZB + ks) * 64 + offF0], w1[ks * 64 + offF2],
+                               w1[(ZB + ks) * 64 + offF2]};
+          mma_split_a_2acc(dh[1], dlo[1], a1, xb[ks][0], xb[ks][1], xb[ks][2], xb[ks][3]);
         }
       }
       if (dst) {
@@ -826,86 +805,6 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) k_contract_admm_pipe(PipeProb
   }
 }
 
-// Many problems, one persistent launch: the producer of each CTA takes items
-// (problem, class) from a device work queue (an atomic counter, QCHUNK items
-// per grab; problems in the queue in the caller's order, largest class blocks
-// first), so that CTAs done with one problem's classes go on with the next.
-// Stages are sized for the largest problem plus a 32-byte tail whose first
-// word names the item's problem + 1 (0: the queue is empty, the consumers stop).
-constexpr int QCHUNK = 8;
-
-__global__ void __launch_bounds__(PIPE_THREADS, 1) k_contract_admm_queue(const PipeProb* __restrict__ probs, int nprob,
-                                                                         int total, int* queue, int stage_bytes,
-                                                                         int S, int o_scr, int zm_max,
-                                                                         int* status_flag, long long max_polls) {
-  extern __shared__ __align__(128) float4 sm_pipe[];
-  unsigned char* sm = reinterpret_cast<unsigned char*>(sm_pipe);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // layout: S stages | consumer scratch | problem table | barriers
-  const int o_part = o_scr, o_bh = o_part + PIPE_CONS_WARPS * zm_max * 32, o_bl = o_bh + zm_max * 32,
-            o_xh = o_bl + zm_max * 32, o_xl = o_xh + zm_max * 32, o_tab = o_xl + zm_max * 32;
-  PipeProb* tab = reinterpret_cast<PipeProb*>(sm + o_tab);
-  const int o_bar = o_tab + ((nprob * (int)sizeof(PipeProb) + 15) & ~15);
-  uint64_t* full = reinterpret_cast<uint64_t*>(sm + o_bar);
-  uint64_t* empty = full + S;
-  volatile int* s_abort = reinterpret_cast<volatile int*>(empty + S);
-  for (int i = threadIdx.x; i < nprob * (int)sizeof(PipeProb) / 4; i += PIPE_THREADS)
-    reinterpret_cast<int*>(tab)[i] = reinterpret_cast<const int*>(probs)[i];
-  pipe_setup(sm, o_tab, full, empty, S, s_abort);
-  if (warp == PIPE_CONS_WARPS) {
-    if (lane != 0) return;
-    int issued = 0, cur = 0, end = 0, pi = 0;
-    for (;;) {
-      if (cur >= end) {
-        cur = atomicAdd(queue, QCHUNK);
-        end = min(cur + QCHUNK, total);
-      }
-      const bool more = cur < total;
-      const int s = issued % S;
-      if (!wait_free(empty + s, ((issued / S) & 1) ^ 1, max_polls, s_abort, status_flag)) break;
-      unsigned char* st = sm + s * stage_bytes;
-      int* slot = reinterpret_cast<int*>(st + stage_bytes - 16);  // the item's problem + 1, 0 = queue empty
-      if (!more) {
-        *slot = 0;
-        mbar_arrive(full + s);
-        ++issued;
-        break;
-      }
-      while (pi + 1 < nprob && tab[pi + 1].item0 <= cur) ++pi;  // items come in increasing order
-      *slot = pi + 1;
-      produce_item(tab[pi], cur - tab[pi].item0, st, full + s);
-      ++cur;
-      ++issued;
-    }
-    drain_fills(full, S, issued);
-    return;
-  }
-  const PipeScratch scr{reinterpret_cast<float*>(sm + o_part), reinterpret_cast<unsigned*>(sm + o_bh),
-                        reinterpret_cast<unsigned*>(sm + o_bl), reinterpret_cast<unsigned*>(sm + o_xh),
-                        reinterpret_cast<unsigned*>(sm + o_xl)};
-  for (int k = 0;; ++k) {
-    const int s = k % S;
-    int gave_up = 0;
-    if (!mbar_wait_bounded(full + s, (uint32_t)((k / S) & 1), max_polls)) {
-      gave_up = 1;
-      atomicExch(status_flag, 1);
-    }
-    const unsigned char* st = sm + s * stage_bytes;
-    const int pi = *reinterpret_cast<const int*>(st + stage_bytes - 16) - 1;
-    if (cons_sync_or(gave_up)) {
-      if (threadIdx.x == 0) *s_abort = 1;
-      break;
-    }
-    if (pi < 0) break;
-    if (consume_item<0>(tab[pi], st, scr, 0)) {
-      if (threadIdx.x == 0) *s_abort = 1;
-      break;
-    }
-    __syncwarp();
-    if (lane == 0) mbar_arrive(empty + s);
-  }
-}
-
 template <int KZ>
 ctof_status launch_pipe(const ctof_kernel_s* k, const PipePlan& P, int grid, const float2* c_hat, const float2* s_hat,
                         float2* x_hat, float2* kx_hat, float inv_scale, cudaStream_t st) {
@@ -925,7 +824,6 @@ ctof_status launch_pipe(const ctof_kernel_s* k, const PipePlan& P, int grid, con
   q.ldt = k->ldt;
   q.ldz = k->ldz;
   q.inv_s = inv_scale;
-  q.item0 = 0;
   k_contract_admm_pipe<KZ><<<grid, PIPE_THREADS, P.total, st>>>(q, k->d_flags, k->max_polls);
   CTOF_CUDA_TRY(cudaGetLastError());
   return CTOF_OK;
@@ -993,125 +891,4 @@ ctof_status contract_admm(const ctof_kernel_s* k, const float2* c_hat, const flo
                                                 k->ldt, s_hat, x_hat, k->ldz, kx_hat, inv_scale);
   CTOF_CUDA_TRY(cudaGetLastError());
   return CTOF_OK;
-}
-
-// ---- many problems in one persistent launch --------------------------------
-
-namespace {
-
-struct QueueLayout {
-  int stage_bytes, stages, o_scr, zm_max, smem;
-};
-
-QueueLayout queue_layout(int max_layout, int zm_max, int nprob, int stages) {
-  QueueLayout L;
-  L.stage_bytes = rup(max_layout + 32, 128);
-  L.stages = stages;
-  L.zm_max = zm_max;
-  L.o_scr = stages * L.stage_bytes;
-  const int scratch = PIPE_CONS_WARPS * zm_max * 32 + 4 * zm_max * 32;
-  const int table = (nprob * (int)sizeof(PipeProb) + 15) & ~15;
-  L.smem = L.o_scr + scratch + table + 2 * stages * 8 + 16;
-  return L;
-}
-
-// The device work-queue counter sits after the problem table.
-size_t queue_counter_offset(int nprob) { return ((size_t)nprob * sizeof(PipeProb) + 255) & ~(size_t)255; }
-
-}  // namespace
-
-ctof_status admm_queue_build(int count, ctof_kernel_s* const* ks, AdmmQueue* out) {
-  admm_queue_free(out);
-  struct Cand {
-    int idx, layout, zm;
-  };
-  std::vector<Cand> cand;
-  for (int i = 0; i < count; ++i) {
-    const ctof_kernel_s* k = ks[i];
-    if (!k->d_what_admm || !pipe_stages(k->nt, k->nz)) continue;
-    const PipePlan P = make_pipe_plan(k->nt, k->nz, 2);
-    cand.push_back({i, P.stage_bytes, P.zm});
-  }
-  // the largest set, taken from the smallest class blocks up, whose two stages fit
-  std::sort(cand.begin(), cand.end(), [](const Cand& a, const Cand& b) { return a.layout < b.layout; });
-  int take = 0, max_layout = 0, zm_max = 16;
-  for (int j = 0; j < (int)cand.size(); ++j) {
-    const int ml = std::max(max_layout, cand[j].layout), zm = std::max(zm_max, cand[j].zm);
-    if (queue_layout(ml, zm, j + 1, 2).smem > PIPE_SMEM_LIMIT) break;
-    max_layout = ml;
-    zm_max = zm;
-    take = j + 1;
-  }
-  if (take < 2) return CTOF_OK;  // nothing to gain: every problem keeps its own launch
-  cand.resize(take);
-  // queue order: largest class blocks first, so that small ones fill in at the end
-  std::sort(cand.begin(), cand.end(), [](const Cand& a, const Cand& b) { return a.layout > b.layout; });
-  int stages = 2;
-  while (stages < 4 && queue_layout(max_layout, zm_max, take, stages + 1).smem <= PIPE_SMEM_LIMIT) ++stages;
-  const QueueLayout L = queue_layout(max_layout, zm_max, take, stages);
-  std::vector<PipeProb> tab(take);
-  int items = 0;
-  for (int j = 0; j < take; ++j) {
-    const ctof_kernel_s* k = ks[cand[j].idx];
-    PipeProb& q = tab[j];
-    q.P = make_pipe_plan(k->nt, k->nz, 2);
-    q.what_o = k->d_what_admm;
-    q.hinv_o = k->d_hinv_admm;
-    q.lap = k->d_lap;
-    q.members = k->d_members;
-    q.nclass = k->nclass;
-    q.c_hat = k->d_spec_t2;
-    q.s_hat = k->d_spec_z;
-    q.x_hat = k->d_spec_z2;
-    q.kx_hat = k->d_spec_t;
-    q.ldt = k->ldt;
-    q.ldz = k->ldz;
-    q.inv_s = (float)(1.0 / k->scale);
-    q.item0 = items;
-    items += k->nclass;
-  }
-  void* d = nullptr;
-  const size_t tbytes = (size_t)take * sizeof(PipeProb);
-  if (cudaMalloc(&d, queue_counter_offset(take) + 256) != cudaSuccess) {
-    cudaGetLastError();
-    return CTOF_ENOMEM;
-  }
-  out->d_mem = d;
-  if (cudaMemcpy(d, tab.data(), tbytes, cudaMemcpyHostToDevice) != cudaSuccess) {
-    admm_queue_free(out);
-    return CTOF_ECUDA;
-  }
-  for (int j = 0; j < take; ++j) out->members.push_back(cand[j].idx);
-  out->nprob = take;
-  out->total = items;
-  out->stage_bytes = L.stage_bytes;
-  out->stages = L.stages;
-  out->o_scr = L.o_scr;
-  out->zm_max = L.zm_max;
-  out->smem = L.smem;
-  out->flag = ks[cand[0].idx]->d_flags;
-  out->max_polls = ks[cand[0].idx]->max_polls;
-  out->nsm = 152;
-  cudaDeviceGetAttribute(&out->nsm, cudaDevAttrMultiProcessorCount, ks[cand[0].idx]->device);
-  return CTOF_OK;
-}
-
-ctof_status admm_queue_launch(const AdmmQueue& q, cudaStream_t st) {
-  if (q.nprob == 0) return CTOF_OK;
-  const PipeProb* tab = static_cast<const PipeProb*>(q.d_mem);
-  int* ctr = reinterpret_cast<int*>(static_cast<char*>(q.d_mem) + queue_counter_offset(q.nprob));
-  CTOF_CUDA_TRY(cudaMemsetAsync(ctr, 0, sizeof(int), st));
-  CTOF_CUDA_TRY(cudaFuncSetAttribute(k_contract_admm_queue, cudaFuncAttributeMaxDynamicSharedMemorySize, q.smem));
-  k_contract_admm_queue<<<q.nsm, PIPE_THREADS, q.smem, st>>>(tab, q.nprob, q.total, ctr, q.stage_bytes, q.stages,
-                                                            q.o_scr, q.zm_max, q.flag, q.max_polls);
-  CTOF_CUDA_TRY(cudaGetLastError());
-  return CTOF_OK;
-}
-
-void admm_queue_free(AdmmQueue* q) {
-  if (q->d_mem) cudaFree(q->d_mem);
-  q->d_mem = nullptr;
-  q->nprob = 0;
-  q->total = 0;
-  q->members.clear();
 }

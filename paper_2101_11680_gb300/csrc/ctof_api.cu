@@ -7,8 +7,6 @@
 #include <string.h>
 
 #include <algorithm>
-#include <atomic>
-#include <mutex>
 #include <new>
 #include <vector>
 
@@ -340,7 +338,9 @@ ctof_status autotune(ctof_kernel_s* k, cudaStream_t st) {
   return s;
 }
 
-ctof_status admm_run(ctof_kernel_s* k, const ctof_solver_params* prm, cudaStream_t st) {
+// The handle's ADMM graph for these parameters (captured on first use; `st`
+// only serves the autotuner).
+ctof_status admm_graph(ctof_kernel_s* k, const ctof_solver_params* prm, cudaStream_t st) {
   CTOF_TRY(autotune(k, st));
   const bool same = k->graph && k->graph_iters == prm->iters && k->graph_rho == prm->rho &&
                     k->graph_beta == prm->tv_beta && k->graph_beta_rel == prm->beta_rel &&
@@ -389,6 +389,11 @@ ctof_status admm_run(ctof_kernel_s* k, const ctof_solver_params* prm, cudaStream
     k->graph_beta = prm->tv_beta;
     k->graph_beta_rel = prm->beta_rel;
   }
+  return CTOF_OK;
+}
+
+ctof_status admm_run(ctof_kernel_s* k, const ctof_solver_params* prm, cudaStream_t st) {
+  CTOF_TRY(admm_graph(k, prm, st));
   CTOF_CUDA_TRY(cudaGraphLaunch(k->graph, st));
   return CTOF_OK;
 }
@@ -538,162 +543,35 @@ ctof_status fill_report(ctof_kernel_s* k, const ctof_solver_params* prm, double 
   return bad ? CTOF_ENONFINITE : CTOF_OK;
 }
 
-// One graph per distinct batch (handles, buffers, parameters): every problem's
-// ADMM chain is captured on its own forked stream so that the problems run
-// concurrently on the GPU; the graph is replayed while the batch repeats.
-struct BatchGraph {
-  std::vector<unsigned long long> uids;
-  std::vector<const void*> ptrs;
-  int iters = 0;
-  double rho = 0, beta = 0, beta_rel = 0;
-  cudaGraphExec_t exec = nullptr;
-  AdmmQueue queue;  // the batched x-update's problem table and work-queue counter
-};
-std::mutex g_batch_mutex;
-BatchGraph g_batch;
-std::vector<cudaStream_t> g_side_streams;
-std::vector<cudaEvent_t> g_side_events;
-
-ctof_status batch_graph_run(int count, const ctof_kernel* ks, const float* const* d_m,
-                            const ctof_solver_params* prm, float* const* d_mu, cudaStream_t st) {
-  std::lock_guard<std::mutex> lock(g_batch_mutex);
-  std::vector<unsigned long long> uids(count);
-  std::vector<const void*> ptrs(2 * count);
+// ADMM on `count` handles at once: every problem runs its own graph (kept with
+// its handle, independent of the callers' buffers, and shared with
+// ctof_reconstruct) on a stream of its own that starts where `st` is; `st`
+// goes on when all are done.
+ctof_status batch_run(int count, const ctof_kernel* ks, const float* const* d_m, const ctof_solver_params* prm,
+                      float* const* d_mu, cudaStream_t st) {
   for (int i = 0; i < count; ++i) {
-    uids[i] = ks[i]->uid;
-    ptrs[2 * i] = d_m[i];
-    ptrs[2 * i + 1] = d_mu[i];
+    ctof_kernel_s* o = ctof_ops(ks[i]);
+    if (!o->batch_stream) CTOF_CUDA_TRY(cudaStreamCreateWithFlags(&o->batch_stream, cudaStreamNonBlocking));
+    if (!o->batch_event) CTOF_CUDA_TRY(cudaEventCreateWithFlags(&o->batch_event, cudaEventDisableTiming));
+    CTOF_TRY(admm_graph(o, prm, st));  // made (and autotuned) before anything of this batch runs
   }
-  const bool same = g_batch.exec && g_batch.uids == uids && g_batch.ptrs == ptrs && g_batch.iters == prm->iters &&
-                    g_batch.rho == prm->rho && g_batch.beta == prm->tv_beta && g_batch.beta_rel == prm->beta_rel;
-  if (!same) {
-    if (g_batch.exec) {
-      cudaGraphExecDestroy(g_batch.exec);
-      g_batch.exec = nullptr;
-    }
-    const int nside = count < 32 ? count : 32;
-    while ((int)g_side_streams.size() < nside) {
-      cudaStream_t s2 = nullptr;
-      CTOF_CUDA_TRY(cudaStreamCreateWithFlags(&s2, cudaStreamNonBlocking));
-      g_side_streams.push_back(s2);
-    }
-    while ((int)g_side_events.size() < nside + 1) {
-      cudaEvent_t e = nullptr;
-      CTOF_CUDA_TRY(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-      g_side_events.push_back(e);
-    }
-    // problems whose x-update runs in the one persistent queue launch per iteration
-    std::vector<ctof_kernel_s*> os(count);  // the operators ADMM runs on
-    for (int i = 0; i < count; ++i) os[i] = ctof_ops(ks[i]);
-    CTOF_TRY(admm_queue_build(count, os.data(), &g_batch.queue));
-    std::vector<char> queued(count, 0);
-    for (int i : g_batch.queue.members) queued[i] = 1;
-    cudaStream_t cap = nullptr;
-    CTOF_CUDA_TRY(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
-    cudaGraph_t graph = nullptr;
-    cudaError_t e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeRelaxed);
-    ctof_status s = e == cudaSuccess ? CTOF_OK : CTOF_ECUDA;
-    // fork the side streams off `cap`, or join them back into it
-    auto fork = [&]() {
-      if (s == CTOF_OK && cudaEventRecord(g_side_events[nside], cap) != cudaSuccess) s = CTOF_ECUDA;
-      for (int j = 0; j < nside && s == CTOF_OK; ++j)
-        if (cudaStreamWaitEvent(g_side_streams[j], g_side_events[nside], 0) != cudaSuccess) s = CTOF_ECUDA;
-    };
-    auto join = [&]() {
-      for (int j = 0; j < nside && s == CTOF_OK; ++j) {
-        if (cudaEventRecord(g_side_events[j], g_side_streams[j]) != cudaSuccess ||
-            cudaStreamWaitEvent(cap, g_side_events[j], 0) != cudaSuccess)
-          s = CTOF_ECUDA;
-      }
-    };
-    // side streams: the problems with their own x-update launch get streams of
-    // their own (they run beside the queue launch), the queued ones share the rest
-    std::vector<int> stream_of(count);
-    {
-      int nown = 0;
-      for (int i = 0; i < count; ++i) nown += !queued[i];
-      const int own_streams = nown < nside / 2 ? nown : nside / 2;
-      int a = 0, b = 0;
-      for (int i = 0; i < count; ++i) {
-        if (!queued[i] && own_streams > 0)
-          stream_of[i] = (a++) % own_streams;
-        else
-          stream_of[i] = own_streams + (b++) % (nside - own_streams > 0 ? nside - own_streams : 1);
-        if (stream_of[i] >= nside) stream_of[i] = nside - 1;
-      }
-    }
-    fork();
-    for (int i = 0; i < count && s == CTOF_OK; ++i) {
-      cudaStream_t side = g_side_streams[stream_of[i]];
-      s = stage_measurement(os[i], d_m[i], os[i]->d_mstage, side);
-      if (s == CTOF_OK) s = admm_setup(os[i], prm, side);
-    }
-    join();
-    // iterations in lockstep: the problems with their own x-update run it and their
-    // T / Z sides from the iteration's start; beside them the queued x-updates of
-    // all other problems run as one launch, after which their T / Z sides follow
-    cudaEvent_t ev_q = g_side_events[nside];
-    for (int it = 0; it < prm->iters && s == CTOF_OK; ++it) {
-      fork();
-      for (int i = 0; i < count && s == CTOF_OK; ++i) {
-        if (queued[i]) continue;
-        cudaStream_t side = g_side_streams[stream_of[i]];
-        s = admm_contract(os[i], side);
-        if (s == CTOF_OK) s = admm_side(os[i], prm, it, side, nullptr);
-      }
-      if (s == CTOF_OK) s = admm_queue_launch(g_batch.queue, cap);
-      if (s == CTOF_OK && cudaEventRecord(ev_q, cap) != cudaSuccess) s = CTOF_ECUDA;
-      for (int i = 0; i < count && s == CTOF_OK; ++i) {
-        if (!queued[i]) continue;
-        cudaStream_t side = g_side_streams[stream_of[i]];
-        if (cudaStreamWaitEvent(side, ev_q, 0) != cudaSuccess) s = CTOF_ECUDA;
-        if (s == CTOF_OK) s = admm_side(os[i], prm, it, side, nullptr);
-      }
-      join();
-    }
-    fork();
-    for (int i = 0; i < count && s == CTOF_OK; ++i) {
-      ctof_kernel_s* k = ks[i];
-      const size_t vb = (size_t)k->nz * k->n * k->n * sizeof(float);
-      if (cudaMemcpyAsync(d_mu[i], k->d_vstage, vb, cudaMemcpyDeviceToDevice, g_side_streams[stream_of[i]]) !=
-          cudaSuccess)
-        s = CTOF_ECUDA;
-    }
-    join();
-    e = cudaStreamEndCapture(cap, &graph);
-    cudaStreamDestroy(cap);
-    if (s == CTOF_OK && e != cudaSuccess) s = CTOF_ECUDA;
-    if (s == CTOF_OK && cudaGraphInstantiate(&g_batch.exec, graph, 0) != cudaSuccess) {
-      g_batch.exec = nullptr;
+  cudaEvent_t start = ctof_ops(ks[0])->batch_event;
+  CTOF_CUDA_TRY(cudaEventRecord(start, st));
+  for (int i = 0; i < count; ++i) CTOF_CUDA_TRY(cudaStreamWaitEvent(ctof_ops(ks[i])->batch_stream, start, 0));
+  ctof_status s = CTOF_OK;
+  for (int i = 0; i < count; ++i) {
+    ctof_kernel_s* o = ctof_ops(ks[i]);
+    cudaStream_t side = o->batch_stream;
+    if (s == CTOF_OK) s = stage_measurement(o, d_m[i], o->d_mstage, side);
+    if (s == CTOF_OK && cudaGraphLaunch(o->graph, side) != cudaSuccess) s = CTOF_ECUDA;
+    const size_t vb = (size_t)o->nz * o->n * o->n * sizeof(float);
+    if (s == CTOF_OK && cudaMemcpyAsync(d_mu[i], o->d_vstage, vb, cudaMemcpyDeviceToDevice, side) != cudaSuccess)
       s = CTOF_ECUDA;
-    }
-    if (graph) cudaGraphDestroy(graph);
-    if (s != CTOF_OK) {
-      cudaGetLastError();
-      return s;
-    }
-    g_batch.uids = uids;
-    g_batch.ptrs = ptrs;
-    g_batch.iters = prm->iters;
-    g_batch.rho = prm->rho;
-    g_batch.beta = prm->tv_beta;
-    g_batch.beta_rel = prm->beta_rel;
-    // the handles' own single-problem graphs stay valid: they stage through the
-    // same buffers and are not affected by this graph
+    // `st` waits for what was enqueued, also after an error
+    if (cudaEventRecord(o->batch_event, side) != cudaSuccess || cudaStreamWaitEvent(st, o->batch_event, 0) != cudaSuccess)
+      s = CTOF_ECUDA;
   }
-  CTOF_CUDA_TRY(cudaGraphLaunch(g_batch.exec, st));
-  return CTOF_OK;
-}
-
-void batch_graph_forget(const ctof_kernel_s* k) {
-  std::lock_guard<std::mutex> lock(g_batch_mutex);
-  for (unsigned long long u : g_batch.uids)
-    if (u == k->uid && g_batch.exec) {
-      cudaGraphExecDestroy(g_batch.exec);
-      g_batch.exec = nullptr;
-      g_batch.uids.clear();
-      break;
-    }
+  return s;
 }
 
 }  // namespace
@@ -718,10 +596,11 @@ const char* ctof_last_error_message(void) { return g_last_error; }
 void ctof_kernel_destroy(ctof_kernel k) {
   if (!k) return;
   DeviceGuard guard(k->device);
-  batch_graph_forget(k);
   for (ctof_kernel_s* o : {k->tz, k}) {  // what either operator made on first use
     if (!o) continue;
     if (o->graph) cudaGraphExecDestroy(o->graph);
+    if (o->batch_stream) cudaStreamDestroy(o->batch_stream);
+    if (o->batch_event) cudaEventDestroy(o->batch_event);
     destroy_events(o);
     if (o->d_bt_cinv) cudaFree(o->d_bt_cinv);
     if (o->d_batch) cudaFree(o->d_batch);
@@ -809,10 +688,6 @@ ctof_status build_any(const ctof_optics* optics, const ctof_emission* emission, 
   k->tik_last = 1;
   k->max_polls = CTOF_DEFAULT_MAX_POLLS;
   for (int i = 0; i < 4; ++i) k->tune_pb[i] = 16;
-  {
-    static std::atomic<unsigned long long> next_id{1};
-    k->uid = next_id++;
-  }
 
   std::vector<int> members;
   std::vector<float> lap;
@@ -1156,8 +1031,7 @@ ctof_status ctof_reconstruct_batch(int count, const ctof_kernel* ks, const float
   DeviceGuard g(ks[0]->device);
   if (!g.ok) return CTOF_ECUDA;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  for (int i = 0; i < count; ++i) CTOF_TRY(autotune(ctof_ops(ks[i]), st));
-  return batch_graph_run(count, ks, d_m, params, d_mu, st);
+  return batch_run(count, ks, d_m, params, d_mu, st);
 }
 
 ctof_status ctof_set_wait_limit(ctof_kernel k, long long polls) {

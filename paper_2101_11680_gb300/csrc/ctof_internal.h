@@ -6,8 +6,6 @@
 #include <cuda_runtime.h>
 #include <stddef.h>
 
-#include <vector>
-
 #include "common.cuh"
 
 // Device workspaces are carved from one allocation per handle.
@@ -105,7 +103,8 @@ struct ctof_kernel_s {
   // autotuned column-pass plane tiles: [T fwd, T inv, Z fwd, Z inv]
   int tune_pb[4];
   int tuned;
-  unsigned long long uid;  // unique per handle (batch graph cache key)
+  cudaStream_t batch_stream;  // ctof_reconstruct_batch: this problem's stream and its start / end
+  cudaEvent_t batch_event;
 
   // Time compression (time_basis.cu): `tz` is this handle's operator on r < nt
   // planes (V = Q^T W_hat in place of W_hat; null where it does not pay).  It
@@ -251,22 +250,6 @@ size_t contract_admm_pipe_floats(int nt, int nz, int which);
 int contract_admm_pipe_stages(int nt, int nz);
 // Fill the pipelined kernel's copies from d_what / d_hinv (after the build).
 ctof_status contract_admm_prepare(ctof_kernel_s* k, cudaStream_t st);
-
-// Batched x-update: the problems of a batch whose class blocks fit two shared
-// stages of the largest among them, in one persistent launch fed by a device
-// work queue.  `members` lists their indices in the batch (queue order); the
-// other problems keep their own contract_admm launch.  Timeouts are reported
-// on the first queued problem's handle.
-struct AdmmQueue {
-  int nprob = 0, total = 0, stage_bytes = 0, stages = 0, o_scr = 0, zm_max = 0, smem = 0, nsm = 152;
-  void* d_mem = nullptr;  // problem table, then the queue counter
-  int* flag = nullptr;
-  long long max_polls = 0;
-  std::vector<int> members;
-};
-ctof_status admm_queue_build(int count, ctof_kernel_s* const* ks, AdmmQueue* out);
-ctof_status admm_queue_launch(const AdmmQueue& q, cudaStream_t st);
-void admm_queue_free(AdmmQueue* q);
 
 // ---- contract_warp.cu -----------------------------------------------------
 // One warp per frequency class, for class blocks of which several fit in
