@@ -34,6 +34,8 @@ __global__ void __launch_bounds__(TX* TY) k_tv_stencil(const float* __restrict__
                                                        float* __restrict__ s_out, const double* __restrict__ beta,
                                                        float inv_rho, int P, int nz, int n,
                                                        float* __restrict__ out_crop) {
+  pdl_trigger();
+  pdl_wait();
   __shared__ float sX[ZP][TY + 2][TX + 2];
   __shared__ float sW2x[ZP][TY][TX + 1];
   __shared__ float sW2y[ZP][TY + 1][TX];
@@ -139,6 +141,8 @@ __global__ void __launch_bounds__(TX* TY) k_tv_stencil(const float* __restrict__
 }
 
 __global__ void k_max_abs(const float* __restrict__ v, size_t count, unsigned int* __restrict__ out) {
+  pdl_trigger();
+  pdl_wait();
   float mx = 0.f;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < count; i += (size_t)gridDim.x * blockDim.x)
     mx = fmaxf(mx, fabsf(v[i]));
@@ -147,6 +151,8 @@ __global__ void k_max_abs(const float* __restrict__ v, size_t count, unsigned in
 }
 
 __global__ void k_set_beta(double* scalars, double beta_fixed, double beta_rel, double inv_s2) {
+  pdl_trigger();
+  pdl_wait();
   if (threadIdx.x == 0) {
     const unsigned int bits = reinterpret_cast<const unsigned int*>(scalars + 1)[0];
     const double mx = (double)__uint_as_float(bits);
@@ -167,6 +173,8 @@ __global__ void k_check_finite(const float* __restrict__ v, size_t count, int* _
 // holding the DC frequency (f = 0), lam0 = scalars[0].  One block.
 __global__ void k_fista_lambda(const double* __restrict__ scalars, const double* __restrict__ gram,
                                const int* __restrict__ members, int nclass, int nz, float* __restrict__ lam) {
+  pdl_trigger();
+  pdl_wait();
   __shared__ int s_c;
   __shared__ double s_max;
   if (threadIdx.x == 0) s_c = -1;
@@ -190,6 +198,8 @@ __global__ void k_fista_lambda(const double* __restrict__ scalars, const double*
 
 // r -= m
 __global__ void k_sub_meas(float* __restrict__ r, const float* __restrict__ m, size_t count) {
+  pdl_trigger();
+  pdl_wait();
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < count; i += (size_t)gridDim.x * blockDim.x)
     r[i] -= m[i];
 }
@@ -198,6 +208,8 @@ __global__ void k_sub_meas(float* __restrict__ r, const float* __restrict__ m, s
 //   x_k = soft(y - g / s^2, lam[z]);  y <- x_k + beta (x_k - x_{k-1});  x <- x_k
 __global__ void k_fista_step(float* __restrict__ y, const float* __restrict__ g, float* __restrict__ x,
                              const float* __restrict__ lam, float beta, float inv_s2, int plane, size_t count) {
+  pdl_trigger();
+  pdl_wait();
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < count; i += (size_t)gridDim.x * blockDim.x) {
     const float v = y[i] - inv_s2 * g[i];
     const float xn = soft(v, lam[i / plane]);
@@ -215,6 +227,8 @@ __global__ void k_fista_step(float* __restrict__ y, const float* __restrict__ g,
 // butterflies (a + b, a - b) run over strides 1..16 across lanes and 32 in
 // registers, which is H_64 in its natural (Sylvester) order.
 __global__ void k_block_hadamard(float* __restrict__ v, int planes, int n) {
+  pdl_trigger();
+  pdl_wait();
   const int warp = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
   const int nb = n >> 3;
   const long long nblk = (long long)planes * nb * nb;
@@ -251,7 +265,7 @@ ctof_status admm_tv_stencil(const ctof_kernel_s* k, const float* x, const float*
                             float* s, const double* beta_dev, float rho, float* out_crop, cudaStream_t st) {
   dim3 block(TX, TY);
   dim3 grid(k->p / TX, k->p / TY, ctof_div_up(k->nz, ZP));
-  k_tv_stencil<<<grid, block, 0, st>>>(x, u2_old, u2_new, u3, s, beta_dev, 1.0f / rho, k->p, k->nz, k->n, out_crop);
+  CTOF_CUDA_TRY(ctof_launch(k_tv_stencil, grid, block, 0, st, x, u2_old, u2_new, u3, s, beta_dev, 1.0f / rho, k->p, k->nz, k->n, out_crop));
   CTOF_CUDA_TRY(cudaGetLastError());
   return CTOF_OK;
 }
@@ -262,13 +276,13 @@ ctof_status reduce_max_abs(const float* v, size_t count, double* out_dev, cudaSt
   int blocks = (int)((count + 255) / 256);
   if (blocks > 152 * 8) blocks = 152 * 8;
   if (blocks < 1) blocks = 1;
-  k_max_abs<<<blocks, 256, 0, st>>>(v, count, reinterpret_cast<unsigned int*>(out_dev));
+  CTOF_CUDA_TRY(ctof_launch(k_max_abs, blocks, 256, 0, st, v, count, reinterpret_cast<unsigned int*>(out_dev)));
   CTOF_CUDA_TRY(cudaGetLastError());
   return CTOF_OK;
 }
 
 ctof_status admm_set_beta(double* scalars, double beta_fixed, double beta_rel, double inv_scale2, cudaStream_t st) {
-  k_set_beta<<<1, 32, 0, st>>>(scalars, beta_fixed, beta_rel, inv_scale2);
+  CTOF_CUDA_TRY(ctof_launch(k_set_beta, 1, 32, 0, st, scalars, beta_fixed, beta_rel, inv_scale2));
   CTOF_CUDA_TRY(cudaGetLastError());
   return CTOF_OK;
 }
@@ -283,20 +297,20 @@ ctof_status check_finite(const float* v, size_t count, int* flag_dev, cudaStream
 }
 
 ctof_status fista_lambda(const ctof_kernel_s* k, const double* scalars, float* lam, cudaStream_t st) {
-  k_fista_lambda<<<1, 128, 0, st>>>(scalars, k->d_gram, k->d_members, k->nclass, k->nz, lam);
+  CTOF_CUDA_TRY(ctof_launch(k_fista_lambda, 1, 128, 0, st, scalars, k->d_gram, k->d_members, k->nclass, k->nz, lam));
   CTOF_CUDA_TRY(cudaGetLastError());
   return CTOF_OK;
 }
 
 ctof_status fista_sub_meas(float* r, const float* m, size_t count, cudaStream_t st) {
-  k_sub_meas<<<grid_elem(count), 256, 0, st>>>(r, m, count);
+  CTOF_CUDA_TRY(ctof_launch(k_sub_meas, grid_elem(count), 256, 0, st, r, m, count));
   CTOF_CUDA_TRY(cudaGetLastError());
   return CTOF_OK;
 }
 
 ctof_status fista_step(float* y, const float* g, float* x, const float* lam, float beta, float inv_s2, int plane,
                        size_t count, cudaStream_t st) {
-  k_fista_step<<<grid_elem(count), 256, 0, st>>>(y, g, x, lam, beta, inv_s2, plane, count);
+  CTOF_CUDA_TRY(ctof_launch(k_fista_step, grid_elem(count), 256, 0, st, y, g, x, lam, beta, inv_s2, plane, count));
   CTOF_CUDA_TRY(cudaGetLastError());
   return CTOF_OK;
 }
@@ -305,7 +319,7 @@ ctof_status block_hadamard(float* v, int planes, int n, cudaStream_t st) {
   if (n % 8 != 0) return CTOF_EUNSUPPORTED;
   const long long warps = (long long)planes * (n / 8) * (n / 8);
   const long long blocks = (warps * 32 + 255) / 256;
-  k_block_hadamard<<<(unsigned)blocks, 256, 0, st>>>(v, planes, n);
+  CTOF_CUDA_TRY(ctof_launch(k_block_hadamard, (unsigned)blocks, 256, 0, st, v, planes, n));
   CTOF_CUDA_TRY(cudaGetLastError());
   return CTOF_OK;
 }

@@ -209,6 +209,8 @@ __global__ void __launch_bounds__(CT_THREADS) k_contract(const float* __restrict
                                                          const float2* __restrict__ vin, int ld_in, size_t in_vstride,
                                                          float2* __restrict__ vout, int ld_out, size_t out_vstride,
                                                          int nvol, const float* __restrict__ hinv, int nbw, int nvs) {
+  pdl_trigger();
+  pdl_wait();
   extern __shared__ __align__(16) char smem[];
   __shared__ int s_mem[2][4];
   const Plan P = make_plan(MODE, nt, nz, nbw, nvs, blockDim.x);
@@ -412,8 +414,8 @@ ctof_status launch(const ctof_kernel_s* k, int nvol, const float2* vin, int ld_i
   if (per_sm > 4) per_sm = 4;
   int grid = 152 * per_sm;
   if (grid > k->nclass) grid = k->nclass;
-  k_contract<MODE><<<grid, CT_THREADS, p.total, st>>>(k->d_what, k->d_members, k->nclass, k->nt, k->nz, vin, ld_in,
-                                                      in_vstride, vout, ld_out, out_vstride, nvol, hinv, nbuf, nvs);
+  CTOF_CUDA_TRY(ctof_launch(k_contract<MODE>, grid, CT_THREADS, p.total, st, k->d_what, k->d_members, k->nclass, k->nt, k->nz, vin, ld_in,
+                                                      in_vstride, vout, ld_out, out_vstride, nvol, hinv, nbuf, nvs));
   CTOF_CUDA_TRY(cudaGetLastError());
   return CTOF_OK;
 }

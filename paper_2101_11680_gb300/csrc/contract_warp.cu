@@ -246,21 +246,25 @@ __device__ __forceinline__ void fwd_pass(const WarpPlan& P, const float* W, cons
   }
 }
 
-// One lane: class c (members f) into a slot, completing on `full`.
+// One lane: class c (members f) into a slot, completing on `full`: the header and
+// the class's tables first, then its vectors.
 template <int MODE>
-__device__ __forceinline__ void fill_slot(const WarpArgs& A, int c, int4 f4, float dl, unsigned char* st,
-                                          uint64_t* full) {
+__device__ __forceinline__ void fill_tables(const WarpArgs& A, int c, int4 f, float dl, unsigned char* st,
+                                            uint64_t* full) {
   const WarpPlan& P = A.P;
-  const int f[4] = {f4.x, f4.y, f4.z, f4.w};
-  unsigned bytes = P.w_bytes + P.h_bytes;
-#pragma unroll
-  for (int m = 0; m < 4; ++m)
-    if (f[m] >= 0) bytes += MODE == WM_FWD ? P.v_bytes : P.c_bytes + (MODE == WM_ADMM ? 2 * P.v_bytes : 0);
-  *reinterpret_cast<int4*>(st + P.o_hdr) = f4;
+  const int present = (f.x >= 0) + (f.y >= 0) + (f.z >= 0) + (f.w >= 0);
+  const unsigned per = MODE == WM_FWD ? P.v_bytes : P.c_bytes + (MODE == WM_ADMM ? 2 * P.v_bytes : 0);
+  *reinterpret_cast<int4*>(st + P.o_hdr) = f;
   if (MODE == WM_ADMM) *reinterpret_cast<float*>(st + P.o_hdr + 16) = dl;
-  bulk::arrive_expect(full, bytes);
+  bulk::arrive_expect(full, P.w_bytes + P.h_bytes + present * per);
   bulk::g2s(st, A.w + (size_t)c * (P.w_bytes >> 2), P.w_bytes, full);
   if (MODE >= WM_TIK) bulk::g2s(st + P.o_h, A.h + (size_t)c * (P.h_bytes >> 2), P.h_bytes, full);
+}
+
+template <int MODE>
+__device__ __forceinline__ void fill_vectors(const WarpArgs& A, int4 f4, unsigned char* st, uint64_t* full) {
+  const WarpPlan& P = A.P;
+  const int f[4] = {f4.x, f4.y, f4.z, f4.w};
 #pragma unroll
   for (int m = 0; m < 4; ++m) {
     if (f[m] < 0) continue;
@@ -547,6 +551,7 @@ template <int MODE, int ZB>
 __global__ void __launch_bounds__(MODE == WM_ADMM ? MAX_PAIRS * 64 : MAX_WARPS * 32, 1) k_contract_warp(const __grid_constant__ WarpArgs A,
                                                                      int* __restrict__ flag, long long max_polls) {
   extern __shared__ __align__(128) unsigned char wsm[];
+  pdl_trigger();
   const WarpPlan& P = A.P;
   // worker: the warp or pair of warps that takes every NW-th class; its first lane fills slots
   constexpr int WT = MODE == WM_ADMM ? 64 : 32;
@@ -562,27 +567,32 @@ __global__ void __launch_bounds__(MODE == WM_ADMM ? MAX_PAIRS * 64 : MAX_WARPS *
     issued[threadIdx.x] = 0;
   }
   __syncthreads();
-  auto fill = [&](int k, int4 f, float dl) {
-    const int s = k % NS;
-    fill_slot<MODE>(A, (int)blockIdx.x + k * (int)gridDim.x, f, dl, wsm + s * P.slot, full + s);
-    publish(issued + s, k / NS + 1);
+  auto cls = [&](int k) { return (int)blockIdx.x + k * (int)gridDim.x; };
+  auto header = [&](int k, int4& f, float& dl) {
+    f = __ldg(reinterpret_cast<const int4*>(A.members) + cls(k));
+    dl = MODE == WM_ADMM ? __ldg(A.lap + cls(k)) + 1.0f : 0.f;
   };
-  // the first ring: slot s by worker s mod NW
-  for (int k = worker; k < NS && k < mine; k += NW) {
-    if (first) {
-      const int c = (int)blockIdx.x + k * (int)gridDim.x;
-      fill(k, __ldg(reinterpret_cast<const int4*>(A.members) + c), MODE == WM_ADMM ? __ldg(A.lap + c) + 1.0f : 0.f);
+  // the first ring, slot s by worker s mod NW: the tables do not depend on earlier work in the stream
+  if (first) {
+    int4 f;
+    float dl;
+    for (int k = worker; k < NS && k < mine; k += NW) {
+      header(k, f, dl);
+      fill_tables<MODE>(A, cls(k), f, dl, wsm + k * P.slot, full + k);
+    }
+    pdl_wait();
+    for (int k = worker; k < NS && k < mine; k += NW) {
+      fill_vectors<MODE>(A, *reinterpret_cast<const int4*>(wsm + k * P.slot + P.o_hdr), wsm + k * P.slot, full + k);
+      publish(issued + k, 1);
     }
   }
+  __syncwarp();
+  pdl_wait();
   for (int k = worker; k < mine; k += NW) {
     const int s = k % NS, kn = k + NS;
     int4 fn = make_int4(-1, -1, -1, -1);
     float dn = 0.f;
-    if (first && kn < mine) {  // the refill's header, ahead of its use
-      const int c = (int)blockIdx.x + kn * (int)gridDim.x;
-      fn = __ldg(reinterpret_cast<const int4*>(A.members) + c);
-      if (MODE == WM_ADMM) dn = __ldg(A.lap + c) + 1.0f;
-    }
+    if (first && kn < mine) header(kn, fn, dn);  // the refill's, ahead of its use
     const bool late = !wait_fill(full + s, issued + s, k / NS + 1, max_polls);
     if (MODE == WM_ADMM ? pair_any(1 + worker, late) : __any_sync(0xffffffffu, late)) {
       if (first) atomicOr(flag, 1);
@@ -598,7 +608,11 @@ __global__ void __launch_bounds__(MODE == WM_ADMM ? MAX_PAIRS * 64 : MAX_WARPS *
       pair_sync(1 + worker);
     else
       __syncwarp();
-    if (first && kn < mine) fill(kn, fn, dn);
+    if (first && kn < mine) {
+      fill_tables<MODE>(A, cls(kn), fn, dn, wsm + s * P.slot, full + s);
+      fill_vectors<MODE>(A, fn, wsm + s * P.slot, full + s);
+      publish(issued + s, kn / NS + 1);
+    }
     __syncwarp();
   }
   __syncthreads();
@@ -646,7 +660,7 @@ ctof_status launch(const ctof_kernel_s* k, const WarpPlan& P, WarpArgs& A, cudaS
   int nsm = 152;
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, k->device);
   const int grid = k->nclass < nsm ? k->nclass : nsm;
-  kern<<<grid, P.nw * (MODE == WM_ADMM ? 64 : 32), P.total, st>>>(A, k->d_flags, k->max_polls);
+  CTOF_CUDA_TRY(ctof_launch(kern, grid, P.nw * (MODE == WM_ADMM ? 64 : 32), P.total, st, A, k->d_flags, k->max_polls));
   CTOF_CUDA_TRY(cudaGetLastError());
   return CTOF_OK;
 }

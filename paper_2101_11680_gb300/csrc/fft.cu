@@ -395,15 +395,18 @@ __device__ __forceinline__ float2* sh_buf(const RowSmem& S, int b) {
   return S.s_h + b * (sh_bytes(P) / (int)sizeof(float2));
 }
 
-// Block-wide prologue: barriers (one per s_h buffer) and twiddles.
+// Block-wide prologue: barriers (one per s_h buffer) and twiddles, then the
+// wait for the work before this kernel.
 template <int P>
 __device__ __forceinline__ void row_prologue(const RowSmem& S, const float2* tw) {
+  pdl_trigger();
   if (threadIdx.x == 0) {
     bulk::bar_init(S.bar, 1);
     bulk::bar_init(S.bar + 1, 1);
   }
   for (int i = threadIdx.x; i < tw_pad(P); i += blockDim.x) S.s_tw[i] = tw[i];
   __syncthreads();  // barriers initialised and twiddles staged before any use
+  pdl_wait();
 }
 
 // Block-wide wait for the copies into buffer (it & 1) of iteration `it`
@@ -735,10 +738,12 @@ template <int P, int PB>
 __device__ __forceinline__ void col_load_issue(uint64_t* bar, float2* tile, float2* s_tw, const float2* tw,
                                                const CUtensorMap* src, int pl0, int kx0, int kb, int nrb) {
   constexpr int RB = col_rb<P>();
+  pdl_trigger();
   bulk::bar_init(bar, 1);
   bulk::arrive_expect(bar, (unsigned)(kb * nrb * RB * PB) * (unsigned)sizeof(float2) +
                                tw_pad(P) * (unsigned)sizeof(float2));
   bulk::g2s(s_tw, tw, tw_pad(P) * sizeof(float2), bar);
+  pdl_wait();  // (only this thread touches global data, here and in col_store)
   for (int j = 0; j < kb; ++j)
     for (int rb = 0; rb < nrb; ++rb) bulk::tensor_g2s(tile + (j * P + rb * RB) * PB, src, pl0, kx0 + j, rb * RB, bar);
 }
@@ -945,8 +950,8 @@ ctof_status fft_rows_forward(const ctof_kernel_s* k, const float* in, int nplane
   const size_t sm = row_smem_bytes(k->p);
   CTOF_P_SWITCH(k->p, {
     CTOF_CUDA_TRY(allow_smem(k_rows_fwd<P_>, sm));
-    k_rows_fwd<P_><<<row_grid(rows, nplanes), ROW_WARPS * 32, sm, st>>>(map, in, nplanes, rows, cols_in, ld_in,
-                                                                         k->d_tw);
+    CTOF_CUDA_TRY(ctof_launch(k_rows_fwd<P_>, row_grid(rows, nplanes), ROW_WARPS * 32, sm, st, map, in, nplanes, rows,
+                              cols_in, ld_in, k->d_tw));
   });
   CTOF_CUDA_TRY(cudaGetLastError());
   return CTOF_OK;
@@ -961,8 +966,8 @@ ctof_status fft_rows_inverse(const ctof_kernel_s* k, const float2* inter, int np
   const float scale = 1.0f / ((float)k->p * (float)k->p);
   CTOF_P_SWITCH(k->p, {
     CTOF_CUDA_TRY(allow_smem(k_rows_inv<P_, false>, sm));
-    k_rows_inv<P_, false><<<row_grid(rows, nplanes), ROW_WARPS * 32, sm, st>>>(
-        map, nplanes, rows, cols_out, out, ld_out, scale, k->d_tw, k->d_flags, k->max_polls, nullptr);
+    CTOF_CUDA_TRY(ctof_launch(k_rows_inv<P_, false>, row_grid(rows, nplanes), ROW_WARPS * 32, sm, st, map, nplanes, rows,
+                              cols_out, out, ld_out, scale, k->d_tw, k->d_flags, k->max_polls, nullptr));
   });
   CTOF_CUDA_TRY(cudaGetLastError());
   return CTOF_OK;
@@ -977,9 +982,8 @@ ctof_status fft_rows_inverse_norm(const ctof_kernel_s* k, const float2* inter, i
   const float scale = 1.0f / ((float)k->p * (float)k->p);
   CTOF_P_SWITCH(k->p, {
     CTOF_CUDA_TRY(allow_smem(k_rows_inv<P_, true>, sm));
-    k_rows_inv<P_, true><<<row_grid(rows, nplanes), ROW_WARPS * 32, sm, st>>>(
-        map, nplanes, rows, cols_out, const_cast<float*>(ref), ld_ref, scale, k->d_tw, k->d_flags, k->max_polls,
-        acc);
+    CTOF_CUDA_TRY(ctof_launch(k_rows_inv<P_, true>, row_grid(rows, nplanes), ROW_WARPS * 32, sm, st, map, nplanes, rows,
+                              cols_out, const_cast<float*>(ref), ld_ref, scale, k->d_tw, k->d_flags, k->max_polls, acc));
   });
   CTOF_CUDA_TRY(cudaGetLastError());
   return CTOF_OK;
@@ -994,8 +998,8 @@ ctof_status fft_rows_admm_t(const ctof_kernel_s* k, float2* inter, const float* 
   CTOF_P_SWITCH(k->p, {
     auto kern = k->n > P_ / 2 ? k_rows_admm_t<P_, false, true> : k_rows_admm_t<P_, false, false>;
     CTOF_CUDA_TRY(allow_smem(kern, sm));
-    kern<<<row_grid(k->n, k->nt), ROW_WARPS * 32, sm, st>>>(map, k->nt, k->n, m, u1, scale, inv_scale, rho, k->d_tw,
-                                                            k->d_flags, k->max_polls);
+    CTOF_CUDA_TRY(ctof_launch(kern, row_grid(k->n, k->nt), ROW_WARPS * 32, sm, st, map, k->nt, k->n, m, u1, scale, inv_scale, rho,
+                              k->d_tw, k->d_flags, k->max_polls));
   });
   CTOF_CUDA_TRY(cudaGetLastError());
   return CTOF_OK;
@@ -1009,8 +1013,8 @@ ctof_status fft_rows_resid_t(const ctof_kernel_s* k, float2* inter, const float*
   CTOF_P_SWITCH(k->p, {
     auto kern = k->n > P_ / 2 ? k_rows_admm_t<P_, true, true> : k_rows_admm_t<P_, true, false>;
     CTOF_CUDA_TRY(allow_smem(kern, sm));
-    kern<<<row_grid(k->n, k->nt), ROW_WARPS * 32, sm, st>>>(map, k->nt, k->n, m, nullptr, scale, 0.f, 0.f, k->d_tw,
-                                                            k->d_flags, k->max_polls);
+    CTOF_CUDA_TRY(ctof_launch(kern, row_grid(k->n, k->nt), ROW_WARPS * 32, sm, st, map, k->nt, k->n, m, nullptr, scale, 0.f, 0.f,
+                              k->d_tw, k->d_flags, k->max_polls));
   });
   CTOF_CUDA_TRY(cudaGetLastError());
   return CTOF_OK;
@@ -1022,7 +1026,7 @@ namespace {
 #define CTOF_COLS_CASE(KERN, PB_, NC_, ...)                                \
   CTOF_P_SWITCH(k->p, {                                                    \
     CTOF_CUDA_TRY(allow_smem(KERN<P_, PB_, NC_>, sm));                     \
-    KERN<P_, PB_, NC_><<<grid, COL_THREADS, sm, st>>>(__VA_ARGS__);        \
+    CTOF_CUDA_TRY(ctof_launch(KERN<P_, PB_, NC_>, grid, COL_THREADS, sm, st, __VA_ARGS__)); \
   })
 
 #define CTOF_COLS_LAUNCH(KERN, ...)                                                      \

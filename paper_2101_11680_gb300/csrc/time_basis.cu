@@ -203,6 +203,7 @@ __global__ void __launch_bounds__(256, 3) k_compress_bulk(const float* __restric
                                                           const float* __restrict__ q, const int4* __restrict__ win,
                                                           int nwin, int rows, float* __restrict__ out,
                                                           int* __restrict__ flag, long long max_polls) {
+  pdl_trigger();
   extern __shared__ __align__(128) unsigned char csm[];
   // the longest windows come last: start with them
   const int k = nwin - 1 - blockIdx.y;
@@ -212,6 +213,7 @@ __global__ void __launch_bounds__(256, 3) k_compress_bulk(const float* __restric
     for (int s = 0; s < CB_STAGES; ++s)
       bulk::bar_init(reinterpret_cast<uint64_t*>(csm + CB_STAGES * cb_stage_bytes(G)) + s, 1);
   __syncthreads();
+  pdl_wait();
   const float* src = m + ((size_t)blockIdx.z * nt + g.x) * npix + p0;
   float* dst = out + ((size_t)blockIdx.z * rows + g.z) * npix + p0;
   const float* qw = q + (size_t)g.x * TZ_R;
@@ -234,6 +236,8 @@ __global__ void __launch_bounds__(256, 3) k_compress_bulk(const float* __restric
 __global__ void __launch_bounds__(256) k_compress(const float* __restrict__ m, int nt, int npix,
                                                   const float* __restrict__ q, const int4* __restrict__ win, int nwin,
                                                   int rows, float* __restrict__ out) {
+  pdl_trigger();
+  pdl_wait();
   __shared__ float s_p[8][TZ_R][32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int4 g = win[blockIdx.y];
@@ -284,6 +288,8 @@ __global__ void __launch_bounds__(256) k_compress(const float* __restrict__ m, i
 template <int V>
 __global__ void __launch_bounds__(256) k_expand(const float* __restrict__ y, int npix, const float* __restrict__ q,
                                                 const int4* __restrict__ tiles, float* __restrict__ m) {
+  pdl_trigger();
+  pdl_wait();
   __shared__ float4 s_q[TZ_TILE * TZ_R / 4];
   const int4 g = tiles[blockIdx.y];  // bins [x, y), first column z, columns w
   if ((int)threadIdx.x < (g.y - g.x) * (TZ_R / 4))
@@ -598,11 +604,11 @@ ctof_status time_compress(const ctof_kernel_s* z, int batch, const float* m, flo
     const float* src = m + (size_t)b0 * z->tz_nt * npix;
     float* dst = out + (size_t)b0 * z->nt * npix;
     if (bulk)
-      kern<<<dim3(ctof_div_up(npix, tile), z->tz_nwin, nb), 256, smem, st>>>(
-          src, z->tz_nt, npix, z->d_tz_q, z->d_tz_win, z->tz_nwin, z->nt, dst, z->d_flags, z->max_polls);
+      CTOF_CUDA_TRY(ctof_launch(kern, dim3(ctof_div_up(npix, tile), z->tz_nwin, nb), 256, smem, st,
+                                src, z->tz_nt, npix, z->d_tz_q, z->d_tz_win, z->tz_nwin, z->nt, dst, z->d_flags, z->max_polls));
     else
-      k_compress<<<dim3(ctof_div_up(npix, 32), z->tz_nwin, nb), 256, 0, st>>>(src, z->tz_nt, npix, z->d_tz_q,
-                                                                             z->d_tz_win, z->tz_nwin, z->nt, dst);
+      CTOF_CUDA_TRY(ctof_launch(k_compress, dim3(ctof_div_up(npix, 32), z->tz_nwin, nb), 256, 0, st, src, z->tz_nt, npix, z->d_tz_q,
+                                                                             z->d_tz_win, z->tz_nwin, z->nt, dst));
   }
   CTOF_CUDA_TRY(cudaGetLastError());
   return CTOF_OK;
@@ -611,9 +617,9 @@ ctof_status time_compress(const ctof_kernel_s* z, int batch, const float* m, flo
 ctof_status time_expand(const ctof_kernel_s* z, const float* y, float* m, cudaStream_t st) {
   const int npix = z->n * z->n;
   if (npix % 2 == 0 && (reinterpret_cast<uintptr_t>(m) & 7) == 0)
-    k_expand<2><<<dim3(ctof_div_up(npix, 512), z->tz_ntiles), 256, 0, st>>>(y, npix, z->d_tz_q, z->d_tz_tiles, m);
+    CTOF_CUDA_TRY(ctof_launch(k_expand<2>, dim3(ctof_div_up(npix, 512), z->tz_ntiles), 256, 0, st, y, npix, z->d_tz_q, z->d_tz_tiles, m));
   else
-    k_expand<1><<<dim3(ctof_div_up(npix, 256), z->tz_ntiles), 256, 0, st>>>(y, npix, z->d_tz_q, z->d_tz_tiles, m);
+    CTOF_CUDA_TRY(ctof_launch(k_expand<1>, dim3(ctof_div_up(npix, 256), z->tz_ntiles), 256, 0, st, y, npix, z->d_tz_q, z->d_tz_tiles, m));
   CTOF_CUDA_TRY(cudaGetLastError());
   return CTOF_OK;
 }
