@@ -16,11 +16,6 @@ namespace {
 
 constexpr int TX = 32, TY = 8;
 
-__device__ __forceinline__ float soft(float a, float thr) {
-  const float m = fabsf(a) - thr;
-  return m > 0.f ? copysignf(m, a) : 0.f;
-}
-
 // One CTA per (32 x 8 lateral tile, ZP consecutive depth planes j0 ..); each
 // thread handles its (x, y) in all ZP planes at once: every load of the block
 // is issued before the first use, and the axial neighbours of planes inside
@@ -196,29 +191,6 @@ __global__ void k_fista_lambda(const double* __restrict__ scalars, const double*
                                      : (float)lam0;
 }
 
-// r -= m
-__global__ void k_sub_meas(float* __restrict__ r, const float* __restrict__ m, size_t count) {
-  pdl_trigger();
-  pdl_wait();
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < count; i += (size_t)gridDim.x * blockDim.x)
-    r[i] -= m[i];
-}
-
-// One FISTA step per voxel (g = A^T (A y - m) unnormalised; x holds x_{k-1} on entry):
-//   x_k = soft(y - g / s^2, lam[z]);  y <- x_k + beta (x_k - x_{k-1});  x <- x_k
-__global__ void k_fista_step(float* __restrict__ y, const float* __restrict__ g, float* __restrict__ x,
-                             const float* __restrict__ lam, float beta, float inv_s2, int plane, size_t count) {
-  pdl_trigger();
-  pdl_wait();
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < count; i += (size_t)gridDim.x * blockDim.x) {
-    const float v = y[i] - inv_s2 * g[i];
-    const float xn = soft(v, lam[i / plane]);
-    const float xo = x[i];
-    x[i] = xn;
-    y[i] = xn + beta * (xn - xo);
-  }
-}
-
 // ---- source multiplexing (Section 5, Eq. 12) ----
 
 // In place: every 8 x 8 block of scan points of every plane ([plane][n][n])
@@ -298,19 +270,6 @@ ctof_status check_finite(const float* v, size_t count, int* flag_dev, cudaStream
 
 ctof_status fista_lambda(const ctof_kernel_s* k, const double* scalars, float* lam, cudaStream_t st) {
   CTOF_CUDA_TRY(ctof_launch(k_fista_lambda, 1, 128, 0, st, scalars, k->d_gram, k->d_members, k->nclass, k->nz, lam));
-  CTOF_CUDA_TRY(cudaGetLastError());
-  return CTOF_OK;
-}
-
-ctof_status fista_sub_meas(float* r, const float* m, size_t count, cudaStream_t st) {
-  CTOF_CUDA_TRY(ctof_launch(k_sub_meas, grid_elem(count), 256, 0, st, r, m, count));
-  CTOF_CUDA_TRY(cudaGetLastError());
-  return CTOF_OK;
-}
-
-ctof_status fista_step(float* y, const float* g, float* x, const float* lam, float beta, float inv_s2, int plane,
-                       size_t count, cudaStream_t st) {
-  CTOF_CUDA_TRY(ctof_launch(k_fista_step, grid_elem(count), 256, 0, st, y, g, x, lam, beta, inv_s2, plane, count));
   CTOF_CUDA_TRY(cudaGetLastError());
   return CTOF_OK;
 }

@@ -60,5 +60,13 @@ cudaError_t ctof_launch(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, 
 }
 #endif
 
+// Soft threshold (proximal map of thr |.|).
+#ifdef __CUDACC__
+__device__ __forceinline__ float soft(float a, float thr) {
+  const float m = fabsf(a) - thr;
+  return m > 0.f ? copysignf(m, a) : 0.f;
+}
+#endif
+
 static inline int ctof_round_up(int x, int m) { return (x + m - 1) / m * m; }
 static inline int ctof_div_up(long long x, long long m) { return (int)((x + m - 1) / m); }

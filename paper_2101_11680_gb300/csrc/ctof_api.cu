@@ -439,40 +439,41 @@ ctof_status tikhonov_run(ctof_kernel_s* k, const ctof_solver_params* prm, cudaSt
 // lam(z) follows the DC depth sensitivity.  With `mux` the operator is the
 // composite S A of Eq. 12 (S = H_64 on every 8 x 8 block of scan points, so
 // the normalisation is 8 s) and the staged measurement is the multiplexed y.
+// S S = 64, so the gradient A^T S (S A x - y) = A^T (64 A x - S y) takes S once,
+// on the measurement.
+// Eight launches per iteration: neither the residual nor the gradient exists as
+// an array of its own, the row passes form them between the two transforms of
+// a row (fourteen launches of 3 to 9 us each before, mostly latency).
 // Workspace: ADMM state buffers.
 ctof_status fista_run(ctof_kernel_s* k, const ctof_solver_params* prm, bool mux, cudaStream_t st) {
-  const size_t vol = (size_t)k->nz * k->n * k->n, meas = (size_t)k->nt * k->n * k->n;
+  const size_t vol = (size_t)k->nz * k->n * k->n;
   float* y = k->d_u3;
   float* x = k->d_xs;
-  float* g = k->d_s;
-  float* r = k->d_u1;
   float* lam = k->d_u2a;
   const double sc = k->scale * (mux ? 8.0 : 1.0);
   const float inv_s2 = (float)(1.0 / (sc * sc));
   CTOF_CUDA_TRY(cudaMemsetAsync(k->d_scalars, 0, 16 * sizeof(double), st));
+  if (mux) CTOF_TRY(block_hadamard(k->d_mstage, k->nt, k->n, st));
   if (prm->tv_beta < 0) {
-    if (mux) {
-      CTOF_CUDA_TRY(cudaMemcpyAsync(r, k->d_mstage, meas * sizeof(float), cudaMemcpyDeviceToDevice, st));
-      CTOF_TRY(block_hadamard(r, k->nt, k->n, st));
-      CTOF_TRY(adjoint_impl(k, r, k->d_vstage, st));
-    } else {
-      CTOF_TRY(adjoint_impl(k, k->d_mstage, k->d_vstage, st));
-    }
+    CTOF_TRY(adjoint_impl(k, k->d_mstage, k->d_vstage, st));
     CTOF_TRY(reduce_max_abs(k->d_vstage, vol, k->d_scalars + 1, st));
   }
   CTOF_TRY(admm_set_beta(k->d_scalars, prm->tv_beta, prm->beta_rel, 1.0 / (sc * sc), st));
   CTOF_TRY(fista_lambda(k, k->d_scalars, lam, st));
   CTOF_CUDA_TRY(cudaMemsetAsync(y, 0, vol * sizeof(float), st));
   CTOF_CUDA_TRY(cudaMemsetAsync(x, 0, vol * sizeof(float), st));
+  CTOF_CUDA_TRY(cudaMemsetAsync(k->d_inter_z, 0, fft_inter_elems(k, k->nz, k->n) * sizeof(float2), st));
   double t = 1.0;
   for (int it = 0; it < prm->iters; ++it) {
-    CTOF_TRY(forward_impl(k, y, r, st));
-    if (mux) CTOF_TRY(block_hadamard(r, k->nt, k->n, st));
-    CTOF_TRY(fista_sub_meas(r, k->d_mstage, meas, st));
-    if (mux) CTOF_TRY(block_hadamard(r, k->nt, k->n, st));  // S^T = S
-    CTOF_TRY(adjoint_impl(k, r, g, st));
+    CTOF_TRY(fft_cols_forward(k, k->d_inter_z, k->nz, k->n, k->d_spec_z, k->ldz, st));
+    CTOF_TRY(contract_forward(k, k->d_spec_z, k->d_spec_t, st));
+    CTOF_TRY(fft_cols_inverse(k, k->d_spec_t, k->ldt, k->nt, k->n, k->d_inter_t, st));
+    CTOF_TRY(fft_rows_resid_t(k, k->d_inter_t, k->d_mstage, mux ? 64.f : 1.f, st));
+    CTOF_TRY(fft_cols_forward(k, k->d_inter_t, k->nt, k->n, k->d_spec_t, k->ldt, st));
+    CTOF_TRY(contract_adjoint(k, k->d_spec_t, k->d_spec_z, st));
+    CTOF_TRY(fft_cols_inverse(k, k->d_spec_z, k->ldz, k->nz, k->n, k->d_inter_z, st));
     const double t_next = 0.5 * (1.0 + sqrt(1.0 + 4.0 * t * t));
-    CTOF_TRY(fista_step(y, g, x, lam, (float)((t - 1.0) / t_next), inv_s2, k->n * k->n, vol, st));
+    CTOF_TRY(fft_rows_fista(k, k->d_inter_z, y, x, lam, inv_s2, (float)((t - 1.0) / t_next), st));
     t = t_next;
   }
   CTOF_CUDA_TRY(cudaMemcpyAsync(k->d_vstage, x, vol * sizeof(float), cudaMemcpyDeviceToDevice, st));

@@ -201,9 +201,14 @@ ctof_status fft_rows_inverse(const ctof_kernel_s* k, const float2* inter, int np
 // the correction c, in place in `inter` ([nt][n][hp]).
 ctof_status fft_rows_admm_t(const ctof_kernel_s* k, float2* inter, const float* m, float* u1,
                             float inv_scale, float rho, cudaStream_t st);
-// Learned-solver T side, in place on inter [n][kx][nt planes]: inverse rows,
-// crop to the scan, c = Kx - m (Kx when m is null), forward rows of c.
-ctof_status fft_rows_resid_t(const ctof_kernel_s* k, float2* inter, const float* m, cudaStream_t st);
+// Residual T side, in place on inter [n][kx][nt planes]: inverse rows, crop to
+// the scan, c = gain Kx - m (gain Kx when m is null; gain a power of two), forward rows of c.
+ctof_status fft_rows_resid_t(const ctof_kernel_s* k, float2* inter, const float* m, float gain, cudaStream_t st);
+// FISTA's proximal step, in place on inter [n][kx][nz planes] holding the
+// gradient's rows: x' = soft(y - step g, thr[plane]), y <- x' + beta (x' - x),
+// x <- x', then the forward rows of y.
+ctof_status fft_rows_fista(const ctof_kernel_s* k, float2* inter, float* y, float* x, const float* thr, float step,
+                           float beta, cudaStream_t st);
 // Inverse rows without a store: acc[0] += sum (z - ref)^2, acc[1] += sum ref^2
 // over the first cols_out columns (ref laid out like fft_rows_inverse's out).
 ctof_status fft_rows_inverse_norm(const ctof_kernel_s* k, const float2* inter, int nplanes, int rows, int cols_out,
@@ -297,11 +302,7 @@ ctof_status reduce_max_abs(const float* v, size_t count, double* out_dev, cudaSt
 ctof_status admm_set_beta(double* scalars, double beta_fixed, double beta_rel, double inv_scale2,
                           cudaStream_t st);
 ctof_status check_finite(const float* v, size_t count, int* flag_dev, cudaStream_t st);
-// FISTA (Eq. 8, Eq. 10): per-depth weights from lam0 = scalars[0], r -= m, and one step
-// (x holds x_{k-1} on entry and x_k on exit; y becomes the next extrapolated point).
+// FISTA (Eq. 8, Eq. 10): per-depth weights from lam0 = scalars[0].
 ctof_status fista_lambda(const ctof_kernel_s* k, const double* scalars, float* lam, cudaStream_t st);
 // In place, [planes][n][n]: every 8 x 8 block of scan points <- H_64 times it (n % 8 == 0).
 ctof_status block_hadamard(float* v, int planes, int n, cudaStream_t st);
-ctof_status fista_sub_meas(float* r, const float* m, size_t count, cudaStream_t st);
-ctof_status fista_step(float* y, const float* g, float* x, const float* lam, float beta, float inv_s2, int plane,
-                       size_t count, cudaStream_t st);

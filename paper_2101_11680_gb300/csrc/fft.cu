@@ -600,18 +600,23 @@ __global__ void __launch_bounds__(ROW_WARPS * 32) k_rows_inv(const __grid_consta
 //   c    = (v1 - u1) - Kx = 2 v1 - a1 - Kx      (zero off the scan)
 //   row spectra <- R2C(c zero-padded to P)
 // so that FFT(v1 - u1) = K x_hat + c_hat without a transform of the full
-// P x P plane.  With RESID the update is the data residual of the gradient
-// A^T (A x - m) instead: c = Kx - m on the scan (Kx alone when m is null;
-// u1, inv_s and rho unused).  m, u1: [nt][n][n]; inter: [n][kx][plane] in
-// place (tensor map `map`).  The m and u1 values of a lane are loaded before
-// its tile is waited for; the next job's tile is requested once the copy out
-// of its buffer has read it.
+// P x P plane.  ROWS_RESID: the data residual of the gradient A^T (A x - m)
+// instead: c = Kx - m on the scan (Kx alone when m is null; u1, inv_s and rho
+// unused).  ROWS_FISTA, on the depth planes: the proximal step that turns the
+// gradient rows g into the next point's rows (m: y, u1: x, both updated; thr:
+// per-plane threshold; inv_s: step, rho: extrapolation weight),
+//   x' = soft(y - inv_s g, thr),  y <- x' + rho (x' - x),  x <- x'.
+// m, u1: [planes][n][n]; inter: [n][kx][plane] in place (tensor map `map`).
+// The m and u1 values of a lane are loaded before its tile is waited for; the
+// next job's tile is requested once the copy out of its buffer has read it.
+constexpr int ROWS_ADMM = 0, ROWS_RESID = 1, ROWS_FISTA = 2;
+
 // WIDE: more than P / 2 scan columns (a circular scan fills the grid).
-template <int P, bool RESID, bool WIDE>
+template <int P, int MODE, bool WIDE>
 __global__ void __launch_bounds__(ROW_WARPS * 32, P >= 512 ? 2 : 3)
-    k_rows_admm_t(const __grid_constant__ CUtensorMap map, int nplanes, int n, const float* __restrict__ m,
-                  float* __restrict__ u1, float scale, float inv_s, float rho, const float2* __restrict__ tw,
-                  int* __restrict__ flag, long long max_polls) {
+    k_rows_admm_t(const __grid_constant__ CUtensorMap map, int nplanes, int n, float* __restrict__ m,
+                  float* __restrict__ u1, const float* __restrict__ thr, float scale, float inv_s, float rho,
+                  const float2* __restrict__ tw, int* __restrict__ flag, long long max_polls) {
   constexpr int R = P / 32;
   constexpr int RN = WIDE || R < 2 ? R : R / 2;  // registers that can hold scan columns
   extern __shared__ float4 row_smem4[];
@@ -631,13 +636,17 @@ __global__ void __launch_bounds__(ROW_WARPS * 32, P >= 512 ? 2 : 3)
     const int p0 = pl0 + 2 * warp, p1 = p0 + 1;
     const bool has0 = p0 < nplanes, has1 = p1 < nplanes;
     float2* s_h = sh_buf<P>(S, it & 1);
-    float mv0[RN], mv1[RN], uv0[RN], uv1[RN];
+    float mv0[RN], mv1[RN], uv0[RN], uv1[RN], th0 = 0.f, th1 = 0.f;
+    if constexpr (MODE == ROWS_FISTA) {
+      if (has0) th0 = thr[p0];
+      if (has1) th1 = thr[p1];
+    }
     const size_t row0 = ((size_t)p0 * n + r) * n, row1 = ((size_t)p1 * n + r) * n;
 #pragma unroll
     for (int i = 0; i < RN; ++i) {
       const int c = lane + 32 * i;
       mv0[i] = uv0[i] = mv1[i] = uv1[i] = 0.f;
-      if constexpr (RESID) {
+      if constexpr (MODE == ROWS_RESID) {
         if (m != nullptr && c < n) {
           if (has0) mv0[i] = m[row0 + c];
           if (has1) mv1[i] = m[row1 + c];
@@ -671,9 +680,22 @@ __global__ void __launch_bounds__(ROW_WARPS * 32, P >= 512 ? 2 : 3)
       const int c = lane + 32 * i;
       if (c < n) {
         const float2 kx = cscale(S.buf[row_pos<P>(c)], scale);
-        if constexpr (RESID) {
+        if constexpr (MODE == ROWS_RESID) {
           if (has0) v[i].x = kx.x - mv0[i];
           if (has1) v[i].y = kx.y - mv1[i];
+          continue;
+        }
+        if constexpr (MODE == ROWS_FISTA) {
+          auto step = [&](float g, float yo, float xo, float t, size_t at) {
+            const float w = yo - inv_s * g;
+            const float xn = soft(w, t);
+            const float yn = xn + rho * (xn - xo);
+            u1[at] = xn;
+            m[at] = yn;
+            return yn;
+          };
+          if (has0) v[i].x = step(kx.x, mv0[i], uv0[i], th0, row0 + c);
+          if (has1) v[i].y = step(kx.y, mv1[i], uv1[i], th1, row1 + c);
           continue;
         }
         if (has0) {
@@ -989,35 +1011,39 @@ ctof_status fft_rows_inverse_norm(const ctof_kernel_s* k, const float2* inter, i
   return CTOF_OK;
 }
 
-ctof_status fft_rows_admm_t(const ctof_kernel_s* k, float2* inter, const float* m, float* u1, float inv_scale,
-                            float rho, cudaStream_t st) {
+namespace {
+
+template <int MODE>
+ctof_status rows_in_place(const ctof_kernel_s* k, float2* inter, int nplanes, float* m, float* u1, const float* thr,
+                          float gain, float inv_s, float rho, cudaStream_t st) {
   CUtensorMap map;
-  CTOF_TRY(row_map(k, &map, inter, k->nt, k->n));
+  CTOF_TRY(row_map(k, &map, inter, nplanes, k->n));
   const size_t sm = row_smem_bytes(k->p);
-  const float scale = 1.0f / ((float)k->p * (float)k->p);
+  const float scale = gain / ((float)k->p * (float)k->p);
   CTOF_P_SWITCH(k->p, {
-    auto kern = k->n > P_ / 2 ? k_rows_admm_t<P_, false, true> : k_rows_admm_t<P_, false, false>;
+    auto kern = k->n > P_ / 2 ? k_rows_admm_t<P_, MODE, true> : k_rows_admm_t<P_, MODE, false>;
     CTOF_CUDA_TRY(allow_smem(kern, sm));
-    CTOF_CUDA_TRY(ctof_launch(kern, row_grid(k->n, k->nt), ROW_WARPS * 32, sm, st, map, k->nt, k->n, m, u1, scale, inv_scale, rho,
-                              k->d_tw, k->d_flags, k->max_polls));
+    CTOF_CUDA_TRY(ctof_launch(kern, row_grid(k->n, nplanes), ROW_WARPS * 32, sm, st, map, nplanes, k->n, m, u1, thr,
+                              scale, inv_s, rho, k->d_tw, k->d_flags, k->max_polls));
   });
   CTOF_CUDA_TRY(cudaGetLastError());
   return CTOF_OK;
 }
 
-ctof_status fft_rows_resid_t(const ctof_kernel_s* k, float2* inter, const float* m, cudaStream_t st) {
-  CUtensorMap map;
-  CTOF_TRY(row_map(k, &map, inter, k->nt, k->n));
-  const size_t sm = row_smem_bytes(k->p);
-  const float scale = 1.0f / ((float)k->p * (float)k->p);
-  CTOF_P_SWITCH(k->p, {
-    auto kern = k->n > P_ / 2 ? k_rows_admm_t<P_, true, true> : k_rows_admm_t<P_, true, false>;
-    CTOF_CUDA_TRY(allow_smem(kern, sm));
-    CTOF_CUDA_TRY(ctof_launch(kern, row_grid(k->n, k->nt), ROW_WARPS * 32, sm, st, map, k->nt, k->n, m, nullptr, scale, 0.f, 0.f,
-                              k->d_tw, k->d_flags, k->max_polls));
-  });
-  CTOF_CUDA_TRY(cudaGetLastError());
-  return CTOF_OK;
+}  // namespace
+
+ctof_status fft_rows_admm_t(const ctof_kernel_s* k, float2* inter, const float* m, float* u1, float inv_scale,
+                            float rho, cudaStream_t st) {
+  return rows_in_place<ROWS_ADMM>(k, inter, k->nt, const_cast<float*>(m), u1, nullptr, 1.f, inv_scale, rho, st);
+}
+
+ctof_status fft_rows_resid_t(const ctof_kernel_s* k, float2* inter, const float* m, float gain, cudaStream_t st) {
+  return rows_in_place<ROWS_RESID>(k, inter, k->nt, const_cast<float*>(m), nullptr, nullptr, gain, 0.f, 0.f, st);
+}
+
+ctof_status fft_rows_fista(const ctof_kernel_s* k, float2* inter, float* y, float* x, const float* thr, float step,
+                           float beta, cudaStream_t st) {
+  return rows_in_place<ROWS_FISTA>(k, inter, k->nz, y, x, thr, 1.f, step, beta, st);
 }
 
 namespace {

@@ -1070,7 +1070,7 @@ ctof_status residual_back(ctof_kernel_s* k, int batch, const float* x, const flo
   for (int b = 0; b < batch; ++b) {
     float2* spec = w.spec_t + b * stt;
     CTOF_TRY(fft_cols_inverse(k, spec, k->ldt, k->nt, k->n, k->d_inter_t, st));
-    CTOF_TRY(fft_rows_resid_t(k, k->d_inter_t, m ? m + b * mt : nullptr, st));
+    CTOF_TRY(fft_rows_resid_t(k, k->d_inter_t, m ? m + b * mt : nullptr, 1.f, st));
     CTOF_TRY(fft_cols_forward(k, k->d_inter_t, k->nt, k->n, spec, k->ldt, st));
   }
   return spectra_adjoint(k, batch, out, tik_hinv, w, st);
