@@ -582,93 +582,174 @@ __global__ void __launch_bounds__(CV_THREADS) k_conv_first(const float* __restri
   }
 }
 
-// Per-CTA partial weight gradients: part[blk][tap][co][ci] = sum over this CTA's
-// voxels of dy[v][co] act(x[v + off(tap)][ci]).  Warp w owns taps w, w+8, w+16, w+24.
-constexpr int WG_ROWS = 16;  // (b, z, y) rows per CTA
-__global__ void __launch_bounds__(256) k_wgrad(const __nv_bfloat16* __restrict__ dy, const __nv_bfloat16* __restrict__ x,
-                                               int relu_in, Geo G, float* __restrict__ part) {
+// Weight and bias gradients of one layer:
+//   dw[tap][co][ci] = sum_v dy[v][co] act(x[v + off(tap)][ci]),  db[co] = sum_v dy[v][co].
+// Per tap a 16 x 16 product over all voxels; 11 GFLOP and 50 MB of activations
+// for four 64 x 64 x 48 problems, so the launch is bound by getting voxels to the
+// warps (a gather of single BF16 values per lane took 293 us, this kernel 68).  A
+// CTA takes 8 rows x up to 64 columns and marches along z: three activation
+// planes (with their halo, ReLU applied once) and one gradient plane sit in
+// shared memory, the next plane is loaded into registers while this one is
+// used.  Fragments come by transposing ldmatrix (voxels are the K dimension of
+// both operands); a voxel's two 16-byte halves are swapped by bit 2 of its
+// column so that eight consecutive voxels, at any shift, fall on distinct banks.
+// Twelve warps: dz (9 taps) x four pairs of rows; the dz = 0 warps also sum dy,
+// as a product with ones.  Partial sums per CTA, in a fixed order.
+constexpr int WG_Y = 8, WG_X = 64, WG_THREADS = 384;
+constexpr int WG_XP = WG_X + 2, WG_YP = WG_Y + 2;
+constexpr int WG_PLANE = WG_YP * WG_XP * 32, WG_DY = WG_Y * WG_X * 32;
+constexpr int WG_SMEM = 3 * WG_PLANE + WG_DY;
+constexpr int WG_OUT = 27 * CH * CH + CH;  // floats per partial: dw, then db
+constexpr int WG_LX = (WG_YP * WG_XP * 2 + WG_THREADS - 1) / WG_THREADS;  // 16-byte loads per thread and plane
+constexpr int WG_LD = (WG_Y * WG_X * 2 + WG_THREADS - 1) / WG_THREADS;
+
+__device__ __forceinline__ int wg_off(int row, int pitch, int vx, int h) {
+  return (row * pitch + vx) * 32 + ((h ^ ((vx >> 2) & 1)) << 4);
+}
+
+__device__ __forceinline__ void ldsm_x4_t(unsigned (&r)[4], uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr));
+}
+
+__global__ void __launch_bounds__(WG_THREADS, 1) k_wgrad(const __nv_bfloat16* __restrict__ dy,
+                                                         const __nv_bfloat16* __restrict__ x, int relu_in, Geo G,
+                                                         int zs, float* __restrict__ part) {
+  extern __shared__ __align__(128) unsigned char wgs[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int g = lane >> 2, tg = lane & 3;
-  const long long rows = (long long)G.b * G.z * G.y;
-  const long long r0 = (long long)blockIdx.x * WG_ROWS;
-  float acc[4][2][4] = {};
-  const __nv_bfloat16* dyb = dy;
-  for (long long row = r0; row < r0 + WG_ROWS && row < rows; ++row) {
-    const int yy = (int)(row % G.y);
-    const int zz = (int)((row / G.y) % G.z);
-    const int bb = (int)(row / ((long long)G.y * G.z));
-    for (int x0 = 0; x0 < G.x; x0 += 16) {
-      const long long vb = neighbour(G, bb, zz, yy, x0);
-      // A = dy^T: rows co, cols the 16 voxels
-      unsigned a[4];
-      a[0] = pack2(dyb[(vb + 2 * tg) * CH + g], dyb[(vb + 2 * tg + 1) * CH + g]);
-      a[1] = pack2(dyb[(vb + 2 * tg) * CH + g + 8], dyb[(vb + 2 * tg + 1) * CH + g + 8]);
-      a[2] = pack2(dyb[(vb + 2 * tg + 8) * CH + g], dyb[(vb + 2 * tg + 9) * CH + g]);
-      a[3] = pack2(dyb[(vb + 2 * tg + 8) * CH + g + 8], dyb[(vb + 2 * tg + 9) * CH + g + 8]);
+  const int g = lane >> 2, tg = lane & 3, mi = lane >> 3, lr = lane & 7;
+  const int nxc = (G.x + WG_X - 1) / WG_X, nyc = (G.y + WG_Y - 1) / WG_Y, nzc = (G.z + zs - 1) / zs;
+  int job = blockIdx.x;
+  const int x0 = (job % nxc) * WG_X;
+  job /= nxc;
+  const int y0 = (job % nyc) * WG_Y;
+  job /= nyc;
+  const int z0 = (job % nzc) * zs, bb = job / nzc, z1 = min(G.z, z0 + zs);
+  const uint4 zero4 = make_uint4(0u, 0u, 0u, 0u);
+  auto load_x = [&](uint4 (&r)[WG_LX], int zz) {
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int tap = warp + 8 * j;
-        if (tap >= 27) break;
-        const int dz = tap / 9 - 1, dy_ = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
-        const long long n0 = neighbour(G, bb, zz + dz, yy + dy_, x0 + 2 * tg + dx);
-        const long long n1 = neighbour(G, bb, zz + dz, yy + dy_, x0 + 2 * tg + 1 + dx);
-        const long long n8 = neighbour(G, bb, zz + dz, yy + dy_, x0 + 2 * tg + 8 + dx);
-        const long long n9 = neighbour(G, bb, zz + dz, yy + dy_, x0 + 2 * tg + 9 + dx);
+    for (int i = 0; i < WG_LX; ++i) {
+      const int e = threadIdx.x + i * WG_THREADS, v = e >> 1, row = v / WG_XP, col = v - row * WG_XP;
+      r[i] = zero4;
+      if (row < WG_YP) {
+        const long long n = neighbour(G, bb, zz, y0 + row - 1, x0 + col - 1);
+        if (n >= 0) r[i] = __ldg(reinterpret_cast<const uint4*>(x + n * CH) + (e & 1));
+      }
+    }
+  };
+  auto put_x = [&](const uint4 (&r)[WG_LX], int zz) {
+    unsigned char* dst = wgs + ((zz + 3) % 3) * WG_PLANE;
 #pragma unroll
-        for (int nt = 0; nt < 2; ++nt) {
-          const int ci = nt * 8 + g;
-          const __nv_bfloat16 zb = __float2bfloat16_rn(0.f);
-          __nv_bfloat16 e0 = n0 >= 0 ? x[n0 * CH + ci] : zb, e1 = n1 >= 0 ? x[n1 * CH + ci] : zb;
-          __nv_bfloat16 e8 = n8 >= 0 ? x[n8 * CH + ci] : zb, e9 = n9 >= 0 ? x[n9 * CH + ci] : zb;
-          unsigned b0 = pack2(e0, e1), b1 = pack2(e8, e9);
-          if (relu_in) {
-            b0 = relu2(b0);
-            b1 = relu2(b1);
-          }
-          mma_bf16(acc[j][nt], a, b0, b1);
+    for (int i = 0; i < WG_LX; ++i) {
+      const int e = threadIdx.x + i * WG_THREADS, v = e >> 1, row = v / WG_XP, col = v - row * WG_XP;
+      uint4 q = r[i];
+      if (relu_in) q = make_uint4(relu2(q.x), relu2(q.y), relu2(q.z), relu2(q.w));
+      if (row < WG_YP) *reinterpret_cast<uint4*>(dst + wg_off(row, WG_XP, col, e & 1)) = q;
+    }
+  };
+  unsigned char* sdy = wgs + 3 * WG_PLANE;
+  auto load_dy = [&](uint4 (&r)[WG_LD], int zz) {
+#pragma unroll
+    for (int i = 0; i < WG_LD; ++i) {
+      const int e = threadIdx.x + i * WG_THREADS, v = e >> 1, row = v / WG_X, col = v - row * WG_X;
+      r[i] = zero4;
+      if (row < WG_Y && zz < z1) {
+        const long long n = neighbour(G, bb, zz, y0 + row, x0 + col);
+        if (n >= 0) r[i] = __ldg(reinterpret_cast<const uint4*>(dy + n * CH) + (e & 1));
+      }
+    }
+  };
+  auto put_dy = [&](const uint4 (&r)[WG_LD]) {
+#pragma unroll
+    for (int i = 0; i < WG_LD; ++i) {
+      const int e = threadIdx.x + i * WG_THREADS, v = e >> 1, row = v / WG_X, col = v - row * WG_X;
+      if (row < WG_Y) *reinterpret_cast<uint4*>(sdy + wg_off(row, WG_X, col, e & 1)) = r[i];
+    }
+  };
+  uint4 rx[WG_LX], rd[WG_LD];
+  load_x(rx, z0 - 1);
+  put_x(rx, z0 - 1);
+  load_x(rx, z0);
+  put_x(rx, z0);
+  load_x(rx, z0 + 1);
+  load_dy(rd, z0);
+  const int dz = warp % 3 - 1, kg = warp / 3;
+  const int ngrp = min(WG_X, G.x - x0) / 16;
+  const uint32_t s_x = (uint32_t)__cvta_generic_to_shared(wgs), s_d = (uint32_t)__cvta_generic_to_shared(sdy);
+  const unsigned ones = pack2(__float2bfloat16_rn(1.f), __float2bfloat16_rn(1.f));
+  float acc[9][2][4] = {}, accb[4] = {};
+  for (int zz = z0; zz < z1; ++zz) {
+    put_x(rx, zz + 1);
+    put_dy(rd);
+    __syncthreads();
+    load_x(rx, zz + 2);
+    load_dy(rd, zz + 1);
+    const uint32_t sp = s_x + ((zz + dz + 3) % 3) * WG_PLANE;
+#pragma unroll
+    for (int rr = 0; rr < 2; ++rr) {
+      const int y = 2 * kg + rr;
+      for (int gx = 0; gx < ngrp; ++gx) {
+        const int vb = gx * 16 + lr;
+        unsigned a[4];  // (voxels 0-7 | 8-15) x (co 0-7 | 8-15), transposed
+        ldsm_x4_t(a, s_d + wg_off(y, WG_X, vb + ((mi >> 1) << 3), mi & 1));
+        if (dz == 0) mma_bf16(accb, a, ones, ones);
+#pragma unroll
+        for (int t = 0; t < 9; ++t) {
+          unsigned b[4];
+          ldsm_x4_t(b, sp + wg_off(y + t / 3, WG_XP, vb + t % 3 + ((mi & 1) << 3), mi >> 1));
+          mma_bf16(acc[t][0], a, b[0], b[1]);
+          mma_bf16(acc[t][1], a, b[2], b[3]);
         }
       }
     }
+    __syncthreads();
   }
-  float* p = part + (size_t)blockIdx.x * 27 * CH * CH;
+  // the four row groups' sums, one after the other
+  float* red = reinterpret_cast<float*>(wgs);
+  for (int r = 0; r < 4; ++r) {
+    if (kg == r) {
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const int tap = warp + 8 * j;
-    if (tap >= 27) break;
+      for (int t = 0; t < 9; ++t) {
+        float* q = red + ((dz + 1) * 9 + t) * CH * CH;
 #pragma unroll
-    for (int nt = 0; nt < 2; ++nt) {
-      const int ci = nt * 8 + 2 * tg;
-      p[(tap * CH + g) * CH + ci] = acc[j][nt][0];
-      p[(tap * CH + g) * CH + ci + 1] = acc[j][nt][1];
-      p[(tap * CH + g + 8) * CH + ci] = acc[j][nt][2];
-      p[(tap * CH + g + 8) * CH + ci + 1] = acc[j][nt][3];
+        for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            float* e = q + (g + 8 * (i >> 1)) * CH + nt * 8 + 2 * tg + (i & 1);
+            *e = r == 0 ? acc[t][nt][i] : *e + acc[t][nt][i];
+          }
+      }
+      if (dz == 0 && tg == 0) {  // every column of the product with ones holds the sum
+        float* e = red + 27 * CH * CH + g;
+        e[0] = r == 0 ? accb[0] : e[0] + accb[0];
+        e[8] = r == 0 ? accb[2] : e[8] + accb[2];
+      }
     }
+    __syncthreads();
   }
+  float* p = part + (size_t)blockIdx.x * WG_OUT;
+  for (int i = threadIdx.x; i < WG_OUT; i += WG_THREADS) p[i] = red[i];
 }
 
-// acc[i] += sum over blocks of part[blk][i]  (i < 27*16*16)
-__global__ void k_reduce_parts(const float* __restrict__ part, int nblk, float* __restrict__ acc) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= 27 * CH * CH) return;
+// dw += sum_b part[b], db likewise: a block takes 32 outputs, its eight warps
+// every eighth partial, and the warps' sums meet in a fixed order.
+__global__ void __launch_bounds__(256) k_reduce_parts(const float* __restrict__ part, int nblk, float* __restrict__ dw,
+                                                      float* __restrict__ db) {
+  __shared__ float red[8][32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, i = blockIdx.x * 32 + lane;
   float s = 0.f;
-  for (int b = 0; b < nblk; ++b) s += part[(size_t)b * 27 * CH * CH + i];
-  acc[i] += s;
-}
-
-// db[c] += sum_v dy[v][c]
-__global__ void k_bias_grad(const __nv_bfloat16* __restrict__ dy, long long nvox, float* __restrict__ db) {
-  __shared__ float red[256][CH + 1];
-  float s[CH] = {};
-  for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < nvox; v += (long long)gridDim.x * blockDim.x)
-#pragma unroll
-    for (int c = 0; c < CH; ++c) s[c] += __bfloat162float(dy[v * CH + c]);
-#pragma unroll
-  for (int c = 0; c < CH; ++c) red[threadIdx.x][c] = s[c];
+  if (i < WG_OUT) {
+#pragma unroll 8
+    for (int b = warp; b < nblk; b += 8) s += part[(size_t)b * WG_OUT + i];
+  }
+  red[warp][lane] = s;
   __syncthreads();
-  if (threadIdx.x < CH) {
-    float t = 0.f;
-    for (int i = 0; i < blockDim.x; ++i) t += red[i][threadIdx.x];
-    atomicAdd(&db[threadIdx.x], t);
+  if (warp == 0 && i < WG_OUT) {
+#pragma unroll
+    for (int w = 1; w < 8; ++w) s += red[w][lane];
+    float* d = i < 27 * CH * CH ? dw + i : db + (i - 27 * CH * CH);
+    *d += s;
   }
 }
 
@@ -805,6 +886,15 @@ cudaError_t sub_inplace(float* a, const float* b, long long n, cudaStream_t st) 
   return cudaGetLastError();
 }
 
+// CTAs of the weight gradient and the planes of a CTA's z segment: segments as
+// long as some 500 CTAs allow (each loads two planes of halo).
+int wg_jobs(const Geo& G, int* zs) {
+  const int cols = G.b * ((G.y + WG_Y - 1) / WG_Y) * ((G.x + WG_X - 1) / WG_X);
+  const long long want = (long long)cols * G.z / 500;
+  *zs = want < 1 ? 1 : want > G.z ? G.z : (int)want;
+  return cols * ((G.z + *zs - 1) / *zs);
+}
+
 int grid_for(long long n) {
   long long b = (n + 255) / 256;
   if (b > 152 * 16) b = 152 * 16;
@@ -855,7 +945,6 @@ struct Ws {
   __nv_bfloat16 *u, *y1, *y2, *y3;  // [S][V][16]
   __nv_bfloat16 *da, *db_;  // [V][16]
   float* part;
-  int nblk;
   float2 *spec_t, *spec_z;  // [batch][nf][ldt], [batch][nf][ldz] (or [nf][ldzb], see zb)
   // Z side as one plane-batched FFT over batch * nz planes (batch >= 4, nz even):
   // spectra interleaved per frequency, row pitch ldzb, own FFT intermediate
@@ -866,8 +955,8 @@ struct Ws {
 ctof_status learned_workspace(ctof_learned_s* L, const ctof_kernel_s* k, int batch, bool train, Ws* w) {
   const long long V = (long long)batch * k->nz * k->n * k->n;
   const int S = train ? L->stages : 1;
-  const long long rows = (long long)batch * k->nz * k->n;
-  const int nblk = (int)((rows + WG_ROWS - 1) / WG_ROWS);
+  int zs;
+  const int nblk = train ? wg_jobs(Geo{batch, k->nz, k->n, k->n}, &zs) : 0;
   size_t need = 0;
   auto add = [&](size_t b) {
     const size_t at = need;
@@ -879,7 +968,7 @@ ctof_status learned_workspace(ctof_learned_s* L, const ctof_kernel_s* k, int bat
   const size_t o_u = add((size_t)S * V * CH * 2), o_y1 = add((size_t)S * V * CH * 2), o_y2 = add((size_t)S * V * CH * 2),
                o_y3 = add((size_t)S * V * CH * 2);
   const size_t o_da = add(V * CH * 2), o_db = add(V * CH * 2);
-  const size_t o_p = add((size_t)nblk * 27 * CH * CH * 4);
+  const size_t o_p = add((size_t)nblk * WG_OUT * 4);
   const size_t o_st = add((size_t)batch * k->nf * k->ldt * 8), o_sz = add((size_t)batch * k->nf * k->ldz * 8);
   const bool zb = batch >= 4 && (k->nz % 2) == 0;
   const size_t o_izb = add(zb ? fft_inter_elems(k, batch * k->nz, k->n) * 8 : 0);
@@ -912,7 +1001,6 @@ ctof_status learned_workspace(ctof_learned_s* L, const ctof_kernel_s* k, int bat
   w->spec_z = reinterpret_cast<float2*>(b + o_sz);
   w->inter_zb = zb ? reinterpret_cast<float2*>(b + o_izb) : nullptr;
   w->ldzb = zb ? ctof_round_up(batch * k->nz, 8) : 0;
-  w->nblk = nblk;
   return CTOF_OK;
 }
 
@@ -1001,11 +1089,14 @@ ctof_status conv(const __nv_bfloat16* in, int relu_in, const __nv_bfloat16* wt, 
   return conv_launch<false, false>(in, nullptr, 0.f, relu_in, wt, bias, mask, out, nullptr, nullptr, G, st);
 }
 
-ctof_status wgrad(const __nv_bfloat16* dy, const __nv_bfloat16* x, int relu_in, Geo G, float* part, int nblk, float* acc,
+ctof_status wgrad(const __nv_bfloat16* dy, const __nv_bfloat16* x, int relu_in, Geo G, float* part, float* dw, float* db,
                   cudaStream_t st) {
-  k_wgrad<<<nblk, 256, 0, st>>>(dy, x, relu_in, G, part);
+  int zs;
+  const int nblk = wg_jobs(G, &zs);
+  CTOF_CUDA_TRY(cudaFuncSetAttribute(k_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, WG_SMEM));
+  k_wgrad<<<nblk, WG_THREADS, WG_SMEM, st>>>(dy, x, relu_in, G, zs, part);
   CTOF_CUDA_TRY(cudaGetLastError());
-  k_reduce_parts<<<(27 * CH * CH + 255) / 256, 256, 0, st>>>(part, nblk, acc);
+  k_reduce_parts<<<(WG_OUT + 31) / 32, 256, 0, st>>>(part, nblk, dw, db);
   CTOF_CUDA_TRY(cudaGetLastError());
   return CTOF_OK;
 }
@@ -1168,7 +1259,6 @@ ctof_status unrolled_backward(ctof_learned_s* L, ctof_kernel_s* k, int batch, co
   CTOF_CUDA_TRY(cudaMemsetAsync(L->d_loss, 0, sizeof(double), st));
   k_loss<<<grid_for(V), 256, 0, st>>>(w.x, mu, V, w.gx, L->d_loss);
   CTOF_CUDA_TRY(cudaGetLastError());
-  const int bg_blocks = grid_for(V) < 304 ? grid_for(V) : 304;
   for (int s = L->stages - 1; s >= 0; --s) {
     const float* g = w.g + (size_t)s * V;
     const __nv_bfloat16* u = w.u + (size_t)s * V * CH;
@@ -1183,9 +1273,7 @@ ctof_status unrolled_backward(ctof_learned_s* L, ctof_kernel_s* k, int batch, co
     __nv_bfloat16* cur = w.da;
     __nv_bfloat16* nxt = w.db_;
     for (int l = NLAYER - 1; l >= 0; --l) {
-      CTOF_TRY(wgrad(cur, acts[l], l > 0 ? 1 : 0, G, w.part, w.nblk, L->d_dw + (size_t)l * 27 * CH * CH, st));
-      k_bias_grad<<<bg_blocks, 256, 0, st>>>(cur, V, L->d_db + l * CH);
-      CTOF_CUDA_TRY(cudaGetLastError());
+      CTOF_TRY(wgrad(cur, acts[l], l > 0 ? 1 : 0, G, w.part, L->d_dw + (size_t)l * 27 * CH * CH, L->d_db + l * CH, st));
       // gradient w.r.t. this layer's input: masked by the ReLU of the previous pre-activation
       CTOF_TRY(conv(cur, 0, L->d_wb + (size_t)l * 27 * CH * CH, nullptr, pre[l], nxt, G, st));
       __nv_bfloat16* t = cur;
