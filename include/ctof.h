@@ -360,7 +360,8 @@ ctof_status ctof_kernel_get_tuning(ctof_kernel k, int* h_pb4);
  * first product alone, then `refine_steps` steps of
  * x += C (b - (G + lambda I) x) with C = (G + lambda I)^-1 from the FP64
  * Cholesky factor, those products in TF32 hi/lo on the tensor cores
- * (FP32-level).  CTOF_FP32: the plain FP32 per-volume path
+ * (FP32-level); with two or more steps and lambda_rel >= 1e-5 the first step is
+ * formed as C b, which differs from it by the rounding of C.  CTOF_FP32: the plain FP32 per-volume path
  * (ctof_reconstruct with CTOF_SOLVER_TIKHONOV) for comparison.
  * lambda = lambda_rel * gram_max_diag; *lambda_out (optional) receives it.
  * The first BF16 / FP8 call for a lambda makes C, G + lambda I and their

@@ -863,7 +863,8 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
     k_batch_tikhonov_ws(const __grid_constant__ CUtensorMap mmap, const __grid_constant__ CUtensorMap wmap, WsPlan P,
                         const unsigned char* __restrict__ tabs, const float* __restrict__ class_scale,
                         const int* __restrict__ members, int nclass, const float2* __restrict__ m_hat, int ldm,
-                        float2* __restrict__ x_hat, int ldx, int refine, int* flag, long long max_polls) {
+                        float2* __restrict__ x_hat, int ldx, int refine, int closed, int* flag,
+                        long long max_polls) {
   extern __shared__ float4 ws_smem4[];
   unsigned char* sm;
   {
@@ -1097,6 +1098,16 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
       umma::fence_after_sync();
       return !ws_sync_or(2, WS_EPI * 32, !w_ok);
     };
+    // b of 16 depths: the accumulated products of all terms
+    auto load_b = [&](uint32_t acc, int j, float sn, float (&out)[16]) {
+      float d1[16], d2[16];
+      umma::tmem_ld16(trow + acc + 16 * j, out);
+      umma::tmem_ld16(trow + acc + zn + 16 * j, d1);
+      if (P.fp8) umma::tmem_ld16(trow + acc + 2 * zn + 16 * j, d2);
+#pragma unroll
+      for (int e = 0; e < 16; ++e)
+        out[e] = P.fp8 ? sn * (out[e] + 0.0625f * d1[e] + 0.00390625f * d2[e]) : out[e] + d1[e];
+    };
     int it = 0, ci = 0;
     bool ok = true;
     for (int c = blockIdx.x; c < nclass && ok; c += gridDim.x, ++ci) {
@@ -1116,14 +1127,21 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
         const uint32_t acc = (uint32_t)(a * acc_cols);
         const float sn = P.fp8 ? reinterpret_cast<const float*>(sm + P.off_sn)[a * NR + n] * sw : 1.f;
         float x[4][16];
-        // x0 = C b0
+        // x0 = C b0, or with `closed` the first refinement step at once:
+        // x0 + C (b - G' x0) = C b + (I - C G') x0 differs from C b by the inverse's
+        // rounding, which the remaining steps square away; three dependent products
+        // (the longest chain of this kernel) instead of five for two steps.
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           if (16 * j < zn) {
             float val[16];
-            umma::tmem_ld16(trow + acc + 16 * j, val);
+            if (closed) {
+              load_b(acc, j, sn, val);
+            } else {
+              umma::tmem_ld16(trow + acc + 16 * j, val);
 #pragma unroll
-            for (int e = 0; e < 16; ++e) val[e] *= sn;
+              for (int e = 0; e < 16; ++e) val[e] *= sn;
+            }
             put_x16(xh, xl, n, j, val);
           }
         }
@@ -1134,7 +1152,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
 #pragma unroll
         for (int j = 0; j < 4; ++j)
           if (16 * j < zn) umma::tmem_ld16(trow + col_work + 16 * j, x[j]);
-        for (int r = 0; r < refine && ok; ++r) {
+        for (int r = closed; r < refine && ok; ++r) {
           // r = b - G' x
 #pragma unroll
           for (int j = 0; j < 4; ++j)
@@ -1146,17 +1164,11 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
             if (16 * j < zn) {
-              float gx[16], d0[16], d1[16], d2[16];
+              float gx[16], rr[16];
               umma::tmem_ld16(trow + col_work + 16 * j, gx);
-              umma::tmem_ld16(trow + acc + 16 * j, d0);
-              umma::tmem_ld16(trow + acc + zn + 16 * j, d1);
-              if (P.fp8) umma::tmem_ld16(trow + acc + 2 * zn + 16 * j, d2);
-              float rr[16];
+              load_b(acc, j, sn, rr);
 #pragma unroll
-              for (int e = 0; e < 16; ++e) {
-                const float bb = P.fp8 ? sn * (d0[e] + 0.0625f * d1[e] + 0.00390625f * d2[e]) : d0[e] + d1[e];
-                rr[e] = bb - gx[e];
-              }
+              for (int e = 0; e < 16; ++e) rr[e] -= gx[e];
               put_x16(xh, xl, n, j, rr);
             }
           }
@@ -1176,6 +1188,8 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
           }
         }
         if (!ok) break;
+        // every solve MMA of this class has completed: the next class's tables may land
+        if (vc == nvc - 1 && et == 0 && c + (int)gridDim.x < nclass) load_tables(c + gridDim.x);
         // the accumulators are read: the MMAs of item it + 2 may overwrite them
         umma::fence_before_sync();
         __syncwarp();
@@ -1198,8 +1212,6 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
           }
         }
       }
-      // every solve MMA of this class has completed: the tables may be replaced
-      if (ok && et == 0 && c + (int)gridDim.x < nclass) load_tables(c + gridDim.x);
     }
     if (et == 0 && tab_loads) bulk::wait(tab_full, (uint32_t)(tab_loads - 1) & 1u, DRAIN_POLLS);
   }
@@ -1374,9 +1386,15 @@ ctof_status batch_tikhonov_contract(const ctof_kernel_s* k, int precision, int b
       if (ctof_encode_map(&mmap, 8, 4, m_hat, mdims, mstr, mbox, 128) == CTOF_OK &&
           ctof_encode_map(&wmap, 4, 2, k->d_what, wdims, wstr, wbox, 128) == CTOF_OK) {
         auto kern = k_batch_tikhonov_ws<32>;
+        // |I - C G'| is ~5e-6 at lambda = 1e-3 of the largest Gram diagonal and grows as its
+        // inverse: from 1e-5 on its square stays below the split's own error (measured against
+        // 64 bits at 24 to 64 depths, BF16 / FP8, both ways: 2e-5 / 1e-4 at 1e-3, 1e-3 / 4e-3 at
+        // 1e-5).  A single step keeps the start from b0.  861 -> 651 us (BF16, 16 volumes of
+        // 128 x 128 x 64, 80 planes), 328 -> 264 us (FP8, 21 of 64 x 64 x 32).
+        const int closed = refine >= 2 && k->bt_lambda >= 1e-5 * k->gram_max;
         CTOF_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, W.total));
         kern<<<grid, WS_THREADS, W.total, st>>>(mmap, wmap, W, k->d_bt_tab, k->d_bt_sw, k->d_members, k->nclass,
-                                                m_hat, ldm, x_hat, ldx, refine, k->d_flags, k->max_polls);
+                                                m_hat, ldm, x_hat, ldx, refine, closed, k->d_flags, k->max_polls);
         CTOF_CUDA_TRY(cudaGetLastError());
         return CTOF_OK;
       }
