@@ -493,16 +493,20 @@ __global__ void __launch_bounds__(TC_THREADS, 2) k_contract_tc_adj(TcPlan P, con
 // n = 32 m + 16 c + v (member, real / imaginary, volume).  Warp 0 (one
 // thread) stages each chunk of 32 t with tensor-map copies (per member one
 // box of 2 halves x 16 volumes x 16 t of r_hat [v][f][t], two W_hat boxes of
-// 32 t x 32 z; 128-byte swizzle) into AW_STAGES raw stages; warps 1-8 split a
+// 32 t x 32 z; 128-byte swizzle) into AW_STAGES raw stages; warps 1-16 split a
 // staged chunk into TF32 high parts and FP32 remainders in the K-major
-// layout (as many term sets as raw stages); warp 9 (one thread) issues three
-// MMAs per K = 8 step into one of two TMEM accumulators; warps 12-15 write
+// layout (as many term sets as raw stages; the split is a
+// chain of waits, shared-memory reads, arithmetic and writes: sixteen warps, so
+// that each thread has one group of four t per chunk; 624 -> 506 us per launch at
+// 16 volumes of 128 x 128 x 48 x 256 against eight warps, 566 us with two groups of
+// eight on alternate chunks); warp 17 (one thread) issues three
+// MMAs per K = 8 step into one of two TMEM accumulators; warps 20-23 write
 // the finished item out.  mbarrier hand-offs; every wait is bounded, a wait
 // that runs out sets the handle's flag and a shared abort word and every
 // role leaves its loop.
-constexpr int AW_CONV = 8;
-constexpr int AW_MMA_WARP = 9;
-constexpr int AW_EPI0 = 12;
+constexpr int AW_CONV = 16;
+constexpr int AW_MMA_WARP = 17;
+constexpr int AW_EPI0 = 20;
 constexpr int AW_THREADS = (AW_EPI0 + 4) * 32;
 constexpr int AW_STAGES = 3;
 constexpr int AW_MBOX = 16 * 16 * 8;  // r_hat box of one member and one 16-t half
@@ -558,13 +562,14 @@ __device__ __forceinline__ bool aw_wait_warp(uint64_t* bar, uint32_t parity, lon
 // Split one staged chunk (converter thread ct of 256): A rows n (K = t) and
 // B = W^T rows z (K = t), TF32 high part and FP32 remainder each.
 __device__ __forceinline__ void aw_convert(const AwPlan& P, const unsigned char* raw, unsigned char* set,
-                                           const int (&mem)[4], int ct) {
+                                           const int (&mem)[4], int ct, int bz, int bg) {
   unsigned char* ahi = set;
   unsigned char* alo = set + P.a_term;
   unsigned char* bhi = set + 2 * P.a_term;
   unsigned char* blo = bhi + P.b_term;
-  for (int i = ct; i < 64 * (TCH / 4); i += AW_CONV * 32) {
-    const int v = i & 15, m = (i >> 4) & 3, gI = i >> 6;  // 4 t values 4 gI ..
+  static_assert(AW_CONV * 32 == 64 * (TCH / 4), "one group of four t per thread and chunk");
+  {
+    const int v = ct & 15, m = (ct >> 4) & 3, gI = ct >> 6;  // 4 t values 4 gI ..
     const int nre = 32 * m + v, nim = nre + 16;
     const uint32_t o_re = umma::kmajor_off(NR, nre, 4 * gI), o_im = umma::kmajor_off(NR, nim, 4 * gI);
     float4 re = make_float4(0.f, 0.f, 0.f, 0.f), im = re;
@@ -592,8 +597,8 @@ __device__ __forceinline__ void aw_convert(const AwPlan& P, const unsigned char*
     *reinterpret_cast<float4*>(alo + o_im) = l;
   }
   const unsigned char* rw = raw + 8 * AW_MBOX;
-  for (int i = ct; i < P.zn * (TCH / 4); i += AW_CONV * 32) {
-    const int z = i % P.zn, gI = i / P.zn;
+  if (bg < TCH / 4) {  // zn (TCH / 4) <= 512: at most one group of W per thread
+    const int z = bz, gI = bg;
     const unsigned char* box = rw + (z >> 5) * AW_WBOX + (z & 3) * 4;
     const int zc = (z & 31) >> 2;
     float w[4];
@@ -690,7 +695,7 @@ __global__ void __launch_bounds__(AW_THREADS, 1)
     }
   } else if (warp <= AW_CONV) {
     // ---------------- converters ----------------
-    const int ct = threadIdx.x - 32;
+    const int ct = threadIdx.x - 32, bg = ct / P.zn, bz = ct - bg * P.zn;
     int gk = 0;
     bool ok = true;
     for (int c = blockIdx.x; c < nclass && ok; c += gridDim.x) {
@@ -706,7 +711,7 @@ __global__ void __launch_bounds__(AW_THREADS, 1)
             ok = false;
             break;
           }
-          aw_convert(P, sm + P.off_raw + s * P.raw_stage, sm + P.off_set + s * P.set_bytes, mem, ct);
+          aw_convert(P, sm + P.off_raw + s * P.raw_stage, sm + P.off_set + s * P.set_bytes, mem, ct, bz, bg);
           umma::fence_proxy_async();  // this lane's term writes, before the MMAs read them
           __syncwarp();
           if (lane == 0) {
