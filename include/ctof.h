@@ -344,7 +344,7 @@ ctof_status ctof_kernel_autotune(ctof_kernel k, void* stream);
 
 /* The tuned tiles [T-side forward, T-side inverse, Z-side forward, Z-side
  * inverse] as tile codes: 8 / 16 = 32-column tiles of that many planes,
- * 108 / 116 = 16-column tiles of 8 / 16 planes; EUNSUPPORTED (defaults 16
+ * 108 / 116 = 16-column tiles of 8 / 16 planes; EUNSUPPORTED (defaults 116
  * reported) if not tuned yet. */
 ctof_status ctof_kernel_get_tuning(ctof_kernel k, int* h_pb4);
 

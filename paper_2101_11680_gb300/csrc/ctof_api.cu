@@ -688,7 +688,7 @@ ctof_status build_any(const ctof_optics* optics, const ctof_emission* emission, 
   k->tik_lambda[0] = k->tik_lambda[1] = -1.0;
   k->tik_last = 1;
   k->max_polls = CTOF_DEFAULT_MAX_POLLS;
-  for (int i = 0; i < 4; ++i) k->tune_pb[i] = 16;
+  for (int i = 0; i < 4; ++i) k->tune_pb[i] = 116;  // untuned: see tile_of in fft.cu
 
   std::vector<int> members;
   std::vector<float> lap;
@@ -1007,9 +1007,12 @@ ctof_status ctof_kernel_autotune(ctof_kernel k, void* stream) {
   if (!k) return CTOF_EINVAL;
   DeviceGuard g(k->device);
   if (!g.ok) return CTOF_ECUDA;
-  k = ctof_ops(k);
-  k->tuned = 0;
-  return autotune(k, static_cast<cudaStream_t>(stream));
+  for (ctof_kernel_s* o : {k, k->tz}) {
+    if (!o) continue;
+    o->tuned = 0;
+    CTOF_TRY(autotune(o, static_cast<cudaStream_t>(stream)));
+  }
+  return CTOF_OK;
 }
 
 ctof_status ctof_kernel_get_tuning(ctof_kernel k, int* h_pb4) {
