@@ -141,20 +141,44 @@ def _check(status, where):
         raise CtofError(status, where)
 
 
+_torch = None
+_raw_stream = None  # current stream handle of a device, without building a Stream object (8 us of a 27 us call)
+
+
+def _t():
+    """The torch module (imported on first use: the binding itself needs no torch)."""
+    global _torch, _raw_stream
+    if _torch is None:
+        import torch
+        _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        _torch = torch
+    return _torch
+
+
 def _stream_handle(stream):
-    import torch
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    torch = _torch or _t()
+    if _raw_stream is None or not torch.cuda.is_initialized():
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(torch.cuda.current_device())
 
 
 def _dev_ptr(t, shape, name):
-    import torch
+    torch = _torch or _t()
     if not isinstance(t, torch.Tensor) or not t.is_cuda or t.dtype != torch.float32 or not t.is_contiguous():
         raise TypeError(f"{name} must be a contiguous float32 CUDA tensor")
-    if tuple(t.shape) != tuple(shape):
+    if t.shape != shape:
         raise ValueError(f"{name} has shape {tuple(t.shape)}, expected {tuple(shape)}")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
+
+
+def _out(out, like, shape):
+    """`out`, or a new float32 tensor of that shape where `like` is."""
+    if out is None:
+        torch = _torch or _t()
+        return torch.empty(shape, device=like.device, dtype=torch.float32)
+    return out
 
 
 def make_optics(mua=0.01, musp=1.0, n=1.4, z0=0.0, clamp_r=True):
@@ -285,8 +309,8 @@ def reconstruct_batch(kernels, ms, params, outs=None, stream=None):
     if outs is None:
         outs = [torch.empty(k._vol_shape(), device=m.device, dtype=torch.float32) for k, m in zip(kernels, ms)]
     hs = (ctypes.c_void_p * n)(*[k._h.value for k in kernels])
-    mp = (ctypes.c_void_p * n)(*[_dev_ptr(m, k._meas_shape(), "m").value for k, m in zip(kernels, ms)])
-    op = (ctypes.c_void_p * n)(*[_dev_ptr(o, k._vol_shape(), "out").value for k, o in zip(kernels, outs)])
+    mp = (ctypes.c_void_p * n)(*[_dev_ptr(m, k._meas_shape(), "m") for k, m in zip(kernels, ms)])
+    op = (ctypes.c_void_p * n)(*[_dev_ptr(o, k._vol_shape(), "out") for k, o in zip(kernels, outs)])
     _check(lib.ctof_reconstruct_batch(n, hs, mp, ctypes.byref(params), op, _stream_handle(stream)),
            "ctof_reconstruct_batch")
     return outs
@@ -324,6 +348,8 @@ class Kernel:
         info = KernelInfo()
         _check(lib.ctof_kernel_get_info(h, ctypes.byref(info)), "ctof_kernel_get_info")
         self.info = info
+        self._vol = (grid.nz, grid.ny, grid.nx)
+        self._meas = (grid.nt, grid.ny, grid.nx)
 
     @property
     def n(self):
@@ -393,18 +419,15 @@ class Kernel:
 
     # ---- operators ----
     def _vol_shape(self):
-        return (self.grid.nz, self.grid.ny, self.grid.nx)
+        return self._vol
 
     def _meas_shape(self):
-        return (self.grid.nt, self.grid.ny, self.grid.nx)
+        return self._meas
 
     def forward(self, mu, out=None, stream=None):
-        import torch
-        if out is None:
-            out = torch.empty(self._meas_shape(), device=mu.device, dtype=torch.float32)
-        _check(self._lib.ctof_forward(self._h, _dev_ptr(mu, self._vol_shape(), "mu"),
-                                      _dev_ptr(out, self._meas_shape(), "out"), _stream_handle(stream)),
-               "ctof_forward")
+        out = _out(out, mu, self._meas)
+        _check(self._lib.ctof_forward(self._h, _dev_ptr(mu, self._vol, "mu"), _dev_ptr(out, self._meas, "out"),
+                                      _stream_handle(stream)), "ctof_forward")
         return out
 
     def forward_static(self, mu, out, stream=None):
@@ -420,12 +443,9 @@ class Kernel:
         return out
 
     def adjoint(self, m, out=None, stream=None):
-        import torch
-        if out is None:
-            out = torch.empty(self._vol_shape(), device=m.device, dtype=torch.float32)
-        _check(self._lib.ctof_adjoint(self._h, _dev_ptr(m, self._meas_shape(), "m"),
-                                      _dev_ptr(out, self._vol_shape(), "out"), _stream_handle(stream)),
-               "ctof_adjoint")
+        out = _out(out, m, self._vol)
+        _check(self._lib.ctof_adjoint(self._h, _dev_ptr(m, self._meas, "m"), _dev_ptr(out, self._vol, "out"),
+                                      _stream_handle(stream)), "ctof_adjoint")
         return out
 
     def forward_multiplexed(self, mu, out=None, stream=None):
@@ -482,12 +502,10 @@ class Kernel:
         return out
 
     def reconstruct(self, m, params, out=None, report=False, stream=None):
-        import torch
-        if out is None:
-            out = torch.empty(self._vol_shape(), device=m.device, dtype=torch.float32)
-        rep = Report()
-        _check(self._lib.ctof_reconstruct(self._h, _dev_ptr(m, self._meas_shape(), "m"), ctypes.byref(params),
-                                          _dev_ptr(out, self._vol_shape(), "out"),
+        out = _out(out, m, self._vol)
+        rep = Report() if report else None
+        _check(self._lib.ctof_reconstruct(self._h, _dev_ptr(m, self._meas, "m"), ctypes.byref(params),
+                                          _dev_ptr(out, self._vol, "out"),
                                           ctypes.byref(rep) if report else None, _stream_handle(stream)),
                "ctof_reconstruct")
         return (out, rep) if report else out
