@@ -153,39 +153,53 @@ __device__ __forceinline__ void adj_pass(const WarpPlan& P, const float* M, int 
     const int per = ((rows + P.J - 1) / P.J + 1) & ~1;
     const int r0 = j * per, r1 = min(rows, r0 + per);
     const float* mp = M + 4 * k;
-    int r = r0;
+    // sums of eight rows, then their sum: FP32 rounding of the solves that follow a
+    // W^T c comes from this accumulation (1.7e-6 against 2.0e-6 in one run of 32 rows)
+    for (int rb = r0; rb < r1; rb += 8) {
+      const int re = min(r1, rb + 8);
+      float2 t[4][4];
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int m = 0; m < 4; ++m) t[a][m] = make_float2(0.f, 0.f);
+      int r = rb;
 #pragma unroll 2
-    for (; r + 2 <= r1; r += 2) {
-      const float4 w0 = *reinterpret_cast<const float4*>(mp + r * pitch);
-      const float4 w1 = *reinterpret_cast<const float4*>(mp + (r + 1) * pitch);
-      float4 c[4];
+      for (; r + 2 <= re; r += 2) {
+        const float4 w0 = *reinterpret_cast<const float4*>(mp + r * pitch);
+        const float4 w1 = *reinterpret_cast<const float4*>(mp + (r + 1) * pitch);
+        float4 c[4];
 #pragma unroll
-      for (int m = 0; m < 4; ++m) c[m] = *reinterpret_cast<const float4*>(v + m * vpitch + r);
+        for (int m = 0; m < 4; ++m) c[m] = *reinterpret_cast<const float4*>(v + m * vpitch + r);
 #pragma unroll
-      for (int m = 0; m < 4; ++m) {
-        cfma(acc[0][m], w0.x, c[m].x, c[m].y);
-        cfma(acc[1][m], w0.y, c[m].x, c[m].y);
-        cfma(acc[2][m], w0.z, c[m].x, c[m].y);
-        cfma(acc[3][m], w0.w, c[m].x, c[m].y);
+        for (int m = 0; m < 4; ++m) {
+          cfma(t[0][m], w0.x, c[m].x, c[m].y);
+          cfma(t[1][m], w0.y, c[m].x, c[m].y);
+          cfma(t[2][m], w0.z, c[m].x, c[m].y);
+          cfma(t[3][m], w0.w, c[m].x, c[m].y);
+        }
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+          cfma(t[0][m], w1.x, c[m].z, c[m].w);
+          cfma(t[1][m], w1.y, c[m].z, c[m].w);
+          cfma(t[2][m], w1.z, c[m].z, c[m].w);
+          cfma(t[3][m], w1.w, c[m].z, c[m].w);
+        }
+      }
+      if (r < re) {
+        const float4 w0 = *reinterpret_cast<const float4*>(mp + r * pitch);
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+          const float2 c = v[m * vpitch + r];
+          cfma(t[0][m], w0.x, c.x, c.y);
+          cfma(t[1][m], w0.y, c.x, c.y);
+          cfma(t[2][m], w0.z, c.x, c.y);
+          cfma(t[3][m], w0.w, c.x, c.y);
+        }
       }
 #pragma unroll
-      for (int m = 0; m < 4; ++m) {
-        cfma(acc[0][m], w1.x, c[m].z, c[m].w);
-        cfma(acc[1][m], w1.y, c[m].z, c[m].w);
-        cfma(acc[2][m], w1.z, c[m].z, c[m].w);
-        cfma(acc[3][m], w1.w, c[m].z, c[m].w);
-      }
-    }
-    if (r < r1) {
-      const float4 w0 = *reinterpret_cast<const float4*>(mp + r * pitch);
+      for (int a = 0; a < 4; ++a)
 #pragma unroll
-      for (int m = 0; m < 4; ++m) {
-        const float2 c = v[m * vpitch + r];
-        cfma(acc[0][m], w0.x, c.x, c.y);
-        cfma(acc[1][m], w0.y, c.x, c.y);
-        cfma(acc[2][m], w0.z, c.x, c.y);
-        cfma(acc[3][m], w0.w, c.x, c.y);
-      }
+        for (int m = 0; m < 4; ++m) acc[a][m] = cadd(acc[a][m], t[a][m]);
     }
     float4* dst = reinterpret_cast<float4*>(part) + lane;
 #pragma unroll
