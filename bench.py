@@ -159,7 +159,8 @@ def make_inputs(kern, cfg, count, seed0, torch):
 def contract_bytes(info, nz, nt):
     """Algorithmic DRAM bytes of one ADMM x-update contraction launch.
 
-    Per frequency class: W_hat (nt x nz FP32) and H^-1 (nz x nz FP32) read once.
+    nt: the planes of the measurement side (the time bins, or fewer where the
+    kernel is compressed in time).  Per frequency class: W_hat (nt x nz FP32) and H^-1 (nz x nz FP32) read once.
     Per half-plane frequency: c_hat (nt complex64) and s_hat (nz) read, x_hat
     (nz) read and written, K x_hat (nt) written.
     """
@@ -359,7 +360,8 @@ def run_precision(args, cfg):
     info = kern.info
     # algorithmic bytes of one contraction launch: m_hat read, x_hat written, W_hat and the solve tables read
     zn = (cfg["nz"] + 15) // 16 * 16
-    alg = (info.n_freq * bsz * (cfg["nt"] + cfg["nz"]) * 8 + info.n_class * cfg["nt"] * ((cfg["nz"] + 3) // 4 * 4) * 4
+    planes = kern.planes()
+    alg = (info.n_freq * bsz * (planes + cfg["nz"]) * 8 + info.n_class * planes * ((cfg["nz"] + 3) // 4 * 4) * 4
            + info.n_class * 4 * zn * zn * 2)
     line = {"metric": "volumes/sec, batched Tikhonov (precision form)", "value": bsz / (times["bf16"] / 1e3),
             "unit": UNIT, "n_gpus": 1, "steps": args.steps, "warmup": args.warmup,
@@ -825,7 +827,8 @@ def main():
 
     peak, peak_src = _peaks()
     avg_contract_ms = timing.contract_ms / max(1, timing.contract_launches)
-    alg_bytes = contract_bytes(info, cfg["nz"], cfg["nt"])
+    planes = kern.planes()
+    alg_bytes = contract_bytes(info, cfg["nz"], planes)
     achieved = alg_bytes / (avg_contract_ms * 1e-3) / 1e9
     traffic = None
     prof = os.path.join(ROOT, "profiles", "contract_admm_cfg2.json")
@@ -833,14 +836,14 @@ def main():
         try:
             with open(prof) as f:
                 pj = json.load(f)
-            src = open(os.path.join(ROOT, "paper_2101_11680_gb300", "csrc", "contract_admm.cu"), "rb").read()
+            src = open(os.path.join(ROOT, "paper_2101_11680_gb300", "csrc", "contract_warp.cu"), "rb").read()
             import hashlib
             if pj.get("source_sha256") == hashlib.sha256(src).hexdigest():
                 traffic = pj.get("dram_bytes_per_launch")
         except Exception:
             traffic = None
 
-    admm_kernel = "k_contract_admm_pipe" if info.admm_stages else "k_contract_admm"
+    admm_kernel = "k_contract_warp"  # (at these sizes; larger class blocks run k_contract_admm_pipe)
     launches_per_step = timing.graph_kernel_nodes
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
@@ -848,8 +851,8 @@ def main():
         "scaling": "weak", "vs_baseline": None, "dtype": "f32", "data": "synthetic",
         "config": {"workload": cfg["workload"], "n": cfg["n"], "nz": cfg["nz"], "nt": cfg["nt"],
                    "iters": cfg["iters"], "parallelism": "replicas" if world > 1 else "single",
-                   "l2": "inputs larger than L2 (W_hat %.0f MB streamed per iteration)"
-                         % (info.n_class * cfg["nt"] * cfg["nz"] * 4 / 1e6),
+                   "l2": "inputs larger than L2 (x-update reads and writes %.0f MB per iteration, %d planes)"
+                         % (alg_bytes / 1e6, planes),
                    "kernel": kernel_desc, "kernel_build_s": round(build_s, 3)},
         "roofline": {"bound": "hbm", "kernel": admm_kernel, "achieved": achieved, "peak": peak,
                      "unit": "GB/s", "frac": achieved / peak, "traffic": traffic,

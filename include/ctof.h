@@ -98,8 +98,8 @@ typedef struct {
   double scale;     /* max_f sigma_max(W_hat(f)) (the ADMM normalisation) */
   double gram_max_diag; /* max over f, j of (W_hat^T W_hat)_jj */
   size_t device_bytes;  /* device memory held by the handle */
-  int admm_stages;      /* shared-memory stages of the pipelined ADMM x-update
-                           kernel at this size (0: the fallback kernel runs) */
+  int admm_stages;      /* shared-memory stages of the ADMM x-update kernel at
+                           this size (0: the fallback kernel runs) */
 } ctof_kernel_info;
 
 /* Solver choice and parameters.  ADMM_TV solves
@@ -203,6 +203,12 @@ ctof_status ctof_build_kernel_ex(const ctof_optics* optics, const ctof_emission*
 void ctof_kernel_destroy(ctof_kernel k);
 
 ctof_status ctof_kernel_get_info(ctof_kernel k, ctof_kernel_info* info);
+
+/* Planes that the solvers' measurement side works on: nt, or fewer where the
+ * handle's kernel was compressed in time (its rows over the nt bins span that
+ * many directions; the factorisation is checked at build time to 2e-8 of each
+ * bin's response and results keep FP32 accuracy bin by bin). */
+ctof_status ctof_kernel_get_planes(ctof_kernel k, int* planes);
 
 /* Copy the FP64 kernel table W[nt][nz][ny][nx] (non-negative offsets |oy|, |ox|;
  * for circular mode the table is [nt][nz][P/2+1][P/2+1]) to host memory.

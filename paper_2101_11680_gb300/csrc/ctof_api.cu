@@ -829,6 +829,12 @@ ctof_status ctof_kernel_get_info(ctof_kernel k, ctof_kernel_info* info) {
   return CTOF_OK;
 }
 
+ctof_status ctof_kernel_get_planes(ctof_kernel k, int* planes) {
+  if (!k || !planes) return CTOF_EINVAL;
+  *planes = ctof_ops(k)->nt;
+  return CTOF_OK;
+}
+
 ctof_status ctof_kernel_get_w(ctof_kernel k, double* h_w) {
   if (!k || !h_w) return CTOF_EINVAL;
   if (!k->d_w) return CTOF_EUNSUPPORTED;

@@ -83,6 +83,7 @@ _SIGNATURES = {
                                             _P, ctypes.POINTER(_P)]),
     "ctof_kernel_destroy": (None, [_P]),
     "ctof_kernel_get_info": (ctypes.c_int, [_P, ctypes.POINTER(KernelInfo)]),
+    "ctof_kernel_get_planes": (ctypes.c_int, [_P, ctypes.POINTER(ctypes.c_int)]),
     "ctof_kernel_get_w": (ctypes.c_int, [_P, _P]),
     "ctof_kernel_get_classes": (ctypes.c_int, [_P, _P]),
     "ctof_kernel_get_what": (ctypes.c_int, [_P, _P]),
@@ -394,6 +395,12 @@ class Kernel:
         out = (ctypes.c_int * 4)()
         self._lib.ctof_kernel_get_tuning(self._h, out)
         return list(out)
+
+    def planes(self):
+        """Planes that the solvers' measurement side works on (nt, or fewer with time compression)."""
+        out = ctypes.c_int()
+        _check(self._lib.ctof_kernel_get_planes(self._h, ctypes.byref(out)), "ctof_kernel_get_planes")
+        return out.value
 
     # ---- parity accessors (synchronous) ----
     def get_w(self):
