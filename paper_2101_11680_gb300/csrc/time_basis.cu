@@ -594,8 +594,11 @@ void time_basis_free(ctof_kernel_s* k) {
 ctof_status time_compress(const ctof_kernel_s* z, int batch, const float* m, float* out, cudaStream_t st) {
   const int npix = z->n * z->n;
   const bool bulk = npix % 4 == 0 && (reinterpret_cast<uintptr_t>(m) & 15) == 0;  // (`out` is the library's own)
-  // at G = 1 a CTA takes 512 points of a window: four groups per CTA while those do not fill the chip twice over
-  const bool few = (long long)ctof_div_up(npix, CB_PIX) * z->tz_nwin * batch < 2 * 3 * 152;
+  // At G = 1 a CTA takes 512 points of a window: four groups per CTA while there are fewer than two of those per SM.
+  // us per call, G = 4 / G = 1: adjoint 64^2 x 48 x 256 (56 CTAs at G = 1) 47.7 / 56.0, 128^2 x 48 x 256 (about 220)
+  // 85.6 / 92.8; batched Tikhonov 16 x 64^2 x 32 x 128 (about 500) 228 / 223, 4 x 128^2 x 48 x 256 586 / 578,
+  // 16 x 128^2 x 64 x 512 1207 / 1115.
+  const bool few = (long long)ctof_div_up(npix, CB_PIX) * z->tz_nwin * batch < 2 * 152;
   auto kern = few ? k_compress_bulk<4> : k_compress_bulk<1>;
   const int smem = few ? cb_smem(4) : cb_smem(1), tile = few ? CB_PIX / 4 : CB_PIX;
   CTOF_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));

@@ -82,3 +82,18 @@ def test_solvers(problem):
     assert rel_l2(k.reconstruct(md, ctof.tikhonov_params()).cpu().numpy(), so.tikhonov(wh, m, g)[0]) <= 1e-5 * scale
     assert rel_l2(k.reconstruct(md, ctof.admm_params(8)).cpu().numpy(), so.admm(wh, m, g, 8)[0]) <= 1e-5
     assert rel_l2(k.reconstruct(md, ctof.fista_params(10)).cpu().numpy(), so.fista_l1(wh, m, g, 10)[0]) <= 1e-5
+
+
+@pytest.mark.parametrize("volumes", [1, 64])
+def test_projection_groups(problem, volumes):
+    """Batched Tikhonov with few and with many projection CTAs, at the precision form's stated 1e-3."""
+    g, wh, k = problem
+    rng = np.random.default_rng(6)
+    mu = rng.uniform(0.0, 0.02, (2, g.nz, g.n, g.n)) * (rng.uniform(size=(2, g.nz, g.n, g.n)) < 0.1)
+    ms = np.stack([op.forward_fft(wh, x, g) for x in mu])
+    md = torch.tensor(ms, dtype=torch.float32, device="cuda")
+    got = k.reconstruct_batch_tikhonov(md[[0] * (volumes - 1) + [1]].contiguous(), precision=ctof.BF16)[0]
+    want = [so.tikhonov(wh, m, g)[0] for m in ms]
+    assert rel_l2(got[-1].cpu().numpy(), want[1]) <= 1e-3
+    for b in range(0, volumes - 1, 9):
+        assert rel_l2(got[b].cpu().numpy(), want[0]) <= 1e-3
