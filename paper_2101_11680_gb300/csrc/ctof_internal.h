@@ -126,9 +126,12 @@ inline ctof_kernel_s* ctof_ops(ctof_kernel_s* k) { return k->tz ? k->tz : k; }
 inline const ctof_kernel_s* ctof_ops(const ctof_kernel_s* k) { return k->tz ? k->tz : k; }
 
 // The operator that a single application (forward, adjoint, one Tikhonov
-// solve) runs on: the projection is a launch of its own, so the T-side
-// spectrum that it saves has to be large.
-constexpr size_t TZ_ONE_SHOT_BYTES = (size_t)8 << 20;
+// solve) runs on: the projection or expansion is a launch of its own, so the
+// T-side spectrum that it saves has to be large.  us per call, planes / bins
+// (saved spectrum): forward 32^2 x 32 x 128 25.2 / 22.2 (1.3 MB), 32^2 x 48 x
+// 256 26.2 / 32.4 (3.1), 64^2 x 32 x 128 35.5 / 42.7 (5.1), 64^2 x 48 x 256
+// 40.6 / 68.3 (12); adjoint 27.3 / 25.2, 31.4 / 34.5, 38.5 / 46.8, 47.7 / 86.7.
+constexpr size_t TZ_ONE_SHOT_BYTES = (size_t)2 << 20;
 inline ctof_kernel_s* ctof_ops_once(ctof_kernel_s* k) {
   return k->tz && (size_t)k->nf * (k->nt - k->tz->nt) * sizeof(float2) >= TZ_ONE_SHOT_BYTES ? k->tz : k;
 }
