@@ -632,7 +632,8 @@ ctof_status admm_copies(ctof_kernel_s* k, cudaStream_t st) {
       if (cudaMalloc(&k->d_admm, k->admm_bytes) != cudaSuccess) {
         cudaGetLastError();
         k->d_admm = nullptr;
-        return CTOF_ENOMEM;
+        k->admm_bytes = 0;
+        return CTOF_OK;  // no room: the kernels that read d_what and d_hinv themselves
       }
       char* b = static_cast<char*>(k->d_admm);
       (warp ? k->d_what_block : k->d_what_admm) = reinterpret_cast<float*>(b + o_w);

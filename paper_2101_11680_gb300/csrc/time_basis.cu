@@ -478,7 +478,7 @@ static int compressed_planes(int nt, int rank) {
   return 2 * rows <= nt ? rows : 0;
 }
 
-ctof_status time_basis_build(ctof_kernel_s* k, const double* what64, cudaStream_t st) {
+static ctof_status make_basis(ctof_kernel_s* k, const double* what64, cudaStream_t st) {
   k->tz = nullptr;
   const int nt = k->nt, nz = k->nz;
   if (compressed_planes(nt, TZ_FIRST) == 0) return CTOF_OK;  // too few bins
@@ -497,8 +497,14 @@ ctof_status time_basis_build(ctof_kernel_s* k, const double* what64, cudaStream_
       if (p) cudaFree(p);
     }
   } d_cls, d_w, d_q, d_worst;
-  CTOF_CUDA_TRY(cudaMalloc(&d_cls.p, cls.size() * sizeof(int)));
-  CTOF_CUDA_TRY(cudaMalloc(&d_w.p, w.size() * sizeof(double)));
+  // device memory that only the compressed operator needs: without it the handle works on the bins
+  auto alloc = [](void** p, size_t bytes) {
+    if (cudaMalloc(p, bytes) == cudaSuccess) return true;
+    cudaGetLastError();
+    *p = nullptr;
+    return false;
+  };
+  if (!alloc(&d_cls.p, cls.size() * sizeof(int)) || !alloc(&d_w.p, w.size() * sizeof(double))) return CTOF_OK;
   CTOF_CUDA_TRY(cudaMemcpyAsync(d_cls.p, cls.data(), cls.size() * sizeof(int), cudaMemcpyHostToDevice, st));
   k_sample_classes<<<152 * 4, 256, 0, st>>>(what64, nt, nz, static_cast<int*>(d_cls.p), ns,
                                             static_cast<double*>(d_w.p));
@@ -541,10 +547,11 @@ ctof_status time_basis_build(ctof_kernel_s* k, const double* what64, cudaStream_
   const size_t o_m = at(off, (size_t)rows * k->n * k->n * sizeof(float));
   z->tz_bytes = off;
   z->d_tz_base = nullptr;
-  if (cudaMalloc(&z->d_tz_base, off) != cudaSuccess) {
-    cudaGetLastError();
+  const size_t qb = b.q.size() * sizeof(double), db = nt * sizeof(double);
+  if (!alloc(&z->d_tz_base, off) || !alloc(&d_q.p, qb + db) || !alloc(&d_worst.p, sizeof(unsigned long long))) {
+    if (z->d_tz_base) cudaFree(z->d_tz_base);
     delete z;
-    return CTOF_ENOMEM;
+    return CTOF_OK;
   }
   k->tz = z;  // freed with the handle from here on
   char* base = static_cast<char*>(z->d_tz_base);
@@ -561,9 +568,6 @@ ctof_status time_basis_build(ctof_kernel_s* k, const double* what64, cudaStream_
   z->tz_nwin = (int)b.win.size();
   z->tz_ntiles = (int)tiles.size();
   z->tz_nt = nt;
-  const size_t qb = b.q.size() * sizeof(double), db = nt * sizeof(double);
-  CTOF_CUDA_TRY(cudaMalloc(&d_q.p, qb + db));
-  CTOF_CUDA_TRY(cudaMalloc(&d_worst.p, sizeof(unsigned long long)));
   double* d_dinv = static_cast<double*>(d_q.p) + b.q.size();
   CTOF_CUDA_TRY(cudaMemcpyAsync(d_q.p, b.q.data(), qb, cudaMemcpyHostToDevice, st));
   CTOF_CUDA_TRY(cudaMemcpyAsync(d_dinv, b.dinv.data(), db, cudaMemcpyHostToDevice, st));
@@ -581,6 +585,14 @@ ctof_status time_basis_build(ctof_kernel_s* k, const double* what64, cudaStream_
   memcpy(&worst, &bits, sizeof(worst));
   if (!(worst <= TZ_CHECK)) time_basis_free(k);
   return CTOF_OK;
+}
+
+ctof_status time_basis_build(ctof_kernel_s* k, const double* what64, cudaStream_t st) {
+  try {
+    return make_basis(k, what64, st);
+  } catch (const std::bad_alloc&) {  // host memory for the fit: the handle works on the bins
+    return CTOF_OK;  // (nothing is allocated on the host once k->tz is set)
+  }
 }
 
 void time_basis_free(ctof_kernel_s* k) {
