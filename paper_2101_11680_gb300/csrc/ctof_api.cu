@@ -980,7 +980,8 @@ ctof_status ctof_reconstruct_batch_tikhonov(ctof_kernel k, int batch, const floa
   k = ctof_ops(k);
   const int ldm = ctof_round_up(batch * k->nt, 8), ldx = ctof_round_up(batch * k->nz, 8);
   const size_t b_sm = (size_t)k->nf * ldm * sizeof(float2), b_sx = (size_t)k->nf * ldx * sizeof(float2);
-  const size_t b_in = (size_t)batch * (k->nt > k->nz ? k->nt : k->nz) * k->n * k->hp * sizeof(float2);
+  // (the row passes pitch their planes to a multiple of 16)
+  const size_t b_in = fft_inter_elems(k, batch * std::max(k->nt, k->nz), k->n) * sizeof(float2);
   const size_t b_fft = ((b_sm + 255) & ~(size_t)255) + ((b_sx + 255) & ~(size_t)255) + ((b_in + 255) & ~(size_t)255);
   const size_t need = b_fft + (tz ? (size_t)batch * k->nt * k->n * k->n * sizeof(float) : 0);
   if (need > k->batch_bytes) {
