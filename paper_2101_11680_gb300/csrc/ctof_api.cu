@@ -976,8 +976,10 @@ ctof_status ctof_reconstruct_batch_tikhonov(ctof_kernel k, int batch, const floa
     }
     return CTOF_OK;
   }
-  const bool tz = k->tz != nullptr;
-  k = ctof_ops(k);
+  // FP8 keeps the time bins: the projection's planes quantise differently, and with few depths that shows
+  // (64-bit error 1.3e-4 on the bins, 1.9e-4 on the planes at 74^2 x 3 x 368; BF16 and FP32 are as good or better on them).
+  const bool tz = k->tz != nullptr && precision != CTOF_FP8E4M3;
+  if (tz) k = k->tz;
   const int ldm = ctof_round_up(batch * k->nt, 8), ldx = ctof_round_up(batch * k->nz, 8);
   const size_t b_sm = (size_t)k->nf * ldm * sizeof(float2), b_sx = (size_t)k->nf * ldx * sizeof(float2);
   // (the row passes pitch their planes to a multiple of 16)
