@@ -1390,7 +1390,7 @@ ctof_status batch_tikhonov_contract(const ctof_kernel_s* k, int precision, int b
         // inverse: from 1e-5 on its square stays below the split's own error (measured against
         // 64 bits at 24 to 64 depths, BF16 / FP8, both ways: 2e-5 / 1e-4 at 1e-3, 1e-3 / 4e-3 at
         // 1e-5).  A single step keeps the start from b0.  861 -> 651 us (BF16, 16 volumes of
-        // 128 x 128 x 64, 80 planes), 328 -> 264 us (FP8, 21 of 64 x 64 x 32).
+        // 128 x 128 x 64, 80 planes), 328 -> 264 us (FP8, 21 of 64 x 64 x 32 at 64 planes).
         const int closed = refine >= 2 && k->bt_lambda >= 1e-5 * k->gram_max;
         CTOF_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, W.total));
         kern<<<grid, WS_THREADS, W.total, st>>>(mmap, wmap, W, k->d_bt_tab, k->d_bt_sw, k->d_members, k->nclass,
