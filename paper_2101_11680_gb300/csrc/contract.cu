@@ -431,21 +431,21 @@ size_t contract_smem_bytes(int nt, int nz) {
   return worst;
 }
 
-// One volume: the one-warp-per-class kernels where the handle has their table,
-// else the CTA-per-class kernel above.
+// One volume: the one-warp-per-class kernels where the handle has their table and
+// the class fits their slots, else the CTA-per-class kernel above.
 ctof_status contract_forward(const ctof_kernel_s* k, const float2* in_z, float2* out_t, cudaStream_t st) {
-  if (k->d_what_pitch) return contract_warp_forward(k, in_z, out_t, st);
+  if (contract_warp_takes(k, WarpCall::Forward)) return contract_warp_forward(k, in_z, out_t, st);
   return contract_forward_batch(k, 1, in_z, out_t, st);
 }
 
 ctof_status contract_adjoint(const ctof_kernel_s* k, const float2* in_t, float2* out_z, cudaStream_t st) {
-  if (k->d_what_pitch) return contract_warp_adjoint(k, in_t, out_z, st);
+  if (contract_warp_takes(k, WarpCall::Adjoint)) return contract_warp_adjoint(k, in_t, out_z, st);
   return contract_adjoint_batch(k, 1, in_t, out_z, st);
 }
 
 ctof_status contract_tikhonov(const ctof_kernel_s* k, const float* hinv, const float2* m_hat, float2* x_hat,
                               cudaStream_t st) {
-  if (k->d_what_pitch) return contract_warp_tikhonov(k, hinv, m_hat, x_hat, st);
+  if (contract_warp_takes(k, WarpCall::Tikhonov)) return contract_warp_tikhonov(k, hinv, m_hat, x_hat, st);
   return contract_tikhonov_batch(k, 1, hinv, m_hat, x_hat, st);
 }
 

@@ -681,6 +681,15 @@ ctof_status launch(const ctof_kernel_s* k, const WarpPlan& P, WarpArgs& A, cudaS
 
 }  // namespace
 
+// Each mode has sizes of its own: rows at the odd pitch and the partials of an adjoint pass take more
+// room than the x-update's blocks (8 depths: the x-update fits to 688 planes, the adjoint to 535, the
+// Tikhonov solve to 528).  Where a mode has no room, the CTA-per-class kernel takes the call.
+bool contract_warp_takes(const ctof_kernel_s* k, WarpCall call) {
+  WarpPlan P;
+  const int mode = call == WarpCall::Forward ? WM_FWD : call == WarpCall::Adjoint ? WM_ADJ : WM_TIK;
+  return k->d_what_pitch && choose_plan(mode, k->nt, k->nz, &P);
+}
+
 int contract_warp_slots(int nt, int nz) {
   WarpPlan P;
   return choose_plan(WM_ADMM, nt, nz, &P) ? P.ns : 0;

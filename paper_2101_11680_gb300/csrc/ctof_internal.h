@@ -267,6 +267,9 @@ ctof_status contract_admm_prepare(ctof_kernel_s* k, cudaStream_t st);
 size_t contract_warp_floats(int nt, int nz, int which);
 int contract_warp_slots(int nt, int nz);
 ctof_status contract_warp_prepare(const ctof_kernel_s* k, cudaStream_t st);
+// Whether the handle's copies are there and a class of this call fits the kernel's slots.
+enum class WarpCall { Forward, Adjoint, Tikhonov };
+bool contract_warp_takes(const ctof_kernel_s* k, WarpCall call);
 ctof_status contract_warp_forward(const ctof_kernel_s* k, const float2* in_z, float2* out_t, cudaStream_t st);
 ctof_status contract_warp_adjoint(const ctof_kernel_s* k, const float2* in_t, float2* out_z, cudaStream_t st);
 ctof_status contract_warp_tikhonov(const ctof_kernel_s* k, const float* hinv, const float2* m_hat, float2* x_hat,
