@@ -16,7 +16,11 @@ constexpr int TZ_R = 16;             // columns of one window's basis at most (r
 constexpr int TZ_FIRST = 16;         // bins of the first window
 constexpr double TZ_FALL = 1e-3;     // a window ends where the response has fallen by this factor
 constexpr double TZ_EPS = 1e-10;     // scaled residual at which a window's rank is reached
-constexpr double TZ_FLOOR = 1e-6;    // depths below this share of a bin's response are scaled by it instead
+constexpr double TZ_FLOOR = 1e-30;   // share of a bin's response below which a depth is not looked at (FP32 ends near it)
+constexpr double TZ_OWN = 2e-8;      // residual of a bin and depth relative to its own DC response
+constexpr double TZ_CHECK = 2e-8;    // residual over all classes, relative to a bin's DC response
+constexpr double TZ_CHECK_OWN = 1e-7;  // the same relative to that of the depth in the bin
+constexpr double TZ_CANCEL = 10.0;   // largest sum_j |Q V| / |sum_j Q V| over the bins and depths of a window
 
 inline double dot(const double* a, const double* b, size_t n) {
   double s[4] = {0, 0, 0, 0};
@@ -31,8 +35,80 @@ inline void axpy(double f, const double* x, double* y, size_t n) {
   for (size_t i = 0; i < n; ++i) y[i] += f * x[i];
 }
 
+// Largest cancellation in the products of an orthonormal basis g [r][len]: over
+// bins and depths of the DC class (sample 0), sum_j |g_j v_j| / |w| with v = g w.
+// FP32 rounding of Q and V grows by it.  Infinite where the basis, in FP64, does
+// not give the response back.
+inline double cancellation(const double* w, int nz, size_t cols, const double* d, int a, int len,
+                           const std::vector<double>& g, int r) {
+  double worst = 1.0;
+  std::vector<double> v(r);
+  for (int z = 0; z < nz; ++z) {
+    for (int j = 0; j < r; ++j) {
+      v[j] = 0.0;
+      for (int t = 0; t < len; ++t) v[j] += g[(size_t)j * len + t] * w[(a + t) * cols + z];
+    }
+    for (int t = 0; t < len; ++t) {
+      const double own = w[(a + t) * cols + z];
+      if (!(fabs(own) > TZ_FLOOR * d[a + t])) continue;
+      double sum = 0.0, mag = 0.0;
+      for (int j = 0; j < r; ++j) {
+        const double f = g[(size_t)j * len + t] * v[j];
+        sum += f;
+        mag += fabs(f);
+      }
+      if (!(fabs(sum - own) <= 2.0 * TZ_OWN * fabs(own))) return INFINITY;
+      worst = std::max(worst, mag / fabs(own));
+    }
+  }
+  return worst;
+}
+
+// The same space in an order of bins: basis vector i is zero at the bins that the
+// vectors before it were taken for.  A deep layer's response rises by many decades
+// over the early windows; in the order of size its early bins are the small
+// difference of large products, in the order of time each is its own product.  A bin is
+// taken in turn when what the vectors so far leave of it is above `theta` (smooth
+// neighbours are not), then the largest remainders complete the basis.
+inline std::vector<double> in_time_order(const std::vector<double>& g, int r, int len, double theta) {
+  std::vector<double> u((size_t)r * r), c(r), h((size_t)r * len, 0.0);
+  std::vector<char> used(len, 0);
+  int m = 0;
+  auto remainder = [&](int t) {
+    for (int j = 0; j < r; ++j) c[j] = g[(size_t)j * len + t];
+    for (int pass = 0; pass < 2; ++pass)
+      for (int l = 0; l < m; ++l) axpy(-dot(c.data(), &u[(size_t)l * r], r), &u[(size_t)l * r], c.data(), r);
+    return sqrt(dot(c.data(), c.data(), r));
+  };
+  auto take = [&](int t) {
+    const double nrm = remainder(t);
+    for (int j = 0; j < r; ++j) u[(size_t)m * r + j] = c[j] / nrm;
+    used[t] = 1;
+    ++m;
+  };
+  for (int t = 0; t < len && m < r; ++t)
+    if (remainder(t) >= theta) take(t);
+  while (m < r) {
+    int best = -1;
+    double most = 0.0;
+    for (int t = 0; t < len; ++t) {
+      const double nrm = used[t] ? 0.0 : remainder(t);
+      if (nrm > most) {
+        most = nrm;
+        best = t;
+      }
+    }
+    if (best < 0) return g;
+    take(best);
+  }
+  for (int i = 0; i < r; ++i)
+    for (int j = 0; j < r; ++j) axpy(u[(size_t)i * r + j], &g[(size_t)j * len], &h[(size_t)i * len], len);
+  return h;
+}
+
 // Basis of the rows [a, b) of w [nt][cols] (column z of sample s at s nz + z):
-// q[t - a][j], j < rank; the rank, or -1 when it is above TZ_R.
+// q[t - a][j], j < rank; the rank, or -1 when it is above TZ_R or the products
+// cancel more than TZ_CANCEL.
 inline int window_basis(const double* w, int nz, int ns, const double* d, int a, int b, double* q) {
   const int len = b - a;
   const size_t cols = (size_t)nz * ns;
@@ -68,7 +144,21 @@ inline int window_basis(const double* w, int nz, int ns, const double* d, int a,
         piv = t;
       }
     }
-    if (!(top >= TZ_EPS)) break;
+    if (!(top >= TZ_EPS)) {  // in the window's scale; then every bin and depth in its own
+      double over = TZ_OWN;
+      piv = -1;
+      for (int t = 0; t < len; ++t)
+        for (size_t i = 0; i < n; ++i) {
+          const int z = (int)(idx[i] % nz);
+          const double own = std::max(fabs(w[(a + t) * cols + z]) / d[a + t], TZ_FLOOR);
+          const double rel = fabs(res[t * n + i]) * cz[z] / own;
+          if (rel > over) {
+            over = rel;
+            piv = t;
+          }
+        }
+      if (piv < 0) break;
+    }
     if (r == TZ_R) return -1;
     std::vector<double> x(res.begin() + piv * n, res.begin() + (piv + 1) * n);
     for (int pass = 0; pass < 2; ++pass)
@@ -95,8 +185,20 @@ inline int window_basis(const double* w, int nz, int ns, const double* d, int a,
       if (!(nrm > 0.0) || !isfinite(nrm)) return -1;
       for (int t = 0; t < len; ++t) g[j * len + t] /= nrm;
     }
-    for (int t = 0; t < len; ++t) q[t * TZ_R + j] = g[j * len + t];
   }
+  double least = cancellation(w, nz, cols, d, a, len, g, r);
+  std::vector<double> pick = g;
+  for (double theta : {0.7, 0.5, 0.25, 0.1}) {
+    std::vector<double> h = in_time_order(g, r, len, theta);
+    const double c = cancellation(w, nz, cols, d, a, len, h, r);
+    if (c < least) {
+      least = c;
+      pick.swap(h);
+    }
+  }
+  if (!(least <= TZ_CANCEL)) return -1;
+  for (int j = 0; j < r; ++j)
+    for (int t = 0; t < len; ++t) q[t * TZ_R + j] = pick[(size_t)j * len + t];
   return r;
 }
 
@@ -108,7 +210,7 @@ struct Window {
 struct Basis {
   std::vector<double> q;      // [nt][TZ_R]
   std::vector<Window> win;
-  std::vector<double> dinv;   // [nt] 1 / DC response of each bin
+  std::vector<double> tol;    // [nt][nz] largest residual that any class may leave
   int rank = 0;
 };
 
@@ -136,8 +238,11 @@ inline bool fit(const std::vector<double>& w, int nt, int nz, int ns, Basis* out
   }
   std::reverse(todo.begin(), todo.end());
   out->q.assign((size_t)nt * TZ_R, 0.0);
-  out->dinv.resize(nt);
-  for (int t = 0; t < nt; ++t) out->dinv[t] = 1.0 / d[t];
+  out->tol.resize((size_t)nt * nz);
+  for (int t = 0; t < nt; ++t)
+    for (int z = 0; z < nz; ++z)
+      out->tol[(size_t)t * nz + z] =
+          std::min(TZ_CHECK * d[t], TZ_CHECK_OWN * std::max(fabs(w[t * cols + z]), TZ_FLOOR * d[t]));
   while (!todo.empty()) {
     const auto [a, b] = todo.back();
     todo.pop_back();

@@ -7,6 +7,9 @@ import subprocess
 import numpy as np
 import pytest
 
+from oracle import operators as op
+from oracle import physics as ph
+
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2101_11680_gb300", "csrc")
 COLUMNS = 16  # row pitch of the device table
 
@@ -66,3 +69,25 @@ def test_seventeen_bins_of_rank_sixteen(fit, nt):
     assert [32, 49] in win[:, :2].tolist()
     assert win[:, 3].max() <= COLUMNS and rank == win[:, 3].sum()
     assert np.abs(project(w, win, q) - w).max() <= 1e-9
+
+
+@pytest.mark.parametrize("nz,nt,d,dt", [(48, 256, 0.5, 25.0), (64, 512, 0.5, 25.0), (40, 160, 1.0, 50.0)])
+def test_every_bin_and_depth_in_fp32(fit, nz, nt, d, dt):
+    """The stored FP32 factors give every bin of every depth's DC response back, also where a deep layer's response
+    rises by many decades within a window.  The products may cancel by 10; Q, V and their sum round to 6e-8 each."""
+    g = op.Grid(8, nz, nt, d, d, d, dt)
+    wh = op.kernel_spectrum(op.kernel_offsets(g, ph.Medium(0.01, 1.0, 1.4, r_min=0.5 * d)), g)
+    w = np.ascontiguousarray(np.moveaxis(wh.real.reshape(nt, nz, -1), 2, 1)[:, ::5])
+    win, q, rank = fit(w)
+    assert win[-1, 1] == nt and rank == win[:, 3].sum()
+    assert 2 * rank <= nt
+    dc = w[:, 0]
+    for a, b, _, r in win:
+        qs = q[a:b, :r].astype(np.float32)
+        assert np.abs(q[a:b, :r].T @ q[a:b, :r] - np.eye(r)).max() <= 1e-12
+        v = (q[a:b, :r].T @ dc[a:b]).astype(np.float32)
+        got = np.zeros((b - a, nz), dtype=np.float32)
+        for j in range(r):
+            got += qs[:, j, None] * v[j]
+        seen = dc[a:b] > 1e-30 * dc[a:b].max(axis=1, keepdims=True)
+        assert (np.abs(got - dc[a:b]) / dc[a:b])[seen].max() <= 10 * 3 * 6e-8
