@@ -11,6 +11,8 @@
 // are split into narrow-format terms whose sum reproduces the FP32 value:
 //
 //   BF16: v = v_hi + v_lo (both BF16); b0 = hi.hi, b = hi.hi + (hi.lo + lo.hi)
+//         (on the planes of a compressed operator v = v_hi + v_lo + v_3 and
+//         the six products down to 2^-16; b0 = b there)
 //   FP8:  v = s (q0 + q1/16 + q2/256), each q an e4m3 value, s a scale that
 //         maps the block's largest magnitude to 448 (per frequency class for
 //         W_hat, per right-hand side for m_hat); products grouped by level:
@@ -150,18 +152,33 @@ __device__ __forceinline__ unsigned pack_bf16x2(float a, float b) {
   return *reinterpret_cast<unsigned*>(&h);
 }
 
-// BF16 split of 8 values into hi / lo 16-byte rows.
-__device__ __forceinline__ void split8_bf16(const float (&v)[8], uint4& hi, uint4& lo) {
+// BF16 split of 8 values into hi / lo 16-byte rows; `rem` receives what they leave.
+__device__ __forceinline__ void split8_bf16(const float (&v)[8], uint4& hi, uint4& lo, float (&rem)[8]) {
   unsigned h[4], l[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const __nv_bfloat162 p = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
     const float2 back = __bfloat1622float2(p);
     h[i] = *reinterpret_cast<const unsigned*>(&p);
-    l[i] = pack_bf16x2(v[2 * i] - back.x, v[2 * i + 1] - back.y);
+    rem[2 * i] = v[2 * i] - back.x;
+    rem[2 * i + 1] = v[2 * i + 1] - back.y;
+    const __nv_bfloat162 q = __floats2bfloat162_rn(rem[2 * i], rem[2 * i + 1]);
+    const float2 qb = __bfloat1622float2(q);
+    l[i] = *reinterpret_cast<const unsigned*>(&q);
+    rem[2 * i] -= qb.x;
+    rem[2 * i + 1] -= qb.y;
   }
   hi = make_uint4(h[0], h[1], h[2], h[3]);
   lo = make_uint4(l[0], l[1], l[2], l[3]);
+}
+
+__device__ __forceinline__ void split8_bf16(const float (&v)[8], uint4& hi, uint4& lo) {
+  float rem[8];
+  split8_bf16(v, hi, lo, rem);
+}
+
+__device__ __forceinline__ uint4 pack8_bf16(const float (&v)[8]) {
+  return make_uint4(pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3]), pack_bf16x2(v[4], v[5]), pack_bf16x2(v[6], v[7]));
 }
 
 // e4m3 pair (round to nearest, saturating) and its value.
@@ -663,6 +680,7 @@ constexpr int WS_WBOX = 32 * 32 * 4;  // W_hat box: 32 t x 32 z x 4 bytes
 
 struct WsPlan {
   int nt, nz, z4, zn, fp8, nterm, nacc, esize, epc;
+  int three;      // BF16 in three terms
   int tc, ns;     // t values per chunk, raw stages = term sets
   int a_term, b_term, set_bytes;
   int nwb;        // W boxes per chunk
@@ -672,18 +690,19 @@ struct WsPlan {
   int batch, nvc;
 };
 
-WsPlan make_ws_plan(int nt, int nz, int fp8, int batch) {
+WsPlan make_ws_plan(int nt, int nz, int fp8, int three, int tc, int batch) {
   WsPlan P{};
   P.nt = nt;
   P.nz = nz;
   P.z4 = rup(nz, 4);
   P.zn = rup(nz, 16);
   P.fp8 = fp8;
-  P.nterm = fp8 ? 3 : 2;
+  P.three = three;
+  P.nterm = fp8 || three ? 3 : 2;
   P.nacc = fp8 ? 3 : 2;
   P.esize = fp8 ? 1 : 2;
   P.epc = 16 / P.esize;
-  P.tc = 32;
+  P.tc = tc;
   P.a_term = NR * P.tc * P.esize;
   P.b_term = P.zn * P.tc * P.esize;
   P.set_bytes = P.nterm * (P.a_term + P.b_term);
@@ -816,17 +835,21 @@ __device__ __forceinline__ void ws_convert(const WsPlan& P, const unsigned char*
         vi[e + 1] = q.w;
       }
       uint4 hi, lo;
-      split8_bf16(vr, hi, lo);
+      float rem[8];
+      split8_bf16(vr, hi, lo, rem);
       *reinterpret_cast<uint4*>(a + o_re) = hi;
       *reinterpret_cast<uint4*>(a + P.a_term + o_re) = lo;
-      split8_bf16(vi, hi, lo);
+      if (P.three) *reinterpret_cast<uint4*>(a + 2 * P.a_term + o_re) = pack8_bf16(rem);
+      split8_bf16(vi, hi, lo, rem);
       *reinterpret_cast<uint4*>(a + o_im) = hi;
       *reinterpret_cast<uint4*>(a + P.a_term + o_im) = lo;
+      if (P.three) *reinterpret_cast<uint4*>(a + 2 * P.a_term + o_im) = pack8_bf16(rem);
     }
   }
   // B = W^T rows z < zn (z >= z4 reads the boxes' zero fill)
   const unsigned char* rw = raw + 4 * (TC / 16) * WS_MBOX;
-  for (int i = ct; i < P.zn * groups; i += WS_CONV * 32) {
+  // (from the other half of the warps: 16-t chunks give A and B at most half of them each)
+  for (int i = ct ^ (WS_CONV * 16); i < P.zn * groups; i += WS_CONV * 32) {
     const int z = i % P.zn, gI = i / P.zn;
     const unsigned char* box = rw + (z >> 5) * (32 * TC * 4) + (z & 3) * 4;
     const int zc = (z & 31) >> 2;
@@ -851,9 +874,11 @@ __device__ __forceinline__ void ws_convert(const WsPlan& P, const unsigned char*
         w[e] = *reinterpret_cast<const float*>(box + t * 128 + ((zc ^ (t & 7)) << 4));
       }
       uint4 hi, lo;
-      split8_bf16(w, hi, lo);
+      float rem[8];
+      split8_bf16(w, hi, lo, rem);
       *reinterpret_cast<uint4*>(b + o) = hi;
       *reinterpret_cast<uint4*>(b + P.b_term + o) = lo;
+      if (P.three) *reinterpret_cast<uint4*>(b + 2 * P.b_term + o) = pack8_bf16(rem);
     }
   }
 }
@@ -1055,6 +1080,11 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
                 mma_bf16(acc, A[0], B[0], idesc_main, first);
                 mma_bf16(acc + zn, A[0], B[1], idesc_main, first);
                 mma_bf16(acc + zn, A[1], B[0], idesc_main, 1);
+                if (P.three) {
+                  mma_bf16(acc + zn, A[1], B[1], idesc_main, 1);
+                  mma_bf16(acc + zn, A[0], B[2], idesc_main, 1);
+                  mma_bf16(acc + zn, A[2], B[0], idesc_main, 1);
+                }
               }
             }
             umma::commit(term_empty + s);
@@ -1135,7 +1165,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
         for (int j = 0; j < 4; ++j) {
           if (16 * j < zn) {
             float val[16];
-            if (closed) {
+            if (closed || P.three) {
               load_b(acc, j, sn, val);
             } else {
               umma::tmem_ld16(trow + acc + 16 * j, val);
@@ -1371,7 +1401,15 @@ ctof_status batch_tikhonov_contract(const ctof_kernel_s* k, int precision, int b
   const int grid = k->nclass < nsm ? k->nclass : nsm;
   if (k->nt % 16 == 0 && rup(k->nz, 16) <= 64) {
     // warp-specialised kernel: m_hat [f][v][t] and W_hat [c t][z] staged by tensor maps
-    const WsPlan W = make_ws_plan(k->nt, k->nz, fp8, batch);
+    // A plane of a compressed operator gathers what a whole window of bins holds: fewer and larger products make
+    // up b, and the rounding of a two-term BF16 split averages out less than over the bins (error against 64 bits,
+    // two terms on the bins / on the planes / three terms: 3 depths from 12 mm 6.5e-5 / 2.0e-4 / 6e-6, 8 depths
+    // from 8 mm 1.7e-4 / 3.3e-4 / 1.3e-5, 100 x 100 x 3 x 368 from 0.5 mm 3.3e-5 / 4.7e-5 / 9e-6, 64 x 64 x 32 x 256
+    // 2.7e-5 / 2.7e-5 / 3e-6).  The third term costs 1117 -> 1143 us a call (16 volumes of 128 x 128 x 64 x 512, 96
+    // planes).  At 64 depths it leaves room for 16-plane chunks only (three stages); where both fit they are equal.
+    const int three = !fp8 && k->tz_nt;
+    WsPlan W = make_ws_plan(k->nt, k->nz, fp8, three, 32, batch);
+    if (three && W.total > 227 * 1024) W = make_ws_plan(k->nt, k->nz, fp8, three, 16, batch);
     if (W.total <= 227 * 1024) {
       // m_hat element (t = 16 h + tt, v, f) as a 4-D tensor (tt, v, h, f): one box
       // of 16 tt x 16 volumes x TC/16 halves per member lands as [half][volume][16 t]
@@ -1385,7 +1423,7 @@ ctof_status batch_tikhonov_contract(const ctof_kernel_s* k, int precision, int b
       const unsigned wbox[2] = {32, (unsigned)W.tc};
       if (ctof_encode_map(&mmap, 8, 4, m_hat, mdims, mstr, mbox, 128) == CTOF_OK &&
           ctof_encode_map(&wmap, 4, 2, k->d_what, wdims, wstr, wbox, 128) == CTOF_OK) {
-        auto kern = k_batch_tikhonov_ws<32>;
+        auto kern = W.tc == 32 ? k_batch_tikhonov_ws<32> : k_batch_tikhonov_ws<16>;
         // |I - C G'| is ~5e-6 at lambda = 1e-3 of the largest Gram diagonal and grows as its
         // inverse: from 1e-5 on its square stays below the split's own error (measured against
         // 64 bits at 24 to 64 depths, BF16 / FP8, both ways: 2e-5 / 1e-4 at 1e-3, 1e-3 / 4e-3 at
