@@ -368,7 +368,7 @@ ctof_status ctof_kernel_get_tuning(ctof_kernel k, int* h_pb4);
  * first product alone, then `refine_steps` steps of
  * x += C (b - (G + lambda I) x) with C = (G + lambda I)^-1 from the FP64
  * Cholesky factor, those products in TF32 hi/lo on the tensor cores
- * (FP32-level).  With two or more steps and lambda_rel >= 1e-5 the first step
+ * (FP32-level).  With two or more steps and lambda_rel >= 1e-4 the first step
  * is formed as C b, which is what it gives but for the rounding of C.  On a
  * handle that is compressed in time (ctof_kernel_get_planes) BF16 takes a third
  * term and six products, b is FP32-level and x0 = C b.  CTOF_FP32: the plain
