@@ -1428,8 +1428,9 @@ ctof_status batch_tikhonov_contract(const ctof_kernel_s* k, int precision, int b
         // difference away.  |I - C G'| is ~5e-6 at lambda = 1e-3 of the largest Gram diagonal and grows as its
         // inverse.  Error against 64 bits with it over without it, BF16 and FP8, 2, 3 and 8 steps, 12 geometries of 2
         // to 64 depths: 0.99 to 1.01 at 1e-3, 0.97 to 1.05 (mean 1.00) at 1e-4; 0.71 to 1.12 at 1e-5, where
-        // refinement itself scatters, so it ends before.  A single step keeps its starting value.  861 -> 651 us
-        // (BF16 in two terms, 16 volumes of 128 x 128 x 64 at 96 planes).
+        // refinement itself scatters, so it ends before.  A single step keeps its starting value.  16 volumes, two
+        // steps: BF16 1386 -> 1143 us at 128 x 128 x 64 x 512, 1103 -> 915 us at 128 x 128 x 48 x 256; FP8 4091 -> 3865
+        // and 1959 -> 1916 us (on the bins, where the contraction sets the pace).
         const int closed = refine >= 2 && k->bt_lambda >= 1e-4 * k->gram_max;
         CTOF_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, W.total));
         kern<<<grid, WS_THREADS, W.total, st>>>(mmap, wmap, W, k->d_bt_tab, k->d_bt_sw, k->d_members, k->nclass,

@@ -344,7 +344,8 @@ ctof_status admm_graph(ctof_kernel_s* k, const ctof_solver_params* prm, cudaStre
   CTOF_TRY(autotune(k, st));
   const bool same = k->graph && k->graph_iters == prm->iters && k->graph_rho == prm->rho &&
                     k->graph_beta == prm->tv_beta && k->graph_beta_rel == prm->beta_rel &&
-                    k->graph_timing == k->timing;
+                    k->graph_timing == k->timing && k->graph_polls == k->max_polls &&
+                    std::equal(k->graph_pb, k->graph_pb + 4, k->tune_pb);
   if (!same) {
     if (k->graph) {
       cudaGraphExecDestroy(k->graph);
@@ -384,6 +385,8 @@ ctof_status admm_graph(ctof_kernel_s* k, const ctof_solver_params* prm, cudaStre
     cudaGraphDestroy(g);
     CTOF_CUDA_TRY(e);
     k->graph_timing = k->timing;
+    k->graph_polls = k->max_polls;
+    std::copy(k->tune_pb, k->tune_pb + 4, k->graph_pb);
     k->graph_iters = prm->iters;
     k->graph_rho = prm->rho;
     k->graph_beta = prm->tv_beta;

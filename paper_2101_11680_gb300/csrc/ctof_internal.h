@@ -84,6 +84,8 @@ struct ctof_kernel_s {
   int graph_iters;
   double graph_rho, graph_beta, graph_beta_rel;
   int graph_timing;
+  long long graph_polls;  // max_polls and column tiles are arguments of its kernels
+  int graph_pb[4];
   int graph_kernel_nodes;
 
   // optional per-stage timing: 4 events per ADMM iteration, recorded inside the graph
