@@ -1396,6 +1396,7 @@ ctof_status batch_tikhonov_prepare(ctof_kernel_s* k, double lambda, cudaStream_t
 ctof_status batch_tikhonov_contract(const ctof_kernel_s* k, int precision, int batch, const float2* m_hat, int ldm,
                                     float2* x_hat, int ldx, int refine, cudaStream_t st) {
   const int fp8 = precision == CTOF_FP8E4M3 ? 1 : 0;
+  const ctof_kernel_s* own = ctof_owner(k);  // keeps the tables
   int nsm = 152;
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, k->device);
   const int grid = k->nclass < nsm ? k->nclass : nsm;
@@ -1431,9 +1432,9 @@ ctof_status batch_tikhonov_contract(const ctof_kernel_s* k, int precision, int b
         // refinement itself scatters, so it ends before.  A single step keeps its starting value.  16 volumes, two
         // steps: BF16 1386 -> 1143 us at 128 x 128 x 64 x 512, 1103 -> 915 us at 128 x 128 x 48 x 256; FP8 4091 -> 3865
         // and 1959 -> 1916 us (on the bins, where the contraction sets the pace).
-        const int closed = refine >= 2 && k->bt_lambda >= 1e-4 * k->gram_max;
+        const int closed = refine >= 2 && own->bt_lambda >= 1e-4 * k->gram_max;
         CTOF_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, W.total));
-        kern<<<grid, WS_THREADS, W.total, st>>>(mmap, wmap, W, k->d_bt_tab, k->d_bt_sw, k->d_members, k->nclass,
+        kern<<<grid, WS_THREADS, W.total, st>>>(mmap, wmap, W, own->d_bt_tab, own->d_bt_sw, k->d_members, k->nclass,
                                                 m_hat, ldm, x_hat, ldx, refine, closed, k->d_flags, k->max_polls);
         CTOF_CUDA_TRY(cudaGetLastError());
         return CTOF_OK;
@@ -1444,7 +1445,7 @@ ctof_status batch_tikhonov_contract(const ctof_kernel_s* k, int precision, int b
   const BtPlan P = make_plan(k->nt, k->nz, fp8, batch);
   if (P.total > 227 * 1024) return CTOF_EUNSUPPORTED;
   CTOF_CUDA_TRY(cudaFuncSetAttribute(k_batch_tikhonov_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, P.total));
-  k_batch_tikhonov_tc<<<grid, BT_THREADS, P.total, st>>>(P, k->d_what, k->d_bt_tab, k->d_bt_sw, k->d_members,
+  k_batch_tikhonov_tc<<<grid, BT_THREADS, P.total, st>>>(P, k->d_what, own->d_bt_tab, own->d_bt_sw, k->d_members,
                                                           k->nclass, m_hat, ldm, x_hat, ldx, refine, k->d_flags,
                                                           k->max_polls);
   CTOF_CUDA_TRY(cudaGetLastError());

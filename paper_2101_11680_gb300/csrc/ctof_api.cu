@@ -405,6 +405,7 @@ ctof_status admm_run(ctof_kernel_s* k, const ctof_solver_params* prm, cudaStream
 
 ctof_status tikhonov_inverse(ctof_kernel_s* k, double lambda, const float** hinv, cudaStream_t st) {
   if (!(lambda > 0.0) || !isfinite(lambda)) return CTOF_EINVAL;
+  k = ctof_owner(k);
   int slot = k->tik_lambda[0] == lambda ? 0 : (k->tik_lambda[1] == lambda ? 1 : -1);
   if (slot < 0) {
     slot = 1 - k->tik_last;  // replace the slot not used last
@@ -606,11 +607,11 @@ void ctof_kernel_destroy(ctof_kernel k) {
     if (o->batch_stream) cudaStreamDestroy(o->batch_stream);
     if (o->batch_event) cudaEventDestroy(o->batch_event);
     destroy_events(o);
-    if (o->d_bt_cinv) cudaFree(o->d_bt_cinv);
-    if (o->d_batch) cudaFree(o->d_batch);
-    for (int i = 0; i < 2; ++i)
-      if (o->d_tik_hinv[i]) cudaFree(o->d_tik_hinv[i]);
   }
+  if (k->d_bt_cinv) cudaFree(k->d_bt_cinv);
+  if (k->d_batch) cudaFree(k->d_batch);
+  for (int i = 0; i < 2; ++i)
+    if (k->d_tik_hinv[i]) cudaFree(k->d_tik_hinv[i]);
   time_basis_free(k);
   if (k->d_admm) cudaFree(k->d_admm);
   if (k->d_w) cudaFree(k->d_w);
@@ -829,7 +830,6 @@ ctof_status ctof_kernel_get_info(ctof_kernel k, ctof_kernel_info* info) {
   info->device_bytes = k->bytes + k->admm_bytes + (k->tz ? k->tz->tz_bytes : 0) +
                        (k->d_w ? (size_t)k->nt * k->nz * k->q * k->q * sizeof(double) : 0) +
                        ((k->d_tik_hinv[0] ? 1 : 0) + (k->d_tik_hinv[1] ? 1 : 0)) * tik_bytes;
-  if (k->tz) info->device_bytes += ((o->d_tik_hinv[0] ? 1 : 0) + (o->d_tik_hinv[1] ? 1 : 0)) * tik_bytes;
   return CTOF_OK;
 }
 
@@ -982,6 +982,7 @@ ctof_status ctof_reconstruct_batch_tikhonov(ctof_kernel k, int batch, const floa
   // FP8 keeps the time bins: the projection's planes quantise differently, and with few depths that shows
   // (64-bit error 1.3e-4 on the bins, 1.9e-4 on the planes at 74^2 x 3 x 368; BF16 and FP32 are as good or better on them).
   const bool tz = k->tz != nullptr && precision != CTOF_FP8E4M3;
+  ctof_kernel_s* own = k;
   if (tz) k = k->tz;
   const int ldm = ctof_round_up(batch * k->nt, 8), ldx = ctof_round_up(batch * k->nz, 8);
   const size_t b_sm = (size_t)k->nf * ldm * sizeof(float2), b_sx = (size_t)k->nf * ldx * sizeof(float2);
@@ -989,19 +990,19 @@ ctof_status ctof_reconstruct_batch_tikhonov(ctof_kernel k, int batch, const floa
   const size_t b_in = fft_inter_elems(k, batch * std::max(k->nt, k->nz), k->n) * sizeof(float2);
   const size_t b_fft = ((b_sm + 255) & ~(size_t)255) + ((b_sx + 255) & ~(size_t)255) + ((b_in + 255) & ~(size_t)255);
   const size_t need = b_fft + (tz ? (size_t)batch * k->nt * k->n * k->n * sizeof(float) : 0);
-  if (need > k->batch_bytes) {
+  if (need > own->batch_bytes) {
     CTOF_CUDA_TRY(cudaStreamSynchronize(st));
-    if (k->d_batch) cudaFree(k->d_batch);
-    k->d_batch = nullptr;
-    k->batch_bytes = 0;
-    if (cudaMalloc(&k->d_batch, need) != cudaSuccess) {
+    if (own->d_batch) cudaFree(own->d_batch);
+    own->d_batch = nullptr;
+    own->batch_bytes = 0;
+    if (cudaMalloc(&own->d_batch, need) != cudaSuccess) {
       cudaGetLastError();
-      k->d_batch = nullptr;
+      own->d_batch = nullptr;
       return CTOF_ENOMEM;
     }
-    k->batch_bytes = need;
+    own->batch_bytes = need;
   }
-  char* base = static_cast<char*>(k->d_batch);
+  char* base = static_cast<char*>(own->d_batch);
   float2* spec_m = reinterpret_cast<float2*>(base);
   float2* spec_x = reinterpret_cast<float2*>(base + ((b_sm + 255) & ~(size_t)255));
   float2* inter = reinterpret_cast<float2*>(base + ((b_sm + 255) & ~(size_t)255) + ((b_sx + 255) & ~(size_t)255));
@@ -1011,7 +1012,7 @@ ctof_status ctof_reconstruct_batch_tikhonov(ctof_kernel k, int batch, const floa
     d_m = planes;
   }
   CTOF_TRY(fft_forward_planes(k, d_m, batch * k->nt, k->n, k->n, k->n, inter, spec_m, ldm, st));
-  CTOF_TRY(batch_tikhonov_prepare(k, lambda, st));
+  CTOF_TRY(batch_tikhonov_prepare(own, lambda, st));
   CTOF_TRY(batch_tikhonov_contract(k, precision, batch, spec_m, ldm, spec_x, ldx, refine_steps, st));
   return fft_inverse_planes(k, spec_x, ldx, batch * k->nz, k->n, k->n, inter, d_mu, k->n, st);
 }

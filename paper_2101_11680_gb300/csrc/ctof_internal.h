@@ -110,9 +110,12 @@ struct ctof_kernel_s {
 
   // Time compression (time_basis.cu): `tz` is this handle's operator on r < nt
   // planes (V = Q^T W_hat in place of W_hat; null where it does not pay).  It
-  // borrows this handle's buffers and tables and owns the rest (d_tz_base, its
-  // graph, Tikhonov and precision-form tables); the fields below are its own.
+  // borrows this handle's buffers and tables and owns the rest (d_tz_base and its
+  // graph); the fields below are its own.  What the Tikhonov solves make on first
+  // use (inverses, precision-form tables, batch workspace) depends on the Gram
+  // matrices alone and is kept once, with this handle.
   ctof_kernel_s* tz;
+  ctof_kernel_s* tz_of;    // in `tz`: this handle
   void* d_tz_base;
   size_t tz_bytes;
   int tz_nt;               // bins of the measurement domain
@@ -126,6 +129,10 @@ struct ctof_kernel_s {
 // run on (one projection of the measurement serves the whole solve).
 inline ctof_kernel_s* ctof_ops(ctof_kernel_s* k) { return k->tz ? k->tz : k; }
 inline const ctof_kernel_s* ctof_ops(const ctof_kernel_s* k) { return k->tz ? k->tz : k; }
+
+// The handle that keeps what both operators share.
+inline ctof_kernel_s* ctof_owner(ctof_kernel_s* k) { return k->tz_of ? k->tz_of : k; }
+inline const ctof_kernel_s* ctof_owner(const ctof_kernel_s* k) { return k->tz_of ? k->tz_of : k; }
 
 // The operator that a single application (forward, adjoint, one Tikhonov
 // solve) runs on: the projection or expansion is a launch of its own, so the

@@ -396,6 +396,7 @@ static ctof_status make_basis(ctof_kernel_s* k, const double* what64, cudaStream
   ctof_kernel_s* z = new (std::nothrow) ctof_kernel_s(*k);
   if (!z) return CTOF_ENOMEM;
   z->tz = nullptr;
+  z->tz_of = k;
   z->nt = rows;
   z->ldt = rows;
   auto at = [](size_t& off, size_t bytes) {
