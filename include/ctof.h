@@ -97,7 +97,7 @@ typedef struct {
   int nt, nz;
   double scale;     /* max_f sigma_max(W_hat(f)) (the ADMM normalisation) */
   double gram_max_diag; /* max over f, j of (W_hat^T W_hat)_jj */
-  size_t device_bytes;  /* device memory held by the handle */
+  size_t device_bytes;  /* device memory held by the handle now (some is made on first use) */
   int admm_stages;      /* shared-memory stages of the ADMM x-update kernel at
                            this size (0: the fallback kernel runs) */
 } ctof_kernel_info;

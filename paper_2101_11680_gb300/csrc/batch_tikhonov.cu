@@ -1372,6 +1372,7 @@ ctof_status batch_tikhonov_prepare(ctof_kernel_s* k, double lambda, cudaStream_t
       cudaGetLastError();
       return CTOF_ENOMEM;
     }
+    k->bt_bytes = 2 * fl + sw + tab;
     unsigned char* b = static_cast<unsigned char*>(p);
     k->d_bt_cinv = reinterpret_cast<float*>(b);
     k->d_bt_glam = reinterpret_cast<float*>(b + fl);

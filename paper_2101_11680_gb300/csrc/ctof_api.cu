@@ -829,7 +829,8 @@ ctof_status ctof_kernel_get_info(ctof_kernel k, ctof_kernel_info* info) {
   const size_t tik_bytes = (size_t)k->nclass * k->nz * k->z4 * sizeof(float);
   info->device_bytes = k->bytes + k->admm_bytes + (k->tz ? k->tz->tz_bytes : 0) +
                        (k->d_w ? (size_t)k->nt * k->nz * k->q * k->q * sizeof(double) : 0) +
-                       ((k->d_tik_hinv[0] ? 1 : 0) + (k->d_tik_hinv[1] ? 1 : 0)) * tik_bytes;
+                       ((k->d_tik_hinv[0] ? 1 : 0) + (k->d_tik_hinv[1] ? 1 : 0)) * tik_bytes + k->bt_bytes +
+                       k->batch_bytes;
   return CTOF_OK;
 }
 

@@ -99,6 +99,7 @@ struct ctof_kernel_s {
   float* d_bt_sw;      // [nclass] FP8 scale of W_hat (max |W_hat| / 448)
   unsigned char* d_bt_tab;  // [nclass] C hi, C lo, G + lambda I hi, lo: BF16 [zn x zn] K-major tiles
   double bt_lambda;
+  size_t bt_bytes;     // of the allocation behind the four above
   void* d_batch;       // batch spectra + row intermediates (one allocation)
   size_t batch_bytes;
 
