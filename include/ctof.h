@@ -370,10 +370,10 @@ ctof_status ctof_kernel_get_tuning(ctof_kernel k, int* h_pb4);
  * Cholesky factor, those products in TF32 hi/lo on the tensor cores
  * (FP32-level).  With two or more steps and lambda_rel >= 1e-4 the first step
  * is formed as C b, which is what it gives but for the rounding of C.  On a
- * handle that is compressed in time (ctof_kernel_get_planes) BF16 takes a third
- * term and six products, b is FP32-level and x0 = C b.  CTOF_FP32: the plain
- * FP32 per-volume path (ctof_reconstruct with CTOF_SOLVER_TIKHONOV) for
- * comparison.
+ * handle that is compressed in time (ctof_kernel_get_planes) BF16 works on the
+ * planes; those that are not bins themselves take a third term and six
+ * products, all of them in b0.  CTOF_FP32: the plain FP32 per-volume path
+ * (ctof_reconstruct with CTOF_SOLVER_TIKHONOV) for comparison.
  * lambda = lambda_rel * gram_max_diag; *lambda_out (optional) receives it.
  * The first BF16 / FP8 call for a lambda makes C, G + lambda I and their
  * tensor-core tables (per class ~4 nz^2 x 4 bytes plus 2 nz z4 x 4); the batch

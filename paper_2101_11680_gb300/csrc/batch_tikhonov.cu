@@ -11,8 +11,8 @@
 // are split into narrow-format terms whose sum reproduces the FP32 value:
 //
 //   BF16: v = v_hi + v_lo (both BF16); b0 = hi.hi, b = hi.hi + (hi.lo + lo.hi)
-//         (on the planes of a compressed operator v = v_hi + v_lo + v_3 and
-//         the six products down to 2^-16; b0 = b there)
+//         (on planes of a compressed operator that are not bins themselves
+//         v = v_hi + v_lo + v_3, and the six products down to 2^-16 are in b0)
 //   FP8:  v = s (q0 + q1/16 + q2/256), each q an e4m3 value, s a scale that
 //         maps the block's largest magnitude to 448 (per frequency class for
 //         W_hat, per right-hand side for m_hat); products grouped by level:
@@ -680,7 +680,8 @@ constexpr int WS_WBOX = 32 * 32 * 4;  // W_hat box: 32 t x 32 z x 4 bytes
 
 struct WsPlan {
   int nt, nz, z4, zn, fp8, nterm, nacc, esize, epc;
-  int three;      // BF16 in three terms
+  int three;      // BF16 in three terms, but for
+  int two_k;      // the first two_k K steps (16 planes each)
   int tc, ns;     // t values per chunk, raw stages = term sets
   int a_term, b_term, set_bytes;
   int nwb;        // W boxes per chunk
@@ -690,7 +691,7 @@ struct WsPlan {
   int batch, nvc;
 };
 
-WsPlan make_ws_plan(int nt, int nz, int fp8, int three, int tc, int batch) {
+WsPlan make_ws_plan(int nt, int nz, int fp8, int three, int two_k, int tc, int batch) {
   WsPlan P{};
   P.nt = nt;
   P.nz = nz;
@@ -698,6 +699,7 @@ WsPlan make_ws_plan(int nt, int nz, int fp8, int three, int tc, int batch) {
   P.zn = rup(nz, 16);
   P.fp8 = fp8;
   P.three = three;
+  P.two_k = three ? two_k : nt;
   P.nterm = fp8 || three ? 3 : 2;
   P.nacc = fp8 ? 3 : 2;
   P.esize = fp8 ? 1 : 2;
@@ -1077,13 +1079,15 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
                 mma_e4m3(acc + 2 * zn, A[1], B[1], idesc_main, 1);
                 mma_e4m3(acc + 2 * zn, A[2], B[0], idesc_main, 1);
               } else {
+                const bool two = kc * ksteps + ks < P.two_k;
+                const uint32_t acc1 = two ? acc + zn : acc;  // three terms: all products make up b0
                 mma_bf16(acc, A[0], B[0], idesc_main, first);
-                mma_bf16(acc + zn, A[0], B[1], idesc_main, first);
-                mma_bf16(acc + zn, A[1], B[0], idesc_main, 1);
-                if (P.three) {
-                  mma_bf16(acc + zn, A[1], B[1], idesc_main, 1);
-                  mma_bf16(acc + zn, A[0], B[2], idesc_main, 1);
-                  mma_bf16(acc + zn, A[2], B[0], idesc_main, 1);
+                mma_bf16(acc1, A[0], B[1], idesc_main, two ? first : 1);
+                mma_bf16(acc1, A[1], B[0], idesc_main, 1);
+                if (!two) {
+                  mma_bf16(acc, A[1], B[1], idesc_main, 1);
+                  mma_bf16(acc, A[0], B[2], idesc_main, 1);
+                  mma_bf16(acc, A[2], B[0], idesc_main, 1);
                 }
               }
             }
@@ -1132,6 +1136,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
     auto load_b = [&](uint32_t acc, int j, float sn, float (&out)[16]) {
       float d1[16], d2[16];
       umma::tmem_ld16(trow + acc + 16 * j, out);
+      if (P.two_k == 0) return;  // the first accumulator holds everything
       umma::tmem_ld16(trow + acc + zn + 16 * j, d1);
       if (P.fp8) umma::tmem_ld16(trow + acc + 2 * zn + 16 * j, d2);
 #pragma unroll
@@ -1165,7 +1170,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
         for (int j = 0; j < 4; ++j) {
           if (16 * j < zn) {
             float val[16];
-            if (closed || P.three) {
+            if (closed) {
               load_b(acc, j, sn, val);
             } else {
               umma::tmem_ld16(trow + acc + 16 * j, val);
@@ -1404,14 +1409,16 @@ ctof_status batch_tikhonov_contract(const ctof_kernel_s* k, int precision, int b
   if (k->nt % 16 == 0 && rup(k->nz, 16) <= 64) {
     // warp-specialised kernel: m_hat [f][v][t] and W_hat [c t][z] staged by tensor maps
     // A plane of a compressed operator gathers what a whole window of bins holds: fewer and larger products make
-    // up b, and the rounding of a two-term BF16 split averages out less than over the bins (error against 64 bits,
-    // two terms on the bins / on the planes / three terms: 3 depths from 12 mm 6.5e-5 / 2.0e-4 / 6e-6, 8 depths
-    // from 8 mm 1.7e-4 / 3.3e-4 / 1.3e-5, 100 x 100 x 3 x 368 from 0.5 mm 3.3e-5 / 4.7e-5 / 9e-6, 64 x 64 x 32 x 256
-    // 2.7e-5 / 2.7e-5 / 3e-6).  The third term costs 1117 -> 1143 us a call (16 volumes of 128 x 128 x 64 x 512, 96
-    // planes).  At 64 depths it leaves room for 16-plane chunks only (three stages); where both fit they are equal.
+    // up b, and the rounding of a two-term BF16 split averages out less than over the bins.  Planes that are bins
+    // themselves (the first windows, as a rule) round as the bins do; the others take a third term.  Error against
+    // 64 bits, two terms on the bins / on the planes / this: 3 depths from 12 mm 6.5e-5 / 2.0e-4 / 1.4e-5, 8 depths
+    // from 8 mm 1.7e-4 / 3.3e-4 / 1.0e-4, 100 x 100 x 3 x 368 from 0.5 mm 3.3e-5 / 4.7e-5 / 9e-6, 64 x 64 x 32 x 256
+    // 2.7e-5 for all.  It costs 1117 -> 1139 us a call (16 volumes of 128 x 128 x 64 x 512, 96 planes).  At 64
+    // depths it leaves room for 16-plane chunks only (three stages); where both fit they are equal.
     const int three = !fp8 && k->tz_nt;
-    WsPlan W = make_ws_plan(k->nt, k->nz, fp8, three, 32, batch);
-    if (three && W.total > 227 * 1024) W = make_ws_plan(k->nt, k->nz, fp8, three, 16, batch);
+    const int two_k = k->tz_bins / 16;
+    WsPlan W = make_ws_plan(k->nt, k->nz, fp8, three, two_k, 32, batch);
+    if (three && W.total > 227 * 1024) W = make_ws_plan(k->nt, k->nz, fp8, three, two_k, 16, batch);
     if (W.total <= 227 * 1024) {
       // m_hat element (t = 16 h + tt, v, f) as a 4-D tensor (tt, v, h, f): one box
       // of 16 tt x 16 volumes x TC/16 halves per member lands as [half][volume][16 t]

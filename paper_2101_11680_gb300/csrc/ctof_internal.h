@@ -120,6 +120,7 @@ struct ctof_kernel_s {
   void* d_tz_base;
   size_t tz_bytes;
   int tz_nt;               // bins of the measurement domain
+  int tz_bins;             // leading planes that are bins themselves
   float* d_tz_q;           // [tz_nt][16] rows of the windows' bases
   int4* d_tz_win;          // windows: bins [x, y), first plane z, planes w
   int4* d_tz_tiles;        // the windows cut into tiles of up to 16 bins

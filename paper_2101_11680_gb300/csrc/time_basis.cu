@@ -441,6 +441,11 @@ static ctof_status make_basis(ctof_kernel_s* k, const double* what64, cudaStream
   z->tz_nwin = (int)wins.size();
   z->tz_ntiles = (int)tiles.size();
   z->tz_nt = nt;
+  z->tz_bins = 0;
+  for (const Window& g : b.win) {
+    if (g.planes < g.end - g.begin) break;
+    z->tz_bins = g.end;
+  }
   double* d_tol = static_cast<double*>(d_q.p) + b.q.size();
   CTOF_CUDA_TRY(cudaMemcpyAsync(d_q.p, b.q.data(), qb, cudaMemcpyHostToDevice, st));
   CTOF_CUDA_TRY(cudaMemcpyAsync(d_tol, b.tol.data(), db, cudaMemcpyHostToDevice, st));
