@@ -5,6 +5,7 @@
 
 #include <math.h>
 #include <stddef.h>
+#include <string.h>
 
 #include <algorithm>
 #include <utility>
@@ -22,17 +23,44 @@ constexpr double TZ_CHECK = 2e-8;    // residual over all classes, relative to a
 constexpr double TZ_CHECK_OWN = 1e-7;  // the same relative to that of the depth in the bin
 constexpr double TZ_CANCEL = 10.0;   // largest sum_j |Q V| / |sum_j Q V| over the bins and depths of a window
 
-inline double dot(const double* a, const double* b, size_t n) {
-  double s[4] = {0, 0, 0, 0};
-  size_t i = 0;
-  for (; i + 4 <= n; i += 4)
-    for (int u = 0; u < 4; ++u) s[u] += a[i + u] * b[i + u];
-  for (; i < n; ++i) s[0] += a[i] * b[i];
-  return (s[0] + s[1]) + (s[2] + s[3]);
+// Pairs of doubles (the 128-bit vectors of either host) in four independent sums:
+// the fit is bound by these loops.
+typedef double pair_t __attribute__((vector_size(16)));
+inline pair_t pair_at(const double* p) {
+  pair_t v;
+  memcpy(&v, p, sizeof(v));
+  return v;
 }
 
-inline void axpy(double f, const double* x, double* y, size_t n) {
-  for (size_t i = 0; i < n; ++i) y[i] += f * x[i];
+inline double dot(const double* a, const double* b, size_t n) {
+  pair_t s[4] = {};
+  size_t i = 0;
+  for (; i + 8 <= n; i += 8)
+    for (int u = 0; u < 4; ++u) s[u] += pair_at(a + i + 2 * u) * pair_at(b + i + 2 * u);
+  const pair_t t = (s[0] + s[1]) + (s[2] + s[3]);
+  double r = t[0] + t[1];
+  for (; i < n; ++i) r += a[i] * b[i];
+  return r;
+}
+
+// y += f x; the squared norm of the new y.
+inline double axpy(double f, const double* x, double* y, size_t n) {
+  pair_t s[4] = {};
+  const pair_t ff = {f, f};
+  size_t i = 0;
+  for (; i + 8 <= n; i += 8)
+    for (int u = 0; u < 4; ++u) {
+      const pair_t v = pair_at(y + i + 2 * u) + ff * pair_at(x + i + 2 * u);
+      memcpy(y + i + 2 * u, &v, sizeof(v));
+      s[u] += v * v;
+    }
+  const pair_t t = (s[0] + s[1]) + (s[2] + s[3]);
+  double r = t[0] + t[1];
+  for (; i < n; ++i) {
+    y[i] += f * x[i];
+    r += y[i] * y[i];
+  }
+  return r;
 }
 
 // Largest cancellation in the products of an orthonormal basis g [r][len]: over
@@ -117,41 +145,48 @@ inline int window_basis(const double* w, int nz, int ns, const double* d, int a,
   for (int t = a; t < b; ++t)
     for (int z = 0; z < nz; ++z) cz[z] = std::max(cz[z], w[t * cols + z] / d[t]);  // sample 0 is DC
   std::vector<char> keep(cols, 0);
-  for (int t = a; t < b; ++t)
-    for (size_t i = 0; i < cols; ++i)
-      if (fabs(w[t * cols + i]) > 0.1 * TZ_EPS * d[t] * cz[i % nz]) keep[i] = 1;
+  std::vector<double> thr(nz);
+  for (int t = a; t < b; ++t) {
+    for (int z = 0; z < nz; ++z) thr[z] = 0.1 * TZ_EPS * d[t] * cz[z];
+    for (int s = 0; s < ns; ++s)
+      for (int z = 0; z < nz; ++z) keep[(size_t)s * nz + z] |= fabs(w[t * cols + (size_t)s * nz + z]) > thr[z];
+  }
   std::vector<size_t> idx;
   for (size_t i = 0; i < cols; ++i)
     if (keep[i]) idx.push_back(i);
   if (idx.empty()) idx.push_back(0);
   const size_t n = idx.size();
+  std::vector<int> zi(n);
+  std::vector<double> sc(n), nn(len);  // 1 / cz of the kept columns, squared norms of the residual rows
+  for (size_t i = 0; i < n; ++i) {
+    zi[i] = (int)(idx[i] % nz);
+    sc[i] = 1.0 / cz[zi[i]];
+  }
   std::vector<double> e(len * n), res;
-  for (int t = 0; t < len; ++t)
-    for (size_t i = 0; i < n; ++i) e[t * n + i] = w[(a + t) * cols + idx[i]] / (d[a + t] * cz[idx[i] % nz]);
+  for (int t = 0; t < len; ++t) {
+    const double dt = 1.0 / d[a + t];
+    for (size_t i = 0; i < n; ++i) e[t * n + i] = w[(a + t) * cols + idx[i]] * dt * sc[i];
+    nn[t] = dot(&e[t * n], &e[t * n], n);
+  }
   res = e;
+  std::vector<double> lim((size_t)len * nz);  // a residual's factor to its bin's and depth's own response
+  for (int t = 0; t < len; ++t)
+    for (int z = 0; z < nz; ++z)
+      lim[t * nz + z] = cz[z] / std::max(fabs(w[(a + t) * cols + z]) / d[a + t], TZ_FLOOR);
   // rows pivoted by norm, orthonormalised twice, until the residual is below TZ_EPS everywhere
   std::vector<double> v;
   int r = 0;
   for (; r < len; ++r) {
-    double top = 0.0, best = -1.0;
-    int piv = 0;
-    for (int t = 0; t < len; ++t) {
-      const double* x = res.data() + t * n;
-      for (size_t i = 0; i < n; ++i) top = std::max(top, fabs(x[i]));
-      const double nn = dot(x, x, n);
-      if (nn > best) {
-        best = nn;
-        piv = t;
-      }
-    }
+    int piv = (int)(std::max_element(nn.begin(), nn.end()) - nn.begin());
+    double top = sqrt(nn[piv] / n);  // a lower bound of the largest entry; the entries themselves where it does not decide
+    if (!(top >= TZ_EPS))
+      for (double u : res) top = std::max(top, fabs(u));
     if (!(top >= TZ_EPS)) {  // in the window's scale; then every bin and depth in its own
       double over = TZ_OWN;
       piv = -1;
       for (int t = 0; t < len; ++t)
         for (size_t i = 0; i < n; ++i) {
-          const int z = (int)(idx[i] % nz);
-          const double own = std::max(fabs(w[(a + t) * cols + z]) / d[a + t], TZ_FLOOR);
-          const double rel = fabs(res[t * n + i]) * cz[z] / own;
+          const double rel = fabs(res[t * n + i]) * lim[t * nz + zi[i]];
           if (rel > over) {
             over = rel;
             piv = t;
@@ -167,7 +202,7 @@ inline int window_basis(const double* w, int nz, int ns, const double* d, int a,
     if (!(nrm > 0.0)) break;
     for (double& u : x) u /= nrm;
     v.insert(v.end(), x.begin(), x.end());
-    for (int t = 0; t < len; ++t) axpy(-dot(&res[t * n], x.data(), n), x.data(), &res[t * n], n);
+    for (int t = 0; t < len; ++t) nn[t] = axpy(-dot(&res[t * n], x.data(), n), x.data(), &res[t * n], n);
   }
   if (r >= len - 1 && len <= TZ_R) {  // nothing to gain: the bins themselves
     for (int t = 0; t < len; ++t)
