@@ -830,20 +830,21 @@ def main():
     planes = kern.planes()
     alg_bytes = contract_bytes(info, cfg["nz"], planes)
     achieved = alg_bytes / (avg_contract_ms * 1e-3) / 1e9
+    admm_kernel = kern.admm_kernel()
+    source = "contract_warp.cu" if admm_kernel == "k_contract_warp" else "contract_admm.cu"
     traffic = None
     prof = os.path.join(ROOT, "profiles", "contract_admm_cfg2.json")
     if args.config == "cfg2" and os.path.exists(prof):
         try:
             with open(prof) as f:
                 pj = json.load(f)
-            src = open(os.path.join(ROOT, "paper_2101_11680_gb300", "csrc", "contract_warp.cu"), "rb").read()
+            src = open(os.path.join(ROOT, "paper_2101_11680_gb300", "csrc", source), "rb").read()
             import hashlib
-            if pj.get("source_sha256") == hashlib.sha256(src).hexdigest():
+            if pj.get("kernel") == admm_kernel and pj.get("source_sha256") == hashlib.sha256(src).hexdigest():
                 traffic = pj.get("dram_bytes_per_launch")
         except Exception:
             traffic = None
 
-    admm_kernel = "k_contract_warp"  # (at these sizes; larger class blocks run k_contract_admm_pipe)
     launches_per_step = timing.graph_kernel_nodes
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,

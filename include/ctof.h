@@ -212,6 +212,11 @@ ctof_status ctof_kernel_get_info(ctof_kernel k, ctof_kernel_info* info);
  * depth by depth). */
 ctof_status ctof_kernel_get_planes(ctof_kernel k, int* planes);
 
+/* Name of the kernel that the handle's ADMM x-update runs (it depends on the
+ * size of a class block and on the memory found at build time): a static
+ * string, empty for a null handle. */
+const char* ctof_kernel_admm_kernel(ctof_kernel k);
+
 /* Copy the FP64 kernel table W[nt][nz][ny][nx] (non-negative offsets |oy|, |ox|;
  * for circular mode the table is [nt][nz][P/2+1][P/2+1]) to host memory.
  * Needs CTOF_KEEP_W at build time (else EUNSUPPORTED).  Synchronous. */

@@ -840,6 +840,12 @@ ctof_status ctof_kernel_get_planes(ctof_kernel k, int* planes) {
   return CTOF_OK;
 }
 
+const char* ctof_kernel_admm_kernel(ctof_kernel k) {
+  if (!k) return "";
+  const ctof_kernel_s* o = ctof_ops(k);
+  return o->d_what_pitch ? "k_contract_warp" : o->d_what_admm ? "k_contract_admm_pipe" : "k_contract_admm";
+}
+
 ctof_status ctof_kernel_get_w(ctof_kernel k, double* h_w) {
   if (!k || !h_w) return CTOF_EINVAL;
   if (!k->d_w) return CTOF_EUNSUPPORTED;

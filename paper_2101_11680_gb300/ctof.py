@@ -117,6 +117,7 @@ _SIGNATURES = {
     "ctof_set_wait_limit": (ctypes.c_int, [_P, ctypes.c_longlong]),
     "ctof_sync_status": (ctypes.c_int, [_P, _P]),
     "ctof_get_timing": (ctypes.c_int, [_P, ctypes.POINTER(Timing)]),
+    "ctof_kernel_admm_kernel": (ctypes.c_char_p, [_P]),
     "ctof_status_string": (ctypes.c_char_p, [ctypes.c_int]),
     "ctof_last_error_message": (ctypes.c_char_p, []),
 }
@@ -401,6 +402,10 @@ class Kernel:
         out = ctypes.c_int()
         _check(self._lib.ctof_kernel_get_planes(self._h, ctypes.byref(out)), "ctof_kernel_get_planes")
         return out.value
+
+    def admm_kernel(self):
+        """Name of the kernel that the ADMM x-update of this handle runs."""
+        return self._lib.ctof_kernel_admm_kernel(self._h).decode()
 
     # ---- parity accessors (synchronous) ----
     def get_w(self):

@@ -39,3 +39,12 @@ def test_large_blocks_on_the_bins(mua, nz, nt, d, dt):
         assert rel_l2(got, so.fista_l1(wh, m, g, 6)[0]) <= 1e-5
     finally:
         k.close()
+
+
+@pytest.mark.parametrize("nz,nt,name", [(6, 32, "k_contract_warp"), (64, 100, "k_contract_admm_pipe")])
+def test_name_of_the_x_update(nz, nt, name):
+    k = ctof.Kernel(ctof.make_optics(), ctof.make_grid(8, nz, nt, 1.0, 1.0, 1.0, 50.0))
+    try:
+        assert k.planes() == nt and k.admm_kernel() == name
+    finally:
+        k.close()
