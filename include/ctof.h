@@ -348,9 +348,9 @@ ctof_status ctof_learned_reconstruct_checked(ctof_learned net, ctof_kernel k, in
 ctof_status ctof_reconstruct_batch(int count, const ctof_kernel* ks, const float* const* d_m,
                                    const ctof_solver_params* params, float* const* d_mu, void* stream);
 
-/* Autotuner: times the column-FFT tile (32 or 16 columns of 8 or 16 planes) for each of the four column-pass shapes of an
- * ADMM iteration on this handle and keeps the fastest; the results are
- * bit-identical for every tile, only the speed changes.  Runs automatically
+/* Autotuner: times the column-FFT tile (32 or 16 columns of 8 or 16 planes)
+ * for each of the four column-pass shapes of an ADMM iteration on this handle
+ * and keeps the fastest; the results are bit-identical for every tile, only the speed changes.  Runs automatically
  * before the first ADMM graph capture of a handle.  Synchronous; not inside a
  * stream capture. */
 ctof_status ctof_kernel_autotune(ctof_kernel k, void* stream);

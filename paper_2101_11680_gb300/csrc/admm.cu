@@ -225,19 +225,14 @@ __global__ void k_block_hadamard(float* __restrict__ v, int planes, int n) {
   base[((lane + 32) >> 3) * n + (lane & 7)] = d;
 }
 
-int grid_elem(size_t count) {
-  size_t b = (count + 255) / 256;
-  if (b > 152 * 8) b = 152 * 8;
-  return b < 1 ? 1 : (int)b;
-}
-
 }  // namespace
 
 ctof_status admm_tv_stencil(const ctof_kernel_s* k, const float* x, const float* u2_old, float* u2_new, float* u3,
                             float* s, const double* beta_dev, float rho, float* out_crop, cudaStream_t st) {
   dim3 block(TX, TY);
   dim3 grid(k->p / TX, k->p / TY, ctof_div_up(k->nz, ZP));
-  CTOF_CUDA_TRY(ctof_launch(k_tv_stencil, grid, block, 0, st, x, u2_old, u2_new, u3, s, beta_dev, 1.0f / rho, k->p, k->nz, k->n, out_crop));
+  CTOF_CUDA_TRY(ctof_launch(k_tv_stencil, grid, block, 0, st, x, u2_old, u2_new, u3, s, beta_dev, 1.0f / rho, k->p,
+                            k->nz, k->n, out_crop));
   CTOF_CUDA_TRY(cudaGetLastError());
   return CTOF_OK;
 }

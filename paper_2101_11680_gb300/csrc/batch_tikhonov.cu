@@ -676,7 +676,6 @@ constexpr int WS_EPI0 = 10;     // epilogue warps 10 .. 13
 constexpr int WS_EPI = 4;
 constexpr int WS_THREADS = (WS_EPI0 + WS_EPI) * 32;
 constexpr int WS_MBOX = 16 * 16 * 8;  // m_hat box: 16 volumes x 16 t x 8 bytes
-constexpr int WS_WBOX = 32 * 32 * 4;  // W_hat box: 32 t x 32 z x 4 bytes
 
 struct WsPlan {
   int nt, nz, z4, zn, fp8, nterm, nacc, esize, epc;

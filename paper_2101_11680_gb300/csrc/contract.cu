@@ -414,8 +414,8 @@ ctof_status launch(const ctof_kernel_s* k, int nvol, const float2* vin, int ld_i
   if (per_sm > 4) per_sm = 4;
   int grid = 152 * per_sm;
   if (grid > k->nclass) grid = k->nclass;
-  CTOF_CUDA_TRY(ctof_launch(k_contract<MODE>, grid, CT_THREADS, p.total, st, k->d_what, k->d_members, k->nclass, k->nt, k->nz, vin, ld_in,
-                                                      in_vstride, vout, ld_out, out_vstride, nvol, hinv, nbuf, nvs));
+  CTOF_CUDA_TRY(ctof_launch(k_contract<MODE>, grid, CT_THREADS, p.total, st, k->d_what, k->d_members, k->nclass,
+                            k->nt, k->nz, vin, ld_in, in_vstride, vout, ld_out, out_vstride, nvol, hinv, nbuf, nvs));
   CTOF_CUDA_TRY(cudaGetLastError());
   return CTOF_OK;
 }

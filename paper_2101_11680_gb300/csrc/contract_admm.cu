@@ -52,6 +52,7 @@
 #include <cuda_runtime.h>
 
 #include "ctof_internal.h"
+#include "tf32_mma.cuh"
 
 namespace {
 
@@ -102,14 +103,6 @@ __device__ __forceinline__ void split_tf32(float x, unsigned& hi, unsigned& lo) 
   asm("cvt.rna.tf32.f32 %0, %1;\n" : "=r"(hi) : "f"(x));
   const float r = x - __uint_as_float(hi);
   asm("cvt.rna.tf32.f32 %0, %1;\n" : "=r"(lo) : "f"(r));
-}
-
-__device__ __forceinline__ void mma_tf32(float (&d)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-      "{%0,%1,%2,%3};\n"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
 // d += A B in 3xTF32 (A_lo B_hi + A_hi B_lo + A_hi B_hi, small terms first), A
@@ -461,32 +454,6 @@ __device__ __forceinline__ int cons_sync_or(int v) {
       : "r"(v)
       : "memory");
   return out;
-}
-
-// W_hat -> [class][tm/8][zm/8][64] and H^-1 -> [class][zm/8][zm/8][64] in the
-// permuted 8 x 8 block layout described at the top of this file (zero padding).
-__global__ void k_admm_reorder(const float* __restrict__ src, int rows, int cols, int ld, int rm, int cm,
-                               float* __restrict__ dst, int nclass) {
-  const size_t per = (size_t)rm * cm, total = per * nclass;
-  const int cb_n = cm >> 3;
-  for (size_t d = (size_t)blockIdx.x * blockDim.x + threadIdx.x; d < total; d += (size_t)gridDim.x * blockDim.x) {
-    const size_t c = d / per;
-    const int rem = (int)(d - c * per), blk = rem >> 6, w = rem & 63;
-    const int rb = blk / cb_n, cb = blk - rb * cb_n;
-    const int half = w >> 5, q = w & 31;
-    const int i = ((q >> 2) - 4 * half) & 7, j = 4 * half + (q & 3);
-    const int r = 8 * rb + i, col = 8 * cb + j;
-    dst[d] = (r < rows && col < cols) ? src[c * (size_t)rows * ld + (size_t)r * ld + col] : 0.f;
-  }
-}
-
-// TF32 split for the pipelined kernel: hi = x rounded to the TF32 grid (to
-// nearest, ties away from zero: the same value as cvt.rna), lo = x - hi
-// exactly, passed to the MMA as raw FP32 bits, of which the tensor core reads
-// the TF32 part (|lo| <= 2^-11 |x|, so what is dropped is below 2^-21 |x|).
-__device__ __forceinline__ void split_fast(float x, unsigned& hi, unsigned& lo) {
-  hi = (__float_as_uint(x) + 0x1000u) & 0xffffe000u;
-  lo = __float_as_uint(x - __uint_as_float(hi));
 }
 
 __device__ __forceinline__ void mma_split_a(float (&d)[4], const float (&a)[4], unsigned bh0, unsigned bh1,
@@ -844,9 +811,9 @@ size_t contract_admm_pipe_floats(int nt, int nz, int which) {
 ctof_status contract_admm_prepare(ctof_kernel_s* k, cudaStream_t st) {
   if (!k->d_what_admm || !k->d_hinv_admm) return CTOF_OK;
   const int tm = rup(k->nt, 16), zm = rup(k->nz, 16);
-  k_admm_reorder<<<152 * 8, 256, 0, st>>>(k->d_what, k->nt, k->nz, k->z4, tm, zm, k->d_what_admm, k->nclass);
+  k_block_rows<<<152 * 8, 256, 0, st>>>(k->d_what, k->nt, k->nz, k->z4, tm / 8, zm / 8, k->d_what_admm, k->nclass);
   CTOF_CUDA_TRY(cudaGetLastError());
-  k_admm_reorder<<<152 * 8, 256, 0, st>>>(k->d_hinv, k->nz, k->nz, k->z4, zm, zm, k->d_hinv_admm, k->nclass);
+  k_block_rows<<<152 * 8, 256, 0, st>>>(k->d_hinv, k->nz, k->nz, k->z4, zm / 8, zm / 8, k->d_hinv_admm, k->nclass);
   CTOF_CUDA_TRY(cudaGetLastError());
   return CTOF_OK;
 }

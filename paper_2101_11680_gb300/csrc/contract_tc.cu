@@ -103,13 +103,6 @@ __device__ __forceinline__ int pick(const int (&mem)[4], int m) {
   return m == 0 ? mem[0] : (m == 1 ? mem[1] : (m == 2 ? mem[2] : mem[3]));
 }
 
-__device__ __forceinline__ void st_split1(unsigned char* hi, unsigned char* lo, uint32_t off, float v) {
-  float h, l;
-  umma::split_tf32(v, h, l);
-  *reinterpret_cast<float*>(hi + off) = h;
-  *reinterpret_cast<float*>(lo + off) = l;
-}
-
 // Setup shared by both kernels: zero shared memory (padding rows and columns
 // of the operand tiles stay zero), allocate TMEM, initialise the mbarrier.
 __device__ __forceinline__ uint32_t tc_setup(unsigned char* sm, const TcPlan& P) {
@@ -559,7 +552,7 @@ __device__ __forceinline__ bool aw_wait_warp(uint64_t* bar, uint32_t parity, lon
   return ok != 0;
 }
 
-// Split one staged chunk (converter thread ct of 256): A rows n (K = t) and
+// Split one staged chunk (converter thread ct of 512): A rows n (K = t) and
 // B = W^T rows z (K = t), TF32 high part and FP32 remainder each.
 __device__ __forceinline__ void aw_convert(const AwPlan& P, const unsigned char* raw, unsigned char* set,
                                            const int (&mem)[4], int ct, int bz, int bg) {

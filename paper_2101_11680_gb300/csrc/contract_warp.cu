@@ -7,17 +7,18 @@
 // for the complex vectors of the up-to-four frequencies that share the real
 // block W [nt][nz] of their class (8 real right-hand sides).
 //
-// A time-compressed block is 12 KB (64 planes x 48 depths): too little work
+// A time-compressed block is 15 KB (80 planes x 48 depths): too little work
 // for a thread block, whose barriers between the phases cost more than the
 // phases.  Launch times with a thread block / a warp per class: forward at
 // 256 x 256 x 32 x 128 (48 planes) 162 / 47 us (42 us of HBM time for what it
-// reads and writes), adjoint at 128 x 128 x 48 x 256 76 / 37 us (20), x-update
-// there 97 / 66 us (37; 73 us before the depth blocks became a template parameter).  Here a CTA (one per SM) holds a ring of shared-memory slots filled by bulk asynchronous
-// copies, one class per slot, and each of its warps takes every NW-th class
-// through all phases by itself: no block barrier, the warps drift apart and
-// their phases overlap.  The warp that finishes a class refills its slot with
-// the class that follows a ring's length later, so up to NS classes (200 KB)
-// are in flight per SM.
+// reads and writes), adjoint at 128 x 128 x 48 x 256 (80 planes) 76 / 37 us (20),
+// x-update there 97 / 70 us (42 us for 287 MB; 73 us before the depth blocks
+// became a template parameter).  Here a CTA (one per SM) holds a ring of
+// shared-memory slots filled by bulk asynchronous copies, one class per slot,
+// and each of its warps takes every NW-th class through all phases by itself:
+// no block barrier, the warps drift apart and their phases overlap.  The warp
+// that finishes a class refills its slot with the class that follows a ring's
+// length later, so up to NS classes (200 KB) are in flight per SM.
 //
 // Arithmetic is FP32 FMA (the x-update: TF32 tensor-core products in three terms,
 // as in contract_admm.cu).  Adjoint passes give a lane one 16-byte chunk of a
@@ -34,6 +35,7 @@
 
 #include "bulk.cuh"
 #include "ctof_internal.h"
+#include "tf32_mma.cuh"
 
 namespace {
 
@@ -330,21 +332,6 @@ __device__ __forceinline__ void do_class(const WarpArgs& A, unsigned char* st, u
   }
 }
 
-// TF32 split: hi = x rounded to the TF32 grid, lo = x - hi (its TF32 part is what
-// the tensor core reads: what is dropped is below 2^-21 |x|).
-__device__ __forceinline__ void split_fast(float x, unsigned& hi, unsigned& lo) {
-  hi = (__float_as_uint(x) + 0x1000u) & 0xffffe000u;
-  lo = __float_as_uint(x - __uint_as_float(hi));
-}
-
-__device__ __forceinline__ void mma_tf32(float (&d)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-      "{%0,%1,%2,%3};\n"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-
 // dh + dl += A B in 3xTF32 (the small products in their own accumulator).
 __device__ __forceinline__ void mma_3x(float (&dh)[4], float (&dl)[4], const float (&a)[4], const unsigned (&b)[4]) {
   unsigned ah[4], al[4];
@@ -534,7 +521,8 @@ __device__ __forceinline__ void do_admm(const WarpArgs& A, const unsigned char* 
         for (int u = 0; u < 2; ++u) {
           const int t = 8 * (r0 + 2 * v + u) + g;
           if (t < nt)
-            dst[t] = make_float2((eh[v][2 * u] + el[v][2 * u]) * A.inv_s, (eh[v][2 * u + 1] + el[v][2 * u + 1]) * A.inv_s);
+            dst[t] = make_float2((eh[v][2 * u] + el[v][2 * u]) * A.inv_s,
+                                 (eh[v][2 * u + 1] + el[v][2 * u + 1]) * A.inv_s);
         }
     }
   }
@@ -562,8 +550,8 @@ __device__ __forceinline__ bool wait_fill(uint64_t* full, const int* issued, int
 
 // ZB: 8-row z blocks of the ADMM products (ceil(nz / 8)).
 template <int MODE, int ZB>
-__global__ void __launch_bounds__(MODE == WM_ADMM ? MAX_PAIRS * 64 : MAX_WARPS * 32, 1) k_contract_warp(const __grid_constant__ WarpArgs A,
-                                                                     int* __restrict__ flag, long long max_polls) {
+__global__ void __launch_bounds__(MODE == WM_ADMM ? MAX_PAIRS * 64 : MAX_WARPS * 32, 1)
+    k_contract_warp(const __grid_constant__ WarpArgs A, int* __restrict__ flag, long long max_polls) {
   extern __shared__ __align__(128) unsigned char wsm[];
   pdl_trigger();
   const WarpPlan& P = A.P;
@@ -645,21 +633,6 @@ __global__ void k_pitch_rows(const float* __restrict__ in, long long rows, int n
   }
 }
 
-// Copies of src [nclass][rows][ld] (cols columns) in 8 x 8 blocks [rb][cb][64] of the
-// permuted word order above (zero padding).
-__global__ void k_block_rows(const float* __restrict__ src, int rows, int cols, int ld, int rb, int cb,
-                             float* __restrict__ dst, int nclass) {
-  const size_t per = (size_t)rb * cb * 64, total = per * nclass;
-  for (size_t d = (size_t)blockIdx.x * blockDim.x + threadIdx.x; d < total; d += (size_t)gridDim.x * blockDim.x) {
-    const size_t c = d / per;
-    const int rem = (int)(d - c * per), blk = rem >> 6, w = rem & 63;
-    const int br = blk / cb, bc = blk - br * cb;
-    const int half = w >> 5, q = w & 31;
-    const int r = 8 * br + (((q >> 2) - 4 * half) & 7), col = 8 * bc + 4 * half + (q & 3);
-    dst[d] = (r < rows && col < cols) ? src[c * (size_t)rows * ld + (size_t)r * ld + col] : 0.f;
-  }
-}
-
 template <int MODE, int ZB>
 ctof_status launch(const ctof_kernel_s* k, const WarpPlan& P, WarpArgs& A, cudaStream_t st) {
   A.P = P;
@@ -674,7 +647,8 @@ ctof_status launch(const ctof_kernel_s* k, const WarpPlan& P, WarpArgs& A, cudaS
   int nsm = 152;
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, k->device);
   const int grid = k->nclass < nsm ? k->nclass : nsm;
-  CTOF_CUDA_TRY(ctof_launch(kern, grid, P.nw * (MODE == WM_ADMM ? 64 : 32), P.total, st, A, k->d_flags, k->max_polls));
+  const int threads = P.nw * (MODE == WM_ADMM ? 64 : 32);
+  CTOF_CUDA_TRY(ctof_launch(kern, grid, threads, P.total, st, A, k->d_flags, k->max_polls));
   CTOF_CUDA_TRY(cudaGetLastError());
   return CTOF_OK;
 }

@@ -573,7 +573,8 @@ ctof_status batch_run(int count, const ctof_kernel* ks, const float* const* d_m,
     if (s == CTOF_OK && cudaMemcpyAsync(d_mu[i], o->d_vstage, vb, cudaMemcpyDeviceToDevice, side) != cudaSuccess)
       s = CTOF_ECUDA;
     // `st` waits for what was enqueued, also after an error
-    if (cudaEventRecord(o->batch_event, side) != cudaSuccess || cudaStreamWaitEvent(st, o->batch_event, 0) != cudaSuccess)
+    if (cudaEventRecord(o->batch_event, side) != cudaSuccess ||
+        cudaStreamWaitEvent(st, o->batch_event, 0) != cudaSuccess)
       s = CTOF_ECUDA;
   }
   return s;
@@ -986,8 +987,9 @@ ctof_status ctof_reconstruct_batch_tikhonov(ctof_kernel k, int batch, const floa
     }
     return CTOF_OK;
   }
-  // FP8 keeps the time bins: the projection's planes quantise differently, and with few depths that shows
-  // (64-bit error 1.3e-4 on the bins, 1.9e-4 on the planes at 74^2 x 3 x 368; BF16 and FP32 are as good or better on them).
+  // FP8 keeps the time bins.  Its terms share one scale per class (W_hat) and right-hand side (m_hat), which a
+  // plane that gathers a window of bins sets for all the others, and rounding errors average out over fewer
+  // planes: with few depths that shows (64-bit error 1.3e-4 on the bins, 1.9e-4 on the planes at 74^2 x 3 x 368).
   const bool tz = k->tz != nullptr && precision != CTOF_FP8E4M3;
   ctof_kernel_s* own = k;
   if (tz) k = k->tz;

@@ -407,7 +407,8 @@ static ctof_status make_basis(ctof_kernel_s* k, const double* what64, cudaStream
   };
   size_t off = 0;
   const size_t wp = contract_warp_floats(rows, nz, 0);
-  const size_t wa = wp ? 0 : contract_admm_pipe_floats(rows, nz, 0), ha = wp ? 0 : contract_admm_pipe_floats(rows, nz, 1);
+  const size_t wa = wp ? 0 : contract_admm_pipe_floats(rows, nz, 0);
+  const size_t ha = wp ? 0 : contract_admm_pipe_floats(rows, nz, 1);
   const size_t o_v = at(off, (size_t)k->nclass * rows * k->z4 * sizeof(float));
   const size_t o_wp = at(off, (size_t)k->nclass * wp * sizeof(float));
   const size_t o_wb = at(off, (size_t)k->nclass * contract_warp_floats(rows, nz, 1) * sizeof(float));
@@ -497,11 +498,11 @@ ctof_status time_compress(const ctof_kernel_s* z, int batch, const float* m, flo
     const float* src = m + (size_t)b0 * z->tz_nt * npix;
     float* dst = out + (size_t)b0 * z->nt * npix;
     if (bulk)
-      CTOF_CUDA_TRY(ctof_launch(kern, dim3(ctof_div_up(npix, tile), z->tz_nwin, nb), 256, smem, st,
-                                src, z->tz_nt, npix, z->d_tz_q, z->d_tz_win, z->tz_nwin, z->nt, dst, z->d_flags, z->max_polls));
+      CTOF_CUDA_TRY(ctof_launch(kern, dim3(ctof_div_up(npix, tile), z->tz_nwin, nb), 256, smem, st, src, z->tz_nt, npix,
+                                z->d_tz_q, z->d_tz_win, z->tz_nwin, z->nt, dst, z->d_flags, z->max_polls));
     else
-      CTOF_CUDA_TRY(ctof_launch(k_compress, dim3(ctof_div_up(npix, 32), z->tz_nwin, nb), 256, 0, st, src, z->tz_nt, npix, z->d_tz_q,
-                                                                             z->d_tz_win, z->tz_nwin, z->nt, dst));
+      CTOF_CUDA_TRY(ctof_launch(k_compress, dim3(ctof_div_up(npix, 32), z->tz_nwin, nb), 256, 0, st, src, z->tz_nt,
+                                npix, z->d_tz_q, z->d_tz_win, z->tz_nwin, z->nt, dst));
   }
   CTOF_CUDA_TRY(cudaGetLastError());
   return CTOF_OK;
@@ -510,9 +511,11 @@ ctof_status time_compress(const ctof_kernel_s* z, int batch, const float* m, flo
 ctof_status time_expand(const ctof_kernel_s* z, const float* y, float* m, cudaStream_t st) {
   const int npix = z->n * z->n;
   if (npix % 2 == 0 && (reinterpret_cast<uintptr_t>(m) & 7) == 0)
-    CTOF_CUDA_TRY(ctof_launch(k_expand<2>, dim3(ctof_div_up(npix, 512), z->tz_ntiles), 256, 0, st, y, npix, z->d_tz_q, z->d_tz_tiles, m));
+    CTOF_CUDA_TRY(ctof_launch(k_expand<2>, dim3(ctof_div_up(npix, 512), z->tz_ntiles), 256, 0, st, y, npix, z->d_tz_q,
+                              z->d_tz_tiles, m));
   else
-    CTOF_CUDA_TRY(ctof_launch(k_expand<1>, dim3(ctof_div_up(npix, 256), z->tz_ntiles), 256, 0, st, y, npix, z->d_tz_q, z->d_tz_tiles, m));
+    CTOF_CUDA_TRY(ctof_launch(k_expand<1>, dim3(ctof_div_up(npix, 256), z->tz_ntiles), 256, 0, st, y, npix, z->d_tz_q,
+                              z->d_tz_tiles, m));
   CTOF_CUDA_TRY(cudaGetLastError());
   return CTOF_OK;
 }

@@ -17,7 +17,7 @@ constexpr int TZ_R = 16;             // columns of one window's basis at most (r
 constexpr int TZ_FIRST = 16;         // bins of the first window
 constexpr double TZ_FALL = 1e-3;     // a window ends where the response has fallen by this factor
 constexpr double TZ_EPS = 1e-10;     // scaled residual at which a window's rank is reached
-constexpr double TZ_FLOOR = 1e-30;   // share of a bin's response below which a depth is not looked at (FP32 ends near it)
+constexpr double TZ_FLOOR = 1e-30;   // share of a bin's response below which a depth is not looked at
 constexpr double TZ_OWN = 2e-8;      // residual of a bin and depth relative to its own DC response
 constexpr double TZ_CHECK = 2e-8;    // residual over all classes, relative to a bin's DC response
 constexpr double TZ_CHECK_OWN = 1e-7;  // the same relative to that of the depth in the bin
@@ -178,7 +178,7 @@ inline int window_basis(const double* w, int nz, int ns, const double* d, int a,
   int r = 0;
   for (; r < len; ++r) {
     int piv = (int)(std::max_element(nn.begin(), nn.end()) - nn.begin());
-    double top = sqrt(nn[piv] / n);  // a lower bound of the largest entry; the entries themselves where it does not decide
+    double top = sqrt(nn[piv] / n);  // bounds the largest entry from below; the entries themselves where that is too low
     if (!(top >= TZ_EPS))
       for (double u : res) top = std::max(top, fabs(u));
     if (!(top >= TZ_EPS)) {  // in the window's scale; then every bin and depth in its own
