@@ -21,7 +21,7 @@ constexpr double TZ_FLOOR = 1e-30;   // share of a bin's response below which a 
 constexpr double TZ_OWN = 2e-8;      // residual of a bin and depth relative to its own DC response
 constexpr double TZ_CHECK = 2e-8;    // residual over all classes, relative to a bin's DC response
 constexpr double TZ_CHECK_OWN = 1e-7;  // the same relative to that of the depth in the bin
-constexpr double TZ_CANCEL = 10.0;   // largest sum_j |Q V| / |sum_j Q V| over the bins and depths of a window
+constexpr double TZ_CANCEL = 16.0;   // largest sum_j |Q V| / |sum_j Q V| over the bins and depths of a window
 
 // Pairs of doubles (the 128-bit vectors of either host) in four independent sums:
 // the fit is bound by these loops.
