@@ -208,7 +208,7 @@ ctof_status ctof_kernel_get_info(ctof_kernel k, ctof_kernel_info* info);
  * handle's kernel was compressed in time (its rows over the nt bins span that
  * many directions; the factorisation is checked at build time to 2e-8 of each
  * bin's response and 1e-7 of each depth's share of it, and its FP32 products
- * cancel by at most 16, so that results keep FP32 accuracy bin by bin and
+ * cancel by at most 20, so that results keep FP32 accuracy bin by bin and
  * depth by depth). */
 ctof_status ctof_kernel_get_planes(ctof_kernel k, int* planes);
 

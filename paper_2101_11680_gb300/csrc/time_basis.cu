@@ -18,13 +18,13 @@
 // own DC response.  In FP32 the products Q V must not cancel either: a deep
 // layer's response rises by up to eight decades from bin 16 to 32, and a basis in
 // the order of size makes its early bins the small difference of large products
-// (7e-3 of bin 16 for an absorber at 28-32 mm).  The basis of such a window is
-// turned into the order of its bins, and a window whose products still cancel by
-// more than 16 in any bin and depth is cut in two.  Emulated in FP32 every bin and
-// depth then stays within 1e-6 (most within 3e-7); a limit of 10 gives 5e-7 but up
-// to nine planes more (48 x 48 x 40 x 169: 67 for 60, 80 planes for 64).  Ranks at
-// 0.5 mm / 25 ps: 67 of 256 bins (128 x 128 scan, 48 depths: 80 planes), 84 of 512
-// (64 depths: 96 planes).
+// (2.4e-3 of bin 16 for an absorber at 28-32 mm, 1.3e-5 at 20-24 mm).  Where they
+// cancel by more than 20 in any bin and depth the basis is turned into the order of
+// its bins, and a window that still cancels by more is cut in two.  Emulated in FP32
+// every bin and depth then stays within 2e-6, most within 3e-7; a limit of 10 gives
+// 5e-7 but up to nine planes more (48 x 48 x 40 x 169: 67 for 60, 80 planes for 64).
+// Ranks at 0.5 mm / 25 ps: 67 of 256 bins (128 x 128 scan, 48 depths: 80 planes), 84
+// of 512 (64 depths: 96 planes).
 // The factorisation is checked on the device over every frequency class and
 // is dropped (the handle then works on the nt bins) if it does not hold.
 #include <cuda_runtime.h>

@@ -21,10 +21,10 @@ constexpr double TZ_FLOOR = 1e-30;   // share of a bin's response below which a 
 constexpr double TZ_OWN = 2e-8;      // residual of a bin and depth relative to its own DC response
 constexpr double TZ_CHECK = 2e-8;    // residual over all classes, relative to a bin's DC response
 constexpr double TZ_CHECK_OWN = 1e-7;  // the same relative to that of the depth in the bin
-constexpr double TZ_CANCEL = 16.0;   // largest sum_j |Q V| / |sum_j Q V| over the bins and depths of a window
+constexpr double TZ_CANCEL = 20.0;   // largest sum_j |Q V| / |sum_j Q V| over the bins and depths of a window
 
-// Pairs of doubles (the 128-bit vectors of either host) in four independent sums:
-// the fit is bound by these loops.
+// Pairs of doubles (the 128-bit vectors of either host), four sums: the fit is
+// bound by these loops.
 typedef double pair_t __attribute__((vector_size(16)));
 inline pair_t pair_at(const double* p) {
   pair_t v;
@@ -33,34 +33,33 @@ inline pair_t pair_at(const double* p) {
 }
 
 inline double dot(const double* a, const double* b, size_t n) {
-  pair_t s[4] = {};
+  pair_t s = {0.0, 0.0}, t = {0.0, 0.0};
   size_t i = 0;
-  for (; i + 8 <= n; i += 8)
-    for (int u = 0; u < 4; ++u) s[u] += pair_at(a + i + 2 * u) * pair_at(b + i + 2 * u);
-  const pair_t t = (s[0] + s[1]) + (s[2] + s[3]);
-  double r = t[0] + t[1];
-  for (; i < n; ++i) r += a[i] * b[i];
-  return r;
+  for (; i + 4 <= n; i += 4) {
+    s += pair_at(a + i) * pair_at(b + i);
+    t += pair_at(a + i + 2) * pair_at(b + i + 2);
+  }
+  for (; i < n; ++i) s[0] += a[i] * b[i];
+  return (s[0] + s[1]) + (t[0] + t[1]);
 }
 
-// y += f x; the squared norm of the new y.
+// y += f x; the squared norm of the new y (as dot forms it).
 inline double axpy(double f, const double* x, double* y, size_t n) {
-  pair_t s[4] = {};
   const pair_t ff = {f, f};
+  pair_t s = {0.0, 0.0}, t = {0.0, 0.0};
   size_t i = 0;
-  for (; i + 8 <= n; i += 8)
-    for (int u = 0; u < 4; ++u) {
-      const pair_t v = pair_at(y + i + 2 * u) + ff * pair_at(x + i + 2 * u);
-      memcpy(y + i + 2 * u, &v, sizeof(v));
-      s[u] += v * v;
-    }
-  const pair_t t = (s[0] + s[1]) + (s[2] + s[3]);
-  double r = t[0] + t[1];
+  for (; i + 4 <= n; i += 4) {
+    const pair_t u = pair_at(y + i) + ff * pair_at(x + i), v = pair_at(y + i + 2) + ff * pair_at(x + i + 2);
+    memcpy(y + i, &u, sizeof(u));
+    memcpy(y + i + 2, &v, sizeof(v));
+    s += u * u;
+    t += v * v;
+  }
   for (; i < n; ++i) {
     y[i] += f * x[i];
-    r += y[i] * y[i];
+    s[0] += y[i] * y[i];
   }
-  return r;
+  return (s[0] + s[1]) + (t[0] + t[1]);
 }
 
 // Largest cancellation in the products of an orthonormal basis g [r][len]: over
@@ -157,15 +156,12 @@ inline int window_basis(const double* w, int nz, int ns, const double* d, int a,
   if (idx.empty()) idx.push_back(0);
   const size_t n = idx.size();
   std::vector<int> zi(n);
-  std::vector<double> sc(n), nn(len);  // 1 / cz of the kept columns, squared norms of the residual rows
-  for (size_t i = 0; i < n; ++i) {
-    zi[i] = (int)(idx[i] % nz);
-    sc[i] = 1.0 / cz[zi[i]];
-  }
+  std::vector<double> den(nz), nn(len);  // a bin's scale per depth, squared norms of the residual rows
+  for (size_t i = 0; i < n; ++i) zi[i] = (int)(idx[i] % nz);
   std::vector<double> e(len * n), res;
   for (int t = 0; t < len; ++t) {
-    const double dt = 1.0 / d[a + t];
-    for (size_t i = 0; i < n; ++i) e[t * n + i] = w[(a + t) * cols + idx[i]] * dt * sc[i];
+    for (int z = 0; z < nz; ++z) den[z] = d[a + t] * cz[z];
+    for (size_t i = 0; i < n; ++i) e[t * n + i] = w[(a + t) * cols + idx[i]] / den[zi[i]];
     nn[t] = dot(&e[t * n], &e[t * n], n);
   }
   res = e;
@@ -223,14 +219,15 @@ inline int window_basis(const double* w, int nz, int ns, const double* d, int a,
   }
   double least = cancellation(w, nz, cols, d, a, len, g, r);
   std::vector<double> pick = g;
-  for (double theta : {0.7, 0.5, 0.25, 0.1}) {
-    std::vector<double> h = in_time_order(g, r, len, theta);
-    const double c = cancellation(w, nz, cols, d, a, len, h, r);
-    if (c < least) {
-      least = c;
-      pick.swap(h);
+  if (!(least <= TZ_CANCEL))
+    for (double theta : {0.7, 0.5, 0.25, 0.1}) {
+      std::vector<double> h = in_time_order(g, r, len, theta);
+      const double c = cancellation(w, nz, cols, d, a, len, h, r);
+      if (c < least) {
+        least = c;
+        pick.swap(h);
+      }
     }
-  }
   if (!(least <= TZ_CANCEL)) return -1;
   for (int j = 0; j < r; ++j)
     for (int t = 0; t < len; ++t) q[t * TZ_R + j] = pick[(size_t)j * len + t];

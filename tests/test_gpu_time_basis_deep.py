@@ -1,9 +1,9 @@
 """Time-compressed operator on absorbers below 20 mm, whose response rises by many decades over the early bins: every
 bin's plane against the FP64 oracle relative to itself (or to the bin that shares its complex transform: bins 2 i and
 2 i + 1 are the two parts of one, on the bins as on the planes), and every depth of the adjoint of early bins relative
-to itself.  The products of a window may cancel (csrc/time_fit.h), by 16 at most and by a few as a rule: ten times the
-rounding of Q, V and the transforms (6e-8, 6e-8 and 1e-7).  A 32 x 32 scan, from which single calls use the planes; the oracle takes the handle's own FP64 kernel table
-(which has its parity tests)."""
+to itself.  The products of a window may cancel (csrc/time_fit.h), by 20 at most and by a few as a rule: ten times the
+rounding of Q, V and the transforms (6e-8, 6e-8 and 1e-7).  A 32 x 32 scan, from which single calls use the planes;
+the oracle takes the handle's own FP64 kernel table (which has its parity tests)."""
 
 import numpy as np
 import pytest

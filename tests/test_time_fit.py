@@ -74,7 +74,7 @@ def test_seventeen_bins_of_rank_sixteen(fit, nt):
 @pytest.mark.parametrize("nz,nt,d,dt", [(48, 256, 0.5, 25.0), (64, 512, 0.5, 25.0), (40, 160, 1.0, 50.0)])
 def test_every_bin_and_depth_in_fp32(fit, nz, nt, d, dt):
     """The stored FP32 factors give every bin of every depth's DC response back, also where a deep layer's response
-    rises by many decades within a window.  The products may cancel, by 16 at most and by a few as a rule: ten times the
+    rises by many decades within a window.  The products may cancel, by 20 at most and by a few as a rule: ten times the
     rounding of Q, V and their sum (6e-8 each)."""
     g = op.Grid(8, nz, nt, d, d, d, dt)
     wh = op.kernel_spectrum(op.kernel_offsets(g, ph.Medium(0.01, 1.0, 1.4, r_min=0.5 * d)), g)
